@@ -61,8 +61,8 @@ def measured_peaks():
 # Source files that define each stage's kernel, its launch configuration and the data it
 # reads: a stored DRAM measurement holds only while these are unchanged.
 STAGE_SOURCES = {
-    "plane_fft": ["kernels.cuh", "fft.cuh", "plan.h", "path_impl.cuh"],
-    "column_fft_contract": ["kernels.cuh", "fft.cuh", "plan.h", "path_impl.cuh"],
+    "plane_fft": ["kernels.cuh", "fft.cuh", "fixed.cuh", "plan.h", "path_impl.cuh", "sized_impl.cuh"],
+    "column_fft_contract": ["kernels.cuh", "fft.cuh", "fixed.cuh", "plan.h", "path_impl.cuh", "sized_impl.cuh"],
     "w_gemm": ["kernels.cuh", "plan.h", "path_impl.cuh", "tcgen05.cuh", "gemm_tc.cuh", "gemm_tc.cu",
                "gemm_f64tc.cuh", "gemm_f64tc.cu"],
 }

@@ -16,8 +16,11 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libltmp2.so")
 
-SOURCES = ["ltmp2_api.cu", "host_plan.cu", "kernels_f64.cu", "kernels_f32.cu", "gemm_tc.cu", "gemm_f64tc.cu", "laplace.cpp",
-           "ltmp2_noalloc.cu", "mlp.cu", "probe.cu", "learned.cu"]
+# the longest compilations first: they start first
+SOURCES = ["persist_f64_planes.cu", "persist_f64_columns.cu", "sized_f64_a.cu", "sized_f64_b.cu", "sized_f64_c.cu",
+           "sized_f64_d.cu", "sized_f64_e.cu", "persist_f32_planes.cu", "persist_f32_columns.cu", "sized_f32_a.cu",
+           "sized_f32_b.cu", "kernels_f64.cu", "kernels_f32.cu", "ltmp2_api.cu", "host_plan.cu", "gemm_tc.cu",
+           "gemm_f64tc.cu", "laplace.cpp", "ltmp2_noalloc.cu", "mlp.cu", "probe.cu", "learned.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O3",
               "--expt-relaxed-constexpr"]

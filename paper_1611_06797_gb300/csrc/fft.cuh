@@ -97,6 +97,17 @@ static inline cudaError_t upload_twiddles() {
   return cudaMemcpyToSymbol(c_tw32, h_tw32, sizeof(h_tw32));
 }
 
+// the same, once per device in each translation unit (the callers serialise)
+static inline cudaError_t upload_twiddles_once() {
+  static bool done[64] = {false};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev < 64 && done[dev])) return e;
+  e = upload_twiddles();
+  if (e == cudaSuccess && dev < 64) done[dev] = true;
+  return e;
+}
+
 template <typename T> struct TwTable;
 template <> struct TwTable<double> {
   static __host__ __device__ __forceinline__ cpx<double> get(int i) {

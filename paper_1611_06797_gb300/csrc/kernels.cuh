@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "fft.cuh"
+#include "fixed.cuh"
 #include "plan.h"
 
 namespace ltmp2 {
@@ -34,6 +35,32 @@ __host__ __device__ __forceinline__ int plane_stride(int n, int nxa) {
   const int base = n * nxa;
   return base + ((nxa - base) % 16 + 16) % 16;
 }
+
+// Type of the co-densities between the plane and the column kernel: T itself in FP32; in FP64
+// 64-bit fixed point (fixed.cuh), times 2^(uen3[i] + wen3[col] - 61) for item (i, col).
+template <typename T> struct Codensity {
+  typedef T W;
+  static __device__ __forceinline__ cpx<T> real(cpx<T> a) { return a; }
+  static __device__ __forceinline__ T scale(const Plan &, int, size_t) { return T(1); }
+};
+constexpr int kFxBits = 61;          // |fixed-point value| <= 2^61, the bound given by the 2-norms
+constexpr int kFxNotFinite = 1 << 20;   // exponent of a state with a NaN or an infinity
+// e with 2^e > sqrt(norm2); squares below 1e-290 count as zero
+__device__ __forceinline__ int fx_exponent(double norm2) {
+  if (!(norm2 < 1e300)) return kFxNotFinite;
+  return norm2 < 1e-290 ? -480 : (ilogb(norm2) >> 1) + 1;
+}
+__device__ __forceinline__ double fx_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+template <> struct Codensity<double> {
+  typedef long long W;
+  static __device__ __forceinline__ cpx<double> real(cpx<long long> a) {
+    return {__ll2double_rn(a.x), __ll2double_rn(a.y)};
+  }
+  static __device__ __forceinline__ double scale(const Plan &p, int i, size_t col) {
+    const int e = p.uen3[i] + p.wen3[col];
+    return e < kFxNotFinite / 2 ? fx_pow2(e - kFxBits) : __longlong_as_double(0x7ff8000000000000ll);
+  }
+};
 
 // position in A of the G' carried by a slot of the current slab
 __device__ __forceinline__ int slot_aux(const Plan &p, int gp0, int np, int slot) {
@@ -617,10 +644,175 @@ __device__ __forceinline__ void planes3_body(const Plan &p, int ib, int z, int c
   }
 }
 
+// sum of v over the block's threads (blockDim.x a multiple of 32 or below 1024), in every thread
+__device__ __forceinline__ double block_sum(double v) {
+  __shared__ double red[32];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int w = threadIdx.x / 32, nw = (blockDim.x + 31) / 32;
+  __syncthreads();
+  if (threadIdx.x % 32 == 0) red[w] = v;
+  __syncthreads();
+  double s = 0.0;
+  for (int k = 0; k < nw; ++k) s += red[k];
+  return s;
+}
+
+// FP64 form of planes3_body on 64-bit fixed point (fixed.cuh).  The FP64 pipe bound the same
+// passes in double (85 % of its issue rate); a launch of 3488 columns of 32 occupied on 24^3 took
+// 62.3 ms in double and takes 11.5 ms on integers (with the column kernel, 14.1 -> 4.2 ms).
+//  w plane: scaled by 2^(61 - e), 2^e > ||w||_2 of the plane (n ||z1||_2 by Parseval), inverse
+//           transformed in fixed point; every partial sum of the transform is at most
+//           sum |z1| <= sqrt(n_dorb) ||z1||_2 < ||w||_2;
+//  x pass : phi_i comes as phi 2^(62 - uen), 2^uen > ||phi_i||_2 of the plane, so the product
+//           is conj(phi_i) w 2^(61 - uen - e), and every partial sum of its forward transform
+//           is at most ||phi_i||_2 ||w||_2 (Cauchy-Schwarz): below 2^61;
+//  y pass, copy: as in planes3_body; the copy shifts to the item's scale 2^(61 - uen3 - wen3), from
+//           the norms over all planes, so that the column kernel's sums over z stay below 2^61.
+template <int N>
+__device__ __forceinline__ void planes3_body_fx(const Plan &p, int ib, int z, int col,
+                                                const cpx<double> *__restrict__ z1, cpx<long long> *__restrict__ tbuf,
+                                                unsigned char *smem_raw) {
+  typedef long long W;
+  constexpr int P = N + 1;
+  cpx<W> *xp = reinterpret_cast<cpx<W> *>(smem_raw);
+  const int nxa = p.mxhi_aux - p.mxlo_aux + 1;
+  const int nd = p.n_daux;
+  const int Q = plane_stride(N, nxa);
+  cpx<W> *wk = xp + N * P;
+  int *ytab = reinterpret_cast<int *>(wk + (size_t)ib * Q);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int no = p.n_occ;
+  const int mlo = p.mxlo_aux, mhi = p.mxhi_aux;
+  const unsigned inv_nxa = ((1u << 20) + nxa - 1) / nxa;   // ceil(2^20 / nxa)
+  const cpx<double> *zrow = z1 + ((size_t)col * N + z) * p.n_dorb;
+  for (int d = tid; d < nd; d += nth) {
+    const int4 c = p.daux[d];
+    ytab[d] = wrapn(c.y, N) * nxa + (c.x - mlo);
+  }
+  for (int e = tid; e < N * P; e += nth) xp[e] = {0, 0};
+  double s2 = 0.0;
+  for (int d = tid; d < p.n_dorb; d += nth) {
+    const cpx<double> v = zrow[d];
+    s2 = fma(v.x, v.x, fma(v.y, v.y, s2));
+  }
+  int ew = fx_exponent(block_sum(s2) * (double)(N * N));   // the sum's barriers order xp's zeros
+  if (ew == kFxNotFinite) ew = 0;   // the column's wen3 says so
+  const double f = fx_pow2(kFxBits - ew);
+  for (int d = tid; d < p.n_dorb; d += nth) {
+    const int4 c = p.dorb[d];
+    const cpx<double> v = zrow[d];
+    xp[wrapn(c.y, N) * P + wrapn(c.x, N)] = {__double2ll_rn(v.x * f), __double2ll_rn(v.y * f)};
+  }
+  __syncthreads();
+  const int nxo = p.mxhi_orb - p.mxlo_orb + 1;
+  for (int t = tid; t < nxo; t += nth) {
+    const int x = wrapn(p.mxlo_orb + t, N);
+    cpx<W> a[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) a[k] = xp[k * P + x];
+    LineFFT<W, N, +1>::run(a);
+#pragma unroll
+    for (int k = 0; k < N; ++k) xp[k * P + x] = a[k];
+  }
+  __syncthreads();
+  for (int t = tid; t < N; t += nth) {
+    cpx<W> a[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) a[k] = xp[t * P + k];
+    LineFFT<W, N, +1>::run(a);
+#pragma unroll
+    for (int k = 0; k < N; ++k) xp[t * P + k] = a[k];
+  }
+  __syncthreads();
+  const cpx<W> *ut = (const cpx<W> *)p.ut;
+  const W *utr = (const W *)p.utr;
+  const int jcol = col % no;
+  const int ni = p.keep_count ? p.keep_count[jcol] : no;
+  const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
+  const int esh = p.wen3[col] - ew;   // >= 0 (a sentinel for a state that is not finite)
+  for (int i0 = 0; i0 < ni; i0 += ib) {
+    const int nb = min(ib, ni - i0);
+    for (int t = tid; t < nb * N; t += nth) {
+      const int il = t / N, y = t - il * N;
+      const int iocc = ilist ? ilist[i0 + il] : i0 + il;
+      cpx<W> a[N];
+      const size_t urow = ((size_t)iocc * N + z) * N * N + y;
+      const cpx<W> *wr = xp + y * P;
+      if (utr) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const W u = utr[urow + k * N];
+          a[k] = {fx_mul62(u, wr[k].x), fx_mul62(u, wr[k].y)};
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const cpx<W> u = ut[urow + k * N], w = wr[k];
+          a[k] = {fx_mul62(u.x, w.x) + fx_mul62(u.y, w.y), fx_mul62(u.x, w.y) - fx_mul62(u.y, w.x)};
+        }
+      }
+      LineFFT<W, N, -1>::run(a);
+      cpx<W> *row = wk + (size_t)il * Q + y * nxa - mlo;   // row[m] for m in [mlo, mhi]
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const int m = freq_of<N>(k);
+        if (m >= mlo && m <= mhi) row[m] = a[k];
+      }
+    }
+    __syncthreads();
+    for (int t = tid; t < nb * nxa; t += nth) {
+      const int il = (int)(((unsigned)t * inv_nxa) >> 20), xa = t - il * nxa;   // t / nxa, exact for t < 2^12
+      cpx<W> *src = wk + (size_t)il * Q + xa;
+      cpx<W> b[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) b[k] = src[k * nxa];
+      LineFFT<W, N, -1>::run(b);
+#pragma unroll
+      for (int k = 0; k < N; ++k) src[k * nxa] = b[k];
+    }
+    __syncthreads();
+    for (int il = 0; il < nb; ++il) {
+      const int iocc = ilist ? ilist[i0 + il] : i0 + il;
+      const size_t item = (size_t)col * no + iocc;
+      cpx<W> *dst = tbuf + (item * N + z) * nd;
+      const cpx<W> *src = wk + (size_t)il * Q;
+      const int sh = min(62, esh + p.uen3[iocc] - p.uen[iocc * N + z]);
+      for (int d = tid; d < nd; d += nth) {
+        const cpx<W> v = src[ytab[d]];
+        dst[d] = {fx_shr(v.x, sh), fx_shr(v.y, sh)};
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Exponent of ||w||_2 over the grid for every column of a slab, from its plane-wave
+// coefficients (||w||^2 = n^3 sum |c|^2); one block per column.  The factor keeps it at or above
+// the exponents that the plane kernel finds per plane.
+static __global__ void k_wnorm(Plan p, const cpx<double> *__restrict__ w) {
+  const cpx<double> *row = w + (size_t)blockIdx.x * p.n_pw;
+  double s2 = 0.0;
+  for (int q = threadIdx.x; q < p.n_pw; q += blockDim.x) {
+    const cpx<double> v = row[q];
+    s2 = fma(v.x, v.x, fma(v.y, v.y, s2));
+  }
+  s2 = block_sum(s2);
+  if (threadIdx.x == 0) p.wen3[blockIdx.x] = fx_exponent(s2 * ((double)p.n * p.n * p.n * (1.0 + 1e-9)));
+}
+
 template <typename T, int N>
-__global__ void k_planes3(Plan p, int ib, const cpx<T> *__restrict__ z1, cpx<T> *__restrict__ tbuf) {
+__device__ __forceinline__ void planes3_any(const Plan &p, int ib, int z, int col, const void *z1, void *tbuf,
+                                            unsigned char *smem_raw) {
+  if constexpr (std::is_same<T, double>::value)
+    planes3_body_fx<N>(p, ib, z, col, (const cpx<double> *)z1, (cpx<long long> *)tbuf, smem_raw);
+  else
+    planes3_body<T, N>(p, ib, z, col, (const cpx<T> *)z1, (cpx<T> *)tbuf, smem_raw);
+}
+
+template <typename T, int N>
+__global__ void k_planes3(Plan p, int ib, const void *__restrict__ z1, void *__restrict__ tbuf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  planes3_body<T, N>(p, ib, blockIdx.x, blockIdx.y, z1, tbuf, smem_raw);
+  planes3_any<T, N>(p, ib, blockIdx.x, blockIdx.y, z1, tbuf, smem_raw);
 }
 
 // Same result as k_planes3 with no block barrier after the w plane is transformed: each of
@@ -702,21 +894,55 @@ __global__ void __launch_bounds__(32 * kPlaneWarps) k_planes4(Plan p, int ib, co
 }
 
 // setup: real-space occupied orbitals u[j][z][y][x] from z1 (cols = occupied orbitals)
-// (and the plane-transposed copy outt[j][z][x][y] that the plane kernel reads row-wise)
+// (and the plane-transposed copy outt[j][z][x][y] that the plane kernel reads row-wise).
+// FP64: the transposed copy (outr's real part where it is given, else outt) is fixed point,
+// phi 2^(62 - uen[j][z]), and un2[j][z] keeps the plane's square norm.
 template <typename T, int N>
 __global__ void k_planes_store(Plan p, const cpx<T> *__restrict__ z1, cpx<T> *__restrict__ out,
-                               cpx<T> *__restrict__ outt, T *__restrict__ outr) {
+                               void *__restrict__ outt, void *__restrict__ outr) {
   constexpr int P = N + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T> *xp = reinterpret_cast<cpx<T> *>(smem_raw);
   const int z = blockIdx.x, col = blockIdx.y;
   plane_inverse<T, N>(p, z1 + ((size_t)col * N + z) * p.n_dorb, xp);
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    const int y = e / N, x = e % N;
-    out[((size_t)col * N + z) * N * N + e] = xp[y * P + x];
-    const cpx<T> v = xp[x * P + y];   // e = x' N + y' with x' = y, y' = x
-    outt[((size_t)col * N + z) * N * N + e] = v;
-    if (outr) outr[((size_t)col * N + z) * N * N + e] = v.x;
+  const size_t base = ((size_t)col * N + z) * N * N;
+  if constexpr (std::is_same<T, double>::value) {
+    double s2 = 0.0;
+    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
+      const cpx<double> v = xp[(e / N) * P + e % N];
+      s2 = fma(v.x, v.x, fma(v.y, v.y, s2));
+    }
+    s2 = block_sum(s2);
+    int eu = fx_exponent(s2);
+    if (threadIdx.x == 0) {
+      p.uen[col * N + z] = eu;
+      p.un2[col * N + z] = s2;
+    }
+    if (eu == kFxNotFinite) eu = 0;
+    const double f = fx_pow2(kFxBits + 1 - eu);
+    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
+      const int y = e / N, x = e % N;
+      if (out) out[base + e] = xp[y * P + x];
+      const cpx<double> v = xp[x * P + y];   // e = x' N + y' with x' = y, y' = x
+      if (outr) ((long long *)outr)[base + e] = __double2ll_rn(v.x * f);
+      else ((cpx<long long> *)outt)[base + e] = {__double2ll_rn(v.x * f), __double2ll_rn(v.y * f)};
+    }
+  } else {
+    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
+      const int y = e / N, x = e % N;
+      out[base + e] = xp[y * P + x];
+      const cpx<T> v = xp[x * P + y];
+      ((cpx<T> *)outt)[base + e] = v;
+      if (outr) ((T *)outr)[base + e] = v.x;
+    }
+  }
+}
+// exponents of the occupied orbitals' norms over the grid, at or above those of their planes
+static __global__ void k_unorm3(Plan p) {
+  for (int i = threadIdx.x; i < p.n_occ; i += blockDim.x) {
+    double s2 = 0.0;
+    for (int z = 0; z < p.n; ++z) s2 += p.un2[i * p.n + z];
+    p.uen3[i] = fx_exponent(s2 * (1.0 + 1e-9));
   }
 }
 
@@ -728,7 +954,8 @@ __global__ void k_planes_store(Plan p, const cpx<T> *__restrict__ z1, cpx<T> *__
 // M values are unnormalised (N^3 times the co-density).  Diagonal items also store
 // M_ii(G;G') in mdiag[slot][G][i] for the direct term.
 template <typename T>
-__device__ __forceinline__ void block_reduce_store(double ax, double ay, double2 *dst, double2 *dst_t) {
+__device__ __forceinline__ void block_reduce_store(double ax, double ay, double2 *dst, double2 *dst_t, double scale_a,
+                                                   double scale_b) {
   __shared__ double red[2][32];
   for (int o = 16; o > 0; o >>= 1) {
     ax += __shfl_xor_sync(0xffffffffu, ax, o);
@@ -740,6 +967,8 @@ __device__ __forceinline__ void block_reduce_store(double ax, double ay, double2
   if (threadIdx.x == 0) {
     double sx = 0, sy = 0;
     for (int k = 0; k < nw; ++k) { sx += red[0][k]; sy += red[1][k]; }
+    sx = sx * scale_a * scale_b;
+    sy = sy * scale_a * scale_b;
     *dst = make_double2(sx, sy);
     if (dst_t) *dst_t = make_double2(sx, -sy);
   }
@@ -751,7 +980,8 @@ __device__ __forceinline__ void block_reduce_store(double ax, double ay, double2
 // running sum is the sum over A_n, stored for n = 1 in dst1 and for n >= 2 in lev.
 template <typename T>
 __device__ __forceinline__ void level_reduce_store(const Plan &p, const cpx<T> *PR, size_t elem, size_t elem_t,
-                                                   bool transpose, double2 *dst1, double2 *lev) {
+                                                   bool transpose, double2 *dst1, double2 *lev, double scale_a,
+                                                   double scale_b) {
   __shared__ double lred[kMaxLevels][2];
   const int tid = threadIdx.x, nth = blockDim.x;
   const int w = tid / 32, l = tid % 32, nw = nth / 32;   // blockDim.x is a multiple of 32
@@ -776,16 +1006,19 @@ __device__ __forceinline__ void level_reduce_store(const Plan &p, const cpx<T> *
       rx += lred[n][0];
       ry += lred[n][1];
       double2 *base = n == 0 ? dst1 : lev + (size_t)n * p.lev_stride;
-      base[elem] = make_double2(rx, ry);
-      if (transpose) base[elem_t] = make_double2(rx, -ry);
+      const double sx = rx * scale_a * scale_b, sy = ry * scale_a * scale_b;
+      base[elem] = make_double2(sx, sy);
+      if (transpose) base[elem_t] = make_double2(sx, -sy);
     }
   }
 }
 
 template <typename T, int N, bool LEV>
-__device__ __forceinline__ void zcol_body(const Plan &p, int gp0, int np, int pair, const cpx<T> *__restrict__ tbuf,
+__device__ __forceinline__ void zcol_body(const Plan &p, int gp0, int np, int pair, const void *__restrict__ tbuf_v,
                                           cpx<T> *__restrict__ mdiag, double2 *__restrict__ sx,
                                           unsigned char *smem_raw) {
+  typedef typename Codensity<T>::W W;
+  const cpx<W> *__restrict__ tbuf = (const cpx<W> *)tbuf_v;
   cpx<T> *MA = reinterpret_cast<cpx<T> *>(smem_raw);
   cpx<T> *PR = MA + p.n_aux;   // LEV only: v(G) times the product, per G
   const int no = p.n_occ;
@@ -822,24 +1055,27 @@ __device__ __forceinline__ void zcol_body(const Plan &p, int gp0, int np, int pa
   const size_t itemB = ((size_t)slotB * no + i) * no + j;   // (j, i, slotB)
   const T *v = vtab<T>(p);
   const int nd = p.n_daux;
+  // the sums run on unscaled fixed-point values (FP64); the two items' scales multiply the result
+  const T scA = Codensity<T>::scale(p, i, (size_t)slotA * no + j), scB = Codensity<T>::scale(p, j, (size_t)slotB * no + i);
   T accx = T(0), accy = T(0);
   for (int d = tid; d < nd; d += nth) {
     const int4 c = p.daux[d];
     const int off = p.daux_off[d];
-    const cpx<T> *src = tbuf + itemA * N * nd + d;
-    cpx<T> a[N];
+    const cpx<W> *src = tbuf + itemA * N * nd + d;
+    cpx<W> a[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) a[k] = src[(size_t)k * nd];
-    LineFFT<T, N, -1>::run(a);
+    LineFFT<W, N, -1>::run(a);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const int m = freq_of<N>(k);
       if (m >= c.z && m <= c.w) {
         const int g = off + m - c.z;
-        MA[g] = a[k];
-        if (diag) mdiag[((size_t)slotA * p.n_aux + g) * no + i] = a[k];
+        const cpx<T> x = Codensity<T>::real(a[k]);
+        MA[g] = x;
+        if (diag) mdiag[((size_t)slotA * p.n_aux + g) * no + i] = cscale(x, scA);
         if (self) {
-          const T t = v[g] * (a[k].x * a[k].x + a[k].y * a[k].y);
+          const T t = v[g] * (x.x * x.x + x.y * x.y);
           if (LEV) PR[g] = {t, T(0)};
           else accx += t;
         }
@@ -851,28 +1087,31 @@ __device__ __forceinline__ void zcol_body(const Plan &p, int gp0, int np, int pa
     for (int d = tid; d < nd; d += nth) {
       const int4 c = p.daux[d];
       const int off = p.daux_off[d];
-      const cpx<T> *src = tbuf + itemB * N * nd + d;
-      cpx<T> a[N];
+      const cpx<W> *src = tbuf + itemB * N * nd + d;
+      cpx<W> a[N];
 #pragma unroll
       for (int k = 0; k < N; ++k) a[k] = src[(size_t)k * nd];
-      LineFFT<T, N, -1>::run(a);
+      LineFFT<W, N, -1>::run(a);
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         const int m = freq_of<N>(k);
         if (m >= c.z && m <= c.w) {
           const int g = off + m - c.z;
+          const cpx<T> x = Codensity<T>::real(a[k]);
           cpx<T> prod;
           if (!p.real_orb) {
-            prod = cmul(MA[p.aux_neg[g]], a[k]);
-            if (diag) mdiag[((size_t)slotB * p.n_aux + g) * no + i] = a[k];
+            prod = cmul(MA[p.aux_neg[g]], x);
+            if (diag) mdiag[((size_t)slotB * p.n_aux + g) * no + i] = cscale(x, scB);
           } else {
-            prod = cmulconj(MA[g], a[k]);
+            // the imaginary part cancels between (i, j) and (j, i) = its conjugate
+            const cpx<T> y = MA[g];
+            prod = {y.x * x.x + y.y * x.y, T(0)};
           }
           if (LEV) {
             PR[g] = {v[g] * prod.x, v[g] * prod.y};
           } else {
             accx += v[g] * prod.x;
-            accy += v[g] * prod.y;
+            if (!p.real_orb) accy += v[g] * prod.y;
           }
         }
       }
@@ -882,14 +1121,15 @@ __device__ __forceinline__ void zcol_body(const Plan &p, int gp0, int np, int pa
   const bool transpose = p.real_orb && i != j;
   if constexpr (LEV) {
     __syncthreads();
-    level_reduce_store<T>(p, PR, elem, elem_t, transpose, sx, p.sxl);
+    level_reduce_store<T>(p, PR, elem, elem_t, transpose, sx, p.sxl, (double)scA, self ? (double)scA : (double)scB);
   } else {
-    block_reduce_store<T>((double)accx, (double)accy, sx + elem, transpose ? sx + elem_t : nullptr);
+    block_reduce_store<T>((double)accx, (double)accy, sx + elem, transpose ? sx + elem_t : nullptr, (double)scA,
+                          self ? (double)scA : (double)scB);
   }
 }
 
 template <typename T, int N, bool LEV>
-__global__ void __launch_bounds__(256) k_zcol(Plan p, int gp0, int np, const cpx<T> *__restrict__ tbuf,
+__global__ void __launch_bounds__(256) k_zcol(Plan p, int gp0, int np, const void *__restrict__ tbuf,
                                               cpx<T> *__restrict__ mdiag, double2 *__restrict__ sx) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   zcol_body<T, N, LEV>(p, gp0, np, blockIdx.x, tbuf, mdiag, sx, smem_raw);
@@ -1134,8 +1374,10 @@ __global__ void k_gather_k(Plan p, int gp0, int np, cpx<T> *__restrict__ st) {
 // Diagonal blocks also store M_II at its canonical index g + [kappa_I < kappa_slot], where
 // every item of a slot has Q = g_c - kappa_slot / n (the direct term pairs g_c with -g_c + e).
 template <typename T, int N>
-__global__ void __launch_bounds__(256) k_zcol_k(Plan p, int gp0, int np, const cpx<T> *__restrict__ tbuf,
+__global__ void __launch_bounds__(256) k_zcol_k(Plan p, int gp0, int np, const void *__restrict__ tbuf_v,
                                                 cpx<T> *__restrict__ mdiag, double2 *__restrict__ sx) {
+  typedef typename Codensity<T>::W W;
+  const cpx<W> *__restrict__ tbuf = (const cpx<W> *)tbuf_v;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T> *MA = reinterpret_cast<cpx<T> *>(smem_raw);
   const int NO = p.n_occ, no = p.no_k, nslots = 2 * np;
@@ -1162,26 +1404,28 @@ __global__ void __launch_bounds__(256) k_zcol_k(Plan p, int gp0, int np, const c
   const size_t colA = ((size_t)kp_index(p, ktA[0], ktA[1], ktA[2]) * nslots + gpl) * no + j;
   const size_t colB = ((size_t)kp_index(p, ktB[0], ktB[1], ktB[2]) * nslots + gpl + np) * no + i;
   const size_t itemA = colA * NO + I, itemB = colB * NO + J;
+  const T scA = Codensity<T>::scale(p, I, colA), scB = Codensity<T>::scale(p, J, colB);
   const bool diag = (I == J);
   const T *vA = vtab_k<T>(p) + (size_t)kp_class(p, dA) * p.n_aux;
   const int nd = p.n_daux;
   for (int d = tid; d < nd; d += nth) {
     const int4 c = p.daux[d];
     const int off = p.daux_off[d];
-    const cpx<T> *src = tbuf + itemA * N * nd + d;
-    cpx<T> a[N];
+    const cpx<W> *src = tbuf + itemA * N * nd + d;
+    cpx<W> a[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) a[k] = src[(size_t)k * nd];
-    LineFFT<T, N, -1>::run(a);
+    LineFFT<W, N, -1>::run(a);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const int m = freq_of<N>(k);
       if (m >= c.z && m <= c.w) {
         const int g = off + m - c.z;
-        MA[g] = a[k];
+        const cpx<T> x = Codensity<T>::real(a[k]);
+        MA[g] = x;
         if (diag) {
           const int q = kp_lut(p, c.x + cA[0], c.y + cA[1], m + cA[2]);
-          if (q >= 0) mdiag[((size_t)gpl * p.n_aux + q) * NO + I] = a[k];
+          if (q >= 0) mdiag[((size_t)gpl * p.n_aux + q) * NO + I] = cscale(x, scA);
         }
       }
     }
@@ -1191,30 +1435,32 @@ __global__ void __launch_bounds__(256) k_zcol_k(Plan p, int gp0, int np, const c
   for (int d = tid; d < nd; d += nth) {
     const int4 c = p.daux[d];
     const int off = p.daux_off[d];
-    const cpx<T> *src = tbuf + itemB * N * nd + d;
-    cpx<T> a[N];
+    const cpx<W> *src = tbuf + itemB * N * nd + d;
+    cpx<W> a[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) a[k] = src[(size_t)k * nd];
-    LineFFT<T, N, -1>::run(a);
+    LineFFT<W, N, -1>::run(a);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const int m = freq_of<N>(k);
       if (m >= c.z && m <= c.w) {
+        const cpx<T> x = Codensity<T>::real(a[k]);
         if (diag) {
           const int q = kp_lut(p, c.x + cB[0], c.y + cB[1], m + cB[2]);
-          if (q >= 0) mdiag[((size_t)(gpl + np) * p.n_aux + q) * NO + I] = a[k];
+          if (q >= 0) mdiag[((size_t)(gpl + np) * p.n_aux + q) * NO + I] = cscale(x, scB);
         }
         const int qa = kp_lut(p, -c.x + del[0], -c.y + del[1], -m + del[2]);
         if (qa >= 0) {
           const T v = vA[qa];
-          const cpx<T> prod = cmul(MA[qa], a[k]);
+          const cpx<T> prod = cmul(MA[qa], x);
           accx += v * prod.x;
           accy += v * prod.y;
         }
       }
     }
   }
-  block_reduce_store<T>((double)accx, (double)accy, sx + ((size_t)gpl * NO + I) * NO + J, nullptr);
+  block_reduce_store<T>((double)accx, (double)accy, sx + ((size_t)gpl * NO + I) * NO + J, nullptr, (double)scA,
+                        (double)scB);
 }
 
 // Direct term per (primary slot, I): Y_IJ = sum_{g_c} v(g_c - kappa'/n) M_II(g_c; Q') M_JJ(-g_c + e; -Q'),

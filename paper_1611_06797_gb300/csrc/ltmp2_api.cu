@@ -226,6 +226,16 @@ int upload_real_coeff_t(ltmp2_ctx *c, const ltmp2_system *sys, const std::vector
   return cuda_status(cudaMemcpy(*dst, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
 }
 
+// FP64: exponent tables of the fixed-point co-densities (the columns' one comes with the slab)
+template <typename T> int dalloc_exponents(ltmp2_ctx *c) {
+  if (!std::is_same<T, double>::value) return LTMP2_OK;
+  Plan &p = c->p;
+  const size_t planes = (size_t)p.n_occ * p.n;
+  int rc;
+  if ((rc = dalloc(c, &p.uen, planes)) || (rc = dalloc(c, &p.un2, planes))) return rc;
+  return dalloc(c, &p.uen3, (size_t)p.n_occ);
+}
+
 template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys, const std::vector<int> &order) {
   Plan &p = c->p;
   cudaError_t e = Path<T>::init_device();
@@ -245,7 +255,9 @@ template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys,
   if ((rc = upload_coeff<T>(c, sys->coeff, p.n_pw, 0, p.n_occ, order, &cocc))) return rc;
   if ((rc = dalloc_bytes(c, &p.cgrid, cs * n3 * p.n_occ))) return rc;
   if ((rc = dalloc_bytes(c, &p.u, cs * n3 * p.n_occ))) return rc;
-  if ((rc = dalloc_bytes(c, &p.ut, cs * n3 * p.n_occ))) return rc;
+  // FP64: the plane kernel reads the real part alone where the orbitals are real
+  if (!(p.real_basis && std::is_same<T, double>::value) && (rc = dalloc_bytes(c, &p.ut, cs * n3 * p.n_occ))) return rc;
+  if ((rc = dalloc_exponents<T>(c))) return rc;
   if (p.real_basis && (rc = dalloc_bytes(c, &p.utr, sizeof(T) * n3 * p.n_occ))) return rc;
   if ((rc = dalloc_bytes(c, &p.dscale, sizeof(T) * p.n_orb))) return rc;
   // real basis: one extra row, for the pair-interleaved Green's function of the tensor-core build
@@ -268,6 +280,7 @@ template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys,
   p.max_prim = (int)mp;
   c->slab_capacity = p.max_prim;
   const size_t max_cols = cols_pp * p.max_prim;
+  if (std::is_same<T, double>::value && (rc = dalloc(c, &p.wen3, max_cols))) return rc;
   if ((rc = dalloc_bytes(c, &p.st, cs * max_cols * p.n_pw))) return rc;
   if ((rc = dalloc_bytes(c, &p.wt, cs * max_cols * p.n_pw))) return rc;
   if ((rc = dalloc_bytes(c, &p.z1, cs * std::max(max_cols, (size_t)p.n_occ) * p.n * p.n_dorb))) return rc;
@@ -337,6 +350,7 @@ int setup_precision_k(ltmp2_ctx *c, const ltmp2_kpoint_system *sys, const std::v
   if ((rc = dalloc_bytes(c, &p.cgrid, cs * n3 * p.n_occ))) return rc;
   if ((rc = dalloc_bytes(c, &p.u, cs * n3 * p.n_occ))) return rc;
   if ((rc = dalloc_bytes(c, &p.ut, cs * n3 * p.n_occ))) return rc;
+  if ((rc = dalloc_exponents<T>(c))) return rc;
   if ((rc = dalloc_bytes(c, &p.dscale, sizeof(T) * (size_t)nk * norb))) return rc;
   if ((rc = dalloc_bytes(c, &p.pt, cs * (size_t)nk * npw * npw))) return rc;
   size_t free_b = 0, total_b = 0;
@@ -352,6 +366,7 @@ int setup_precision_k(ltmp2_ctx *c, const ltmp2_kpoint_system *sys, const std::v
   p.max_prim = (int)mp;
   c->slab_capacity = p.max_prim;
   const size_t max_cols = cols_pp * p.max_prim;
+  if (std::is_same<T, double>::value && (rc = dalloc(c, &p.wen3, max_cols))) return rc;
   if ((rc = dalloc_bytes(c, &p.st, cs * max_cols * npw))) return rc;
   if ((rc = dalloc_bytes(c, &p.wt, cs * max_cols * npw))) return rc;
   if ((rc = dalloc_bytes(c, &p.z1, cs * std::max(max_cols, (size_t)p.n_occ) * p.n * p.n_dorb))) return rc;
@@ -581,7 +596,8 @@ template <typename T> int tune_ctx(ltmp2_ctx *c, int *slab_out, int *var_out) {
     const int ncols = best_slab * p.slots_per_prim() * p.n_occ;
     double best_plane = 1e300;
     static const int kIbs[2][4] = {{2, 4, 8, 16}, {1, 2, 3, 4}};   // planes per block; kernel 3: per warp step
-    for (int pk = 0; pk < 4 && !rc; ++pk)
+    // FP64 has one plane kernel
+    for (int pk = std::is_same<T, double>::value ? 2 : 0; pk < (std::is_same<T, double>::value ? 3 : 4) && !rc; ++pk)
       for (int ibk = 0; ibk < 4; ++ibk) {
         const int ib = kIbs[pk == 3 ? 1 : 0][ibk];
         if (ib > p.n_occ) continue;

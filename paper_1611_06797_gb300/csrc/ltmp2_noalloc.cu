@@ -124,8 +124,15 @@ int run_noalloc(const ltmp2_system *sys, Plan &p, Arena &ar, const std::vector<i
   void *cocc = ar.take(ho.size() * cs);
   p.cv = p.real_basis ? ar.take(hr.size() * sizeof(T)) : ar.take(hv.size() * cs);
   p.cgrid = ar.take(cs * n3 * p.n_occ);
-  p.u = ar.take(cs * n3 * p.n_occ);
+  // the orbitals themselves are read by FP32's other plane kernels only
+  if (std::is_same<T, float>::value && !(p.u = ar.take(cs * n3 * p.n_occ))) return LTMP2_ERR_UNSUPPORTED;
   p.ut = ar.take(cs * n3 * p.n_occ);
+  if (std::is_same<T, double>::value) {   // exponents of the fixed-point co-densities
+    p.uen = (int *)ar.take(sizeof(int) * p.n_occ * p.n);
+    p.un2 = (double *)ar.take(sizeof(double) * p.n_occ * p.n);
+    p.uen3 = (int *)ar.take(sizeof(int) * p.n_occ);
+    if (!p.uen || !p.un2 || !p.uen3) return LTMP2_ERR_UNSUPPORTED;
+  }
   p.dscale = ar.take(sizeof(T) * p.n_orb);
   p.pt = ar.take((p.real_basis ? sizeof(T) : cs) * (size_t)p.n_pw * p.n_pw);
   const size_t no2 = (size_t)p.n_occ * p.n_occ;
@@ -134,14 +141,15 @@ int run_noalloc(const ltmp2_system *sys, Plan &p, Arena &ar, const std::vector<i
   p.exi = (double *)ar.take(no2 * sizeof(double));
   p.edi = (double *)ar.take(no2 * sizeof(double));
   p.esum = (double *)ar.take(4 * sizeof(double));
-  if (!cocc || !p.cv || !p.cgrid || !p.u || !p.ut || !p.dscale || !p.pt || !p.ex || !p.ed || !p.exi || !p.edi || !p.esum)
+  if (!cocc || !p.cv || !p.cgrid || !p.ut || !p.dscale || !p.pt || !p.ex || !p.ed || !p.exi || !p.edi || !p.esum)
     return LTMP2_ERR_UNSUPPORTED;
   // slab of primary G' sized to what is left of the array
   const int spp = p.slots_per_prim();
   const size_t cols_pp = (size_t)spp * p.n_occ;
   const size_t per_prim = cs * cols_pp * (2 * (size_t)p.n_pw + (size_t)p.n * p.n_dorb +
                                           (size_t)p.n_occ * p.n * p.n_daux) +
-                          cs * spp * (size_t)p.n_aux * p.n_occ + 2 * sizeof(double2) * no2 + 8 * kAlign;
+                          cs * spp * (size_t)p.n_aux * p.n_occ + 2 * sizeof(double2) * no2 +
+                          sizeof(int) * cols_pp + 9 * kAlign;
   const size_t z1_min = cs * (size_t)p.n_occ * p.n * p.n_dorb + kAlign;
   if (ar.left() < z1_min + per_prim) return LTMP2_ERR_UNSUPPORTED;
   long long mp = (long long)((ar.left() - z1_min) / per_prim);
@@ -149,6 +157,7 @@ int run_noalloc(const ltmp2_system *sys, Plan &p, Arena &ar, const std::vector<i
   mp = std::min<long long>(mp, p.n_prim);
   p.max_prim = (int)std::max<long long>(1, mp);
   const size_t max_cols = cols_pp * p.max_prim;
+  if (std::is_same<T, double>::value && !(p.wen3 = (int *)ar.take(sizeof(int) * max_cols))) return LTMP2_ERR_UNSUPPORTED;
   p.st = ar.take(cs * max_cols * p.n_pw);
   p.wt = ar.take(cs * max_cols * p.n_pw);
   p.z1 = ar.take(cs * std::max(max_cols, (size_t)p.n_occ) * p.n * p.n_dorb);

@@ -5,15 +5,29 @@
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "sized.h"
 
 namespace ltmp2 {
 
-#define LTMP2_FOR_EACH_N(X) X(8) X(10) X(12) X(16) X(18) X(20) X(24) X(25) X(27) X(30) X(32) X(36) X(40)
+// f(integral_constant<int, n>) for the grid size n; false when no kernel is compiled for it
+template <typename F> static bool with_size(int n, F &&f) {
+  switch (n) {
+#define LTMP2_CASE(NN)                      \
+  case NN:                                  \
+    f(std::integral_constant<int, NN>{});   \
+    return true;
+    LTMP2_FOR_EACH_N(LTMP2_CASE)
+#undef LTMP2_CASE
+    default:
+      return false;
+  }
+}
 
 // Plane kernels: 0 = k_planes (full-plane passes), 1 = k_planes2 (compacted passes),
 // 2 = k_planes3 (product in registers, compact intermediate), 3 = k_planes4 (as 2, each
 // warp on its own occupied planes without block barriers).
 // ib = occupied planes per block (kernel 3: per warp step); 0 picks the default of each kernel.
+// FP64 has one plane kernel, 2 in fixed point: the others are accepted and run it.
 template <typename T> static int plane_ib_default(const Plan &p, int kernel) {
   const int n = p.n;
   const size_t plane = (size_t)n * (n + 1) * sizeof(cpx<T>);
@@ -59,28 +73,18 @@ template <typename T> static size_t plane_smem(const Plan &p, int kernel, int ib
 
 // launch the plane kernel for the ncols columns of the current slab (z1 -> tbuf)
 template <typename T> static cudaError_t launch_planes(const Plan &p, int ncols, int kernel, int ib, cudaStream_t st) {
+  if (std::is_same<T, double>::value) {
+    kernel = 2;
+    if (ib > 256 / p.n) ib = 256 / p.n;   // registers: at most 256 threads of up to 255
+    while (ib > 1 && plane_smem<T>(p, kernel, ib) > 200 * 1024) --ib;
+  }
   if (ib <= 0) ib = plane_ib_default<T>(p, kernel);
   const size_t smem = plane_smem<T>(p, kernel, ib);
   int threads = kernel == 3 ? 32 * kPlaneWarps : ib * p.n;
   if (threads < 64) threads = 64;
   if (threads > 1024 || smem > 200 * 1024) return cudaErrorInvalidValue;
-  switch (p.n) {
-#define LTMP2_CASE(NN)                                                                                     \
-  case NN:                                                                                                 \
-    if (kernel == 0)                                                                                       \
-      k_planes<T, NN><<<dim3(NN, ncols), threads, smem, st>>>(p, ib, (const cpx<T> *)p.z1, (cpx<T> *)p.tbuf);  \
-    else if (kernel == 1)                                                                                  \
-      k_planes2<T, NN><<<dim3(NN, ncols), threads, smem, st>>>(p, ib, (const cpx<T> *)p.z1, (cpx<T> *)p.tbuf); \
-    else if (kernel == 2)                                                                                  \
-      k_planes3<T, NN><<<dim3(NN, ncols), threads, smem, st>>>(p, ib, (const cpx<T> *)p.z1, (cpx<T> *)p.tbuf); \
-    else                                                                                                   \
-      k_planes4<T, NN><<<dim3(NN, ncols), threads, smem, st>>>(p, ib, (const cpx<T> *)p.z1, (cpx<T> *)p.tbuf); \
-    break;
-    LTMP2_FOR_EACH_N(LTMP2_CASE)
-#undef LTMP2_CASE
-    default:
-      return cudaErrorInvalidValue;
-  }
+  if (!with_size(p.n, [&](auto n) { Sized<T, decltype(n)::value>::planes(p, ncols, kernel, ib, threads, smem, st); }))
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
@@ -112,26 +116,10 @@ template <typename T> cudaError_t Path<T>::init_device() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 64 && done[dev]) return cudaSuccess;
-  e = upload_twiddles();
+  // twiddle tables and dynamic shared memory limits of the FFT kernels
+  for (int n : kFftSizes)
+    if (e == cudaSuccess) with_size(n, [&](auto c) { e = Sized<T, decltype(c)::value>::init(); });
   if (e != cudaSuccess) return e;
-  // dynamic shared memory limits of the FFT kernels
-#define LTMP2_SET_SMEM(NN)                                                                          \
-  e = cudaFuncSetAttribute(k_planes<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  if (e != cudaSuccess) return e;                                                                   \
-  e = cudaFuncSetAttribute(k_zcol<T, NN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  if (e != cudaSuccess) return e;                                                                   \
-  e = cudaFuncSetAttribute(k_zcol<T, NN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  if (e != cudaSuccess) return e;                                                                   \
-  e = cudaFuncSetAttribute(k_planes2<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  if (e != cudaSuccess) return e;                                                                   \
-  e = cudaFuncSetAttribute(k_planes3<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  if (e != cudaSuccess) return e;                                                                   \
-  e = cudaFuncSetAttribute(k_planes4<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  if (e != cudaSuccess) return e;                                                                   \
-  e = cudaFuncSetAttribute(k_zcol_k<T, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  if (e != cudaSuccess) return e;
-  LTMP2_FOR_EACH_N(LTMP2_SET_SMEM)
-#undef LTMP2_SET_SMEM
   if (dev < 64) done[dev] = true;
   return cudaSuccess;
 }
@@ -146,21 +134,13 @@ cudaError_t Path<T>::setup_occupied(const Plan &p, const void *c_occ_dev, cudaSt
   k_scatter_grid<T><<<dim3((p.n_pw + 255) / 256, p.n_occ), 256, 0, st>>>(p, p.n_occ, c, (cpx<T> *)p.cgrid);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // z1 scratch: reuse p.z1 when it is large enough (max_cols >= n_occ always holds)
-  cpx<T> *z1 = (cpx<T> *)p.z1;
-  const size_t smem = (size_t)n * (n + 1) * sizeof(cpx<T>);
-  switch (n) {
-#define LTMP2_CASE(NN)                                                                            \
-  case NN:                                                                                        \
-    k_w_zinv<T, NN><<<dim3((p.n_dorb + 127) / 128, p.n_occ), 128, 0, st>>>(p, p.n_pw, c, z1);     \
-    k_planes_store<T, NN><<<dim3(NN, p.n_occ), 128, smem, st>>>(p, z1, (cpx<T> *)p.u, (cpx<T> *)p.ut,       \
-                                                                (T *)p.utr);                                  \
-    break;
-    LTMP2_FOR_EACH_N(LTMP2_CASE)
-#undef LTMP2_CASE
-    default:
-      return cudaErrorInvalidValue;
-  }
+  // p.z1 is the scratch (max_cols >= n_occ always holds)
+  if (!with_size(n, [&](auto c) {
+        Sized<T, decltype(c)::value>::zinv(p, p.n_occ, c_occ_dev, p.z1, st);
+        Sized<T, decltype(c)::value>::planes_store(p, p.z1, st);
+      }))
+    return cudaErrorInvalidValue;
+  if constexpr (std::is_same<T, double>::value) k_unorm3<<<1, 256, 0, st>>>(p);
   return cudaGetLastError();
 }
 
@@ -319,17 +299,16 @@ cudaError_t Path<T>::slab_pre(const Plan &p, int gp0, int np, cudaStream_t st, S
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     w_pw = (const cpx<T> *)p.st;
   }
-  switch (n) {
-#define LTMP2_CASE(NN)                                                                                  \
-  case NN: {                                                                                            \
-    ScopedStage s(tm, kStageGatherZ);                                                                   \
-    k_w_zinv<T, NN><<<dim3((p.n_dorb + 127) / 128, ncols), 128, 0, st>>>(p, p.n_pw, w_pw, (cpx<T> *)p.z1); \
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;                                              \
-  } break;
-    LTMP2_FOR_EACH_N(LTMP2_CASE)
-#undef LTMP2_CASE
-    default:
+  if constexpr (std::is_same<T, double>::value) {
+    ScopedStage s(tm, kStageGatherZ);
+    k_wnorm<<<ncols, 128, 0, st>>>(p, (const cpx<T> *)w_pw);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  {
+    ScopedStage s(tm, kStageGatherZ);
+    if (!with_size(n, [&](auto c) { Sized<T, decltype(c)::value>::zinv(p, ncols, w_pw, p.z1, st); }))
       return cudaErrorInvalidValue;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -346,28 +325,17 @@ cudaError_t Path<T>::slab(const Plan &p, int gp0, int np, double coef, cudaStrea
   const int npairs = p.real_orb ? np * (no * (no + 1) / 2) : np * no * no;
   int col_threads = ((p.n_daux + 31) / 32) * 32;
   if (col_threads > 256) col_threads = 256;   // the column kernel's launch bound (FP64 N >= 36 uses ~255 registers)
-  switch (n) {
-#define LTMP2_CASE(NN)                                                                                  \
-  case NN: {                                                                                            \
-    {                                                                                                   \
-      ScopedStage s(tm, kStagePlane);                                                                   \
-      if ((e = launch_planes<T>(p, ncols, p.plane_kernel, p.plane_ib, st)) != cudaSuccess) return e;    \
-    }                                                                                                   \
-    {                                                                                                   \
-      ScopedStage s(tm, kStageColumn);                                                                  \
-      if (lev)                                                                                          \
-        k_zcol<T, NN, true><<<npairs, col_threads, smem_col, st>>>(p, gp0, np, (const cpx<T> *)p.tbuf,  \
-                                                                   (cpx<T> *)p.mdiag, p.sx);            \
-      else                                                                                              \
-        k_zcol<T, NN, false><<<npairs, col_threads, smem_col, st>>>(p, gp0, np, (const cpx<T> *)p.tbuf, \
-                                                                    (cpx<T> *)p.mdiag, p.sx);           \
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;                                            \
-    }                                                                                                   \
-  } break;
-    LTMP2_FOR_EACH_N(LTMP2_CASE)
-#undef LTMP2_CASE
-    default:
+  {
+    ScopedStage s(tm, kStagePlane);
+    if ((e = launch_planes<T>(p, ncols, p.plane_kernel, p.plane_ib, st)) != cudaSuccess) return e;
+  }
+  {
+    ScopedStage s(tm, kStageColumn);
+    if (!with_size(n, [&](auto c) {
+          Sized<T, decltype(c)::value>::zcol(p, gp0, np, npairs, col_threads, smem_col, lev, st);
+        }))
       return cudaErrorInvalidValue;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return slab_post(p, gp0, np, coef, st, tm);
 }
@@ -454,34 +422,29 @@ cudaError_t Path<T>::slab_k(const Plan &p, int gp0, int np, double coef, cudaStr
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
   }
+  if constexpr (std::is_same<T, double>::value) {
+    ScopedStage s(tm, kStageGatherZ);
+    k_wnorm<<<ncols, 128, 0, st>>>(p, (const cpx<T> *)p.wt);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   const size_t smem_col = (size_t)p.n_aux * sizeof(cpx<T>);
   const int npairs = np * NO * NO;
   int col_threads = ((p.n_daux + 31) / 32) * 32;
   if (col_threads > 256) col_threads = 256;
-  switch (n) {
-#define LTMP2_CASE(NN)                                                                                 \
-  case NN: {                                                                                           \
-    {                                                                                                  \
-      ScopedStage s(tm, kStageGatherZ);                                                                \
-      k_w_zinv<T, NN><<<dim3((p.n_dorb + 127) / 128, ncols), 128, 0, st>>>(p, p.n_pw, (const cpx<T> *)p.wt, \
-                                                                          (cpx<T> *)p.z1);              \
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;                                           \
-    }                                                                                                  \
-    {                                                                                                  \
-      ScopedStage s(tm, kStagePlane);                                                                  \
-      if ((e = launch_planes<T>(p, ncols, p.plane_kernel, p.plane_ib, st)) != cudaSuccess) return e;   \
-    }                                                                                                  \
-    {                                                                                                  \
-      ScopedStage s(tm, kStageColumn);                                                                 \
-      k_zcol_k<T, NN><<<npairs, col_threads, smem_col, st>>>(p, gp0, np, (const cpx<T> *)p.tbuf,       \
-                                                             (cpx<T> *)p.mdiag, p.sx);                 \
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;                                           \
-    }                                                                                                  \
-  } break;
-    LTMP2_FOR_EACH_N(LTMP2_CASE)
-#undef LTMP2_CASE
-    default:
+  {
+    ScopedStage s(tm, kStageGatherZ);
+    if (!with_size(n, [&](auto c) { Sized<T, decltype(c)::value>::zinv(p, ncols, p.wt, p.z1, st); }))
       return cudaErrorInvalidValue;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  {
+    ScopedStage s(tm, kStagePlane);
+    if ((e = launch_planes<T>(p, ncols, p.plane_kernel, p.plane_ib, st)) != cudaSuccess) return e;
+  }
+  {
+    ScopedStage s(tm, kStageColumn);
+    with_size(n, [&](auto c) { Sized<T, decltype(c)::value>::zcol_k(p, gp0, np, npairs, col_threads, smem_col, st); });
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   {
     ScopedStage s(tm, kStageDirect);
@@ -497,97 +460,22 @@ cudaError_t Path<T>::slab_k(const Plan &p, int gp0, int np, double coef, cudaStr
   return cudaSuccess;
 }
 
-// ---------------------------------------------------------------- batching form: persistent stages
-// Thread blocks of kPersistThreads stay resident and take items from a device counter:
-// plane items (system, column, z) and column items (system, pair) of every active system of
-// the round, each run by the same body as the system's own kernel (dispatch on its grid).
-template <typename T>
-__global__ void __launch_bounds__(kPersistThreads) k_planes_persist(const Plan *__restrict__ plans, BatchRound r,
-                                                                     int *__restrict__ counter) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_item;
-  // the round's tables in shared memory: indexed by the item's system, which a kernel
-  // parameter array would have to copy to local memory for
-  __shared__ BatchRound sr;
-  if (threadIdx.x == 0) sr = r;
-  const int total = r.first[r.nsys];
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-    __syncthreads();
-    const int item = s_item;
-    if (item >= total) return;
-    int e = 0;
-    while (item >= sr.first[e + 1]) ++e;
-    const Plan &p = plans[sr.sys[e]];
-    const int local = item - sr.first[e];
-    const int z = local % p.n, col = local / p.n;
-    switch (p.n) {
-#define LTMP2_CASE(NN)                                                                                        \
-  case NN:                                                                                                    \
-    planes3_body<T, NN>(p, sr.ib[e], z, col, (const cpx<T> *)p.z1, (cpx<T> *)p.tbuf, smem_raw);              \
-    break;
-      LTMP2_FOR_EACH_N(LTMP2_CASE)
-#undef LTMP2_CASE
-      default:
-        break;
-    }
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kPersistThreads) k_zcol_persist(const Plan *__restrict__ plans, BatchRound r,
-                                                                   int *__restrict__ counter) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_item;
-  // the round's tables in shared memory: indexed by the item's system, which a kernel
-  // parameter array would have to copy to local memory for
-  __shared__ BatchRound sr;
-  if (threadIdx.x == 0) sr = r;
-  const int total = r.first[r.nsys];
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-    __syncthreads();
-    const int item = s_item;
-    if (item >= total) return;
-    int e = 0;
-    while (item >= sr.first[e + 1]) ++e;
-    const Plan &p = plans[sr.sys[e]];
-    const int local = item - sr.first[e];
-    switch (p.n) {
-#define LTMP2_CASE(NN)                                                                                        \
-  case NN:                                                                                                    \
-    zcol_body<T, NN, false>(p, sr.gp0[e], sr.np[e], local, (const cpx<T> *)p.tbuf, (cpx<T> *)p.mdiag, p.sx,   \
-                            smem_raw);                                                                        \
-    break;
-      LTMP2_FOR_EACH_N(LTMP2_CASE)
-#undef LTMP2_CASE
-      default:
-        break;
-    }
-  }
-}
-
 template <typename T> size_t Path<T>::plane_smem_for(const Plan &p, int ib) { return plane_smem<T>(p, 2, ib); }
 
 template <typename T> cudaError_t Path<T>::persist_attributes(size_t plane_smem_b, size_t col_smem_b) {
-  cudaError_t e = cudaFuncSetAttribute(k_planes_persist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)plane_smem_b);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_zcol_persist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)col_smem_b);
+  cudaError_t e = PersistPlanes<T>::init();
+  if (e == cudaSuccess) e = PersistColumns<T>::init();
+  if (e == cudaSuccess) e = PersistPlanes<T>::attributes(plane_smem_b);
+  if (e == cudaSuccess) e = PersistColumns<T>::attributes(col_smem_b);
+  return e;
 }
 
 // resident blocks of the persistent kernel: every SM filled to its occupancy
 template <typename T> int Path<T>::persist_blocks(bool planes, size_t smem) {
-  int dev = 0, sms = 0, per = 0;
+  int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 0;
-  const cudaError_t e = planes
-      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_planes_persist<T>, kPersistThreads, smem)
-      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_zcol_persist<T>, kPersistThreads, smem);
-  if (e != cudaSuccess) return 0;
-  return sms * (per > 0 ? per : 1);
+  return sms * (planes ? PersistPlanes<T>::blocks_per_sm(smem) : PersistColumns<T>::blocks_per_sm(smem));
 }
 
 template <typename T>
@@ -595,7 +483,7 @@ cudaError_t Path<T>::planes_persist(const Plan *d_plans, const BatchRound &r, in
                                     cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_planes_persist<T><<<blocks, kPersistThreads, smem, st>>>(d_plans, r, counter);
+  PersistPlanes<T>::launch(d_plans, r, counter, blocks, smem, st);
   return cudaGetLastError();
 }
 
@@ -604,7 +492,7 @@ cudaError_t Path<T>::zcol_persist(const Plan *d_plans, const BatchRound &r, int 
                                   cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_zcol_persist<T><<<blocks, kPersistThreads, smem, st>>>(d_plans, r, counter);
+  PersistColumns<T>::launch(d_plans, r, counter, blocks, smem, st);
   return cudaGetLastError();
 }
 

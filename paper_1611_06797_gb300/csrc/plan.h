@@ -94,6 +94,13 @@ struct Plan {
   void *ut = nullptr;        // [n_occ][n^3] the same, each z plane transposed: [z][x][y]
   void *utr = nullptr;       // real orbitals at Gamma: the real part of ut, T [n_occ][z][x][y]
                              // (the orbitals are real in real space), else null
+  // FP64: exponents of the fixed-point co-densities (fixed.cuh): 2^uen bounds the 2-norm of
+  // plane z of orbital i, 2^uen3 that of the orbital, 2^wen3 that of a transformed state; ut (or utr
+  // where the orbitals are real) holds phi 2^(62 - uen) as integers
+  int *uen = nullptr;        // [n_occ][n]
+  int *uen3 = nullptr;       // [n_occ]
+  int *wen3 = nullptr;       // [max_cols]
+  double *un2 = nullptr;     // [n_occ][n] square norms of the planes (set-up)
   void *dscale = nullptr;    // [n_orb] T: virtual e^{-(e_a-mu)tau}, occupied e^{(e_j-mu)tau}
   void *pt = nullptr;        // [n_pw][n_pw] transposed Green's function P^T (real P if real_basis)
   void *st = nullptr;        // [max_cols][n_pw] gathered, scaled e^{-iG'r}|j> (S^T)
@@ -223,11 +230,11 @@ template <typename T> struct Path {
     return 2;
   }
   static int slab_launches(const Plan &p) {
-    if (p.route == 1) return 7 + (p.n_lev > 1 ? 1 : 0);   // no gather, CUDA-core product
+    if (p.route == 1) return 7 + (p.precision == 0 ? 1 : 0) + (p.n_lev > 1 ? 1 : 0);   // no gather, CUDA-core product
     // W: one product; FP64 on the tensor cores: split + product; through the virtual space:
     // two products (CUDA cores) or split, product, split, split, product (tensor cores)
     const int w = p.w_virtual ? (p.oz ? 5 : 2) : (p.oz ? 2 : 1);
-    return (p.tc ? 8 : 7) - 1 + w + (p.real_basis ? 1 : 0) + (p.n_lev > 1 ? 1 : 0) +
+    return (p.tc ? 8 : 7) - 1 + (p.precision == 0 ? 1 : 0) + w + (p.real_basis ? 1 : 0) + (p.n_lev > 1 ? 1 : 0) +
            (p.tc && p.tc->direct_on() && p.n_lev < 2 ? 2 : 0);   // direct term: pack, product, combine
   }
   // route 1 setup: the overlap densities of every primary G' into rt (uses st and pt as
@@ -267,7 +274,7 @@ template <typename T> struct Path {
   static cudaError_t green_k(const Plan &p, double tau, cudaStream_t st, StageTimer *tm);
   static cudaError_t slab_k(const Plan &p, int gp0, int np, double coef, cudaStream_t st, StageTimer *tm);
   static int green_k_launches(const Plan &p) { return 1 + p.nk; }
-  static int slab_k_launches(const Plan &p) { return 6 + p.nk; }
+  static int slab_k_launches(const Plan &p) { return 6 + p.nk + (p.precision == 0 ? 1 : 0); }
   // opposite-spin direct term of one slab (alpha plan pa, beta plan pb, same slab):
   // y [slab][na][nb] scratch, acc [na][nb] accumulated
   static cudaError_t direct_cross(const Plan &pa, const Plan &pb, int gp0, int np, double coef, double *y,

@@ -52,6 +52,25 @@ def test_bad_slab_and_quadrature_are_rejected():
     L.ltmp2_destroy(ctx)
 
 
+@pytest.mark.parametrize("real", [True, False], ids=["real", "general"])
+@pytest.mark.parametrize("scale", [1e-3, 1e2, 1e4])
+def test_fixed_point_scales_follow_the_states(real, scale):
+    """The co-densities' fixed-point scales come from the norms of the orbitals' and the states'
+    planes: one Laplace point at 1e-3, 1e2 and 1e4 times 1/gap takes the transformed states through
+    norms of order one, e^-100 and below the smallest double, where they count as zero."""
+    s = solid("tiny2")
+    tau, w = np.array([scale / (2.0 * s.gap)]), np.array([1.0])
+    ref = mp2_energy(OracleSystem.from_solid(s), laplace_denominator(tau, w))
+    ctx = L.setup_from_solid(s, precision=L.FP64, real=real)
+    ed, ex, ep = L.ltmp2_energy(ctx, tau, w)
+    L.ltmp2_destroy(ctx)
+    # sums of FP64 rounding errors relative to the sum of the magnitudes, which the direct term
+    # (all of one sign) is; nothing below 1e-290 survives on either side's scale
+    tol = 1e-12 * abs(ref["E_d"]) + 1e-280
+    assert abs(ed - ref["E_d"]) <= tol and abs(ex - ref["E_x"]) <= tol
+    assert np.abs(ep - ref["e_d"] - ref["e_x"]).max() <= tol
+
+
 def test_gprime_shares_add_up_to_the_energy():
     """Three ranks' shares of the outer G' loop (evaluated here one after another) add up
     to the full energy: the split a multi-GPU run of one system would use."""
