@@ -25,24 +25,24 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-int make_map(CUtensorMap *m, float *base, int rows, int kpad, int box_rows, int box_k = tc::BK,
-             CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B) {
+int make_map(CUtensorMap *m, void *base, int rows, int kpad, int box_rows, int box_k = tc::BK,
+             CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B, bool f16 = false) {
   cuuint64_t dims[2] = {(cuuint64_t)kpad, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)kpad * sizeof(float)};
+  cuuint64_t strides[1] = {(cuuint64_t)kpad * (f16 ? 2 : sizeof(float))};
   cuuint32_t box[2] = {(cuuint32_t)box_k, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1u, 1u};
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
   if (!fn) return -1;
-  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
+  const CUresult r = fn(m, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
                                             CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
                                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : -1;
 }
 }  // namespace
 
-// 64-byte-swizzled K-major fp32 operand map (the FP64 tensor-core GEMM's slices use it too)
-int tc_make_map_sw64(CUtensorMap *m, float *base, int rows, int kpad, int box_rows, int box_k) {
-  return make_map(m, base, rows, kpad, box_rows, box_k, CU_TENSOR_MAP_SWIZZLE_64B);
+// 64-byte-swizzled K-major fp16 operand map (the slices of the FP64 tensor-core GEMM)
+int tc_make_map_sw64_f16(CUtensorMap *m, void *base, int rows, int kpad, int box_rows, int box_k) {
+  return make_map(m, base, rows, kpad, box_rows, box_k, CU_TENSOR_MAP_SWIZZLE_64B, true);
 }
 
 // Layouts the autotuner chooses from: 4 drained (separate Re / Im operands, N 64, two-stage

@@ -168,8 +168,9 @@ struct Plan {
 struct OzResources {
   int rows_cap = 0, npw = 0, kpad = 0, arows = 0;  // complex rows, K = n_pw, padded K, stacked rows
   int nv = 0;                                      // virtuals (rows of the static slices bv)
-  float *a = nullptr, *b = nullptr;                // slices [8][arows][kpad], [8][npw][kpad]
-  float *bv = nullptr;                             // slices of R_v [8][nv][kpad], once per context
+  // FP16 slices (integers of at most 8 bits) [8][arows][kpad], [8][npw][kpad]
+  void *a = nullptr, *b = nullptr;
+  void *bv = nullptr;                              // slices of R_v [8][nv][kpad], once per context
   double *sa = nullptr, *sb = nullptr, *sbv = nullptr;  // row scales (powers of two)
   int *err = nullptr;                              // device flag: a bounded wait ran out
   void *maps = nullptr;                            // host copy of the three tensor maps
