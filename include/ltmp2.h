@@ -59,13 +59,12 @@ extern "C" {
 
 /* ---------------------------------------------------------------- precision */
 /* LTMP2_FP64: complex128 FFTs, FP64 GEMMs, FP64 accumulation (the plain path).   */
-/* LTMP2_FP32: complex64 FFTs; transformed-state GEMM on tcgen05 tensor cores in  */
-/*             3xTF32 split precision (hi*hi + hi*lo + lo*hi), each 16-wide k    */
-/*             block's tensor-memory partial added to FP32 register sums; with   */
-/*             real orbitals the Green's function P_r = R_v^T D R_v and the      */
-/*             direct-term products sum_G v M_ii conj(M_jj) per G' too (general  */
-/*             orbitals: CUDA cores, compensated FP32 sums); per-pair, per-tau   */
-/*             and final sums in FP64.                                           */
+/* LTMP2_FP32: complex64 FFTs; the Green's function and the transformed states on     */
+/*             tcgen05 tensor cores from 4 exact integer slices of 7 bits per        */
+/*             operand (28 bits below a row's maximum, exact sums); with real        */
+/*             orbitals the direct-term products sum_G v M_ii conj(M_jj) per G' in   */
+/*             3xTF32 split precision (hi*hi + hi*lo + lo*hi); per-pair, per-tau     */
+/*             and final sums in FP64.                                               */
 #define LTMP2_FP64 0
 #define LTMP2_FP32 1
 
@@ -75,9 +74,9 @@ extern "C" {
  * half of the G' set is transformed; the library checks the property in setup.  */
 #define LTMP2_FLAG_REAL_ORBITALS 1
 /* Run the dense products on the CUDA cores instead of the tcgen05 tensor cores: in
- * LTMP2_FP32 the transformed-state GEMM in FP32 with two-level summation instead of the
- * 3xTF32 kernel; in LTMP2_FP64 the Green's function and transformed-state GEMMs in FP64
- * instead of the exact-slice products (see ltmp2_dgemm_nt).  For comparisons.       */
+ * LTMP2_FP32 the Green's function and transformed-state GEMMs in FP32 with two-level
+ * summation, in LTMP2_FP64 the same in FP64, instead of the exact-slice products (see
+ * ltmp2_dgemm_nt).  For comparisons.                                                */
 #define LTMP2_FLAG_SIMT_GEMM 2
 
 typedef struct ltmp2_ctx ltmp2_ctx; /* opaque; owns all device memory of one system */
@@ -190,15 +189,15 @@ int ltmp2_set_slab_size(ltmp2_ctx *ctx, int n);
  * TIMEOUT.                                                                          */
 int ltmp2_autotune(ltmp2_ctx *ctx, int *slab, int *gemm_variant);
 
-/* Settings in effect for ctx: values[0] slab size, [1] tensor-core GEMM layout (-1 in
+/* Settings in effect for ctx: values[0] slab size, [1] tensor-core GEMM layout (5, or 4 for general orbitals; one kernel serves both; -1 in
  * FP64 or with LTMP2_FLAG_SIMT_GEMM), [2] plane FFT kernel (0 full-plane passes,
  * 1 compacted passes, 2 product in registers with a compact intermediate, 3 the same with
  * every warp on its own occupied planes and no block barriers; set-up chooses 3 in
  * LTMP2_FP32 and 2 in LTMP2_FP64), [3] occupied planes per plane-kernel block, for
  * kernel 3 per warp step (0 = default), [4] the precision form's
- * Green's function on the tensor cores (1; 3xTF32, set up at first use) or on the CUDA
- * cores with compensated sums (0, the default: the tensor-core build's plain FP32 sums
- * over K = n_v left 4x the error in E_d on the 36^3 workload), [5] its direct-term
+ * Green's function and transformed states in 3xTF32 (1; set up at first use) or from
+ * exact slices (0, the default: the 3xTF32 build's plain FP32 sums over K = n_v left
+ * 4x the error in E_d on the 36^3 workload), [5] its direct-term
  * contraction on the tensor cores (1, the default) or the CUDA cores (0); [4] and [5] are
  * -1 where there is no choice (FP64, general orbitals, LTMP2_FLAG_SIMT_GEMM).
  * The autotuner also chooses [2] and [3], timing the plane kernel alone.  values holds
@@ -365,15 +364,15 @@ int ltmp2_energy_uhf(ltmp2_ctx *alpha, ltmp2_ctx *beta, int n_tau, const double 
 int ltmp2_set_route(ltmp2_ctx *ctx, int route);
 
 /* ---------------------------------------------------------------- FP64 products on the tensor cores
- * The FP64 path's products in the real basis (the Green's function P_r, the transformed
- * states W^T = (U S)^T P_r of step (iii), Sec. III A, and at large tau the two products
- * through the kept virtuals) run on the tcgen05 tensor cores with FP64 accuracy, unless
- * LTMP2_FLAG_SIMT_GEMM is set: every row of both operands is scaled by a power of two and
- * cut into 8 slices of 7 bits (exact in TF32); the 36 slice products with s + t < 8 are
- * accumulated per order s + t in FP32 tensor memory, where sums of at most 400 k stay
- * below 2^24 and are therefore exact, and combined in FP64 registers.  A dropped term is
- * at most 7 x 2^-56 of the product of the two rows' largest magnitudes; the result
- * differs from an FP64 GEMM by about its own rounding.
+ * The products (the Green's function, the transformed states of step (iii), Sec. III A,
+ * and at large tau the two products through the kept virtuals) run on the tcgen05 tensor
+ * cores, unless LTMP2_FLAG_SIMT_GEMM is set: every row of both operands is scaled by a
+ * power of two and cut into 8 slices of 7 bits (FP32: 4), exact in FP16; the 36 (10) slice
+ * products with s + t < 8 (4) are accumulated per order s + t in FP32 tensor memory, where
+ * sums of at most 384 (640) k stay below 2^24 and are therefore exact, and combined in 64-bit
+ * integers.  A dropped term is at most 7 x 2^-56 of the product of the two rows' largest
+ * magnitudes; the result differs from an FP64 GEMM by about its own rounding.  A row that
+ * holds a NaN or an infinity gives NaN.
  * ltmp2_dgemm_nt: C = A B^T with that scheme.  A [m][lda], B [n][ldb], C [m][ldc]: DEVICE
  * pointers to row-major doubles (first k columns of A and B used), lda, ldb >= k,
  * ldc >= n.  Allocates and frees its own slice buffers (about 32 (m + n) k bytes) and

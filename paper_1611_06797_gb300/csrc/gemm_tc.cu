@@ -1,5 +1,5 @@
-// Host side of the tcgen05 3xTF32 transformed-state GEMM: operand buffers, TMA tensor
-// maps (built once per context) and the launchers used by the precision form.
+// Host side of the tcgen05 3xTF32 GEMMs of the precision form: operand buffers, TMA tensor
+// maps (built once per context) and the launchers.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
@@ -25,81 +25,78 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-int make_map(CUtensorMap *m, void *base, int rows, int kpad, int box_rows, int box_k = tc::BK,
-             CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B, bool f16 = false) {
+// 64-byte-swizzled K-major fp32 operand
+int make_map(CUtensorMap *m, float *base, int rows, int kpad, int box_rows) {
   cuuint64_t dims[2] = {(cuuint64_t)kpad, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)kpad * (f16 ? 2 : sizeof(float))};
-  cuuint32_t box[2] = {(cuuint32_t)box_k, (cuuint32_t)box_rows};
+  cuuint64_t strides[1] = {(cuuint64_t)kpad * sizeof(float)};
+  cuuint32_t box[2] = {(cuuint32_t)tc::S_BK, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1u, 1u};
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
   if (!fn) return -1;
-  const CUresult r = fn(m, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
-                                            CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
+                                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : -1;
 }
 }  // namespace
 
-// 64-byte-swizzled K-major fp16 operand map (the slices of the FP64 tensor-core GEMM)
-int tc_make_map_sw64_f16(CUtensorMap *m, void *base, int rows, int kpad, int box_rows, int box_k) {
-  return make_map(m, base, rows, kpad, box_rows, box_k, CU_TENSOR_MAP_SWIZZLE_64B, true);
+// K-major fp16 slices of the exact-slice products, [planes][rows][width]: boxes of one 64-byte
+// swizzle row, box_rows rows and every plane
+int tc_make_map_slices(CUtensorMap *m, void *base, int planes, int rows, int width, int box_rows) {
+  cuuint64_t dims[3] = {(cuuint64_t)width, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {(cuuint64_t)width * 2, (cuuint64_t)width * 2 * rows};
+  cuuint32_t box[3] = {32u, (cuuint32_t)box_rows, (cuuint32_t)planes};
+  cuuint32_t estr[3] = {1u, 1u, 1u};
+  PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+  if (!fn) return -1;
+  const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? 0 : -1;
 }
-
-// Layouts the autotuner chooses from: 4 drained (separate Re / Im operands, N 64, two-stage
-// ring), 5 stacked Re / Im rows with a three-stage 64-byte-swizzle ring (the default and
-// the only layout for real orbitals).
-int tc_variant_bn(int variant) { return variant == 5 ? tc::S_BN : 64; }
-
-int tc_kpad(int npw) { return ((2 * npw + tc::BK - 1) / tc::BK) * tc::BK; }
 
 static int rows_pad(int rows) { return ((rows + 127) / 128) * 128; }
+static int kpad_of(int k) { return ((k + tc::BK - 1) / tc::BK) * tc::BK; }
 
-size_t tc_bytes(int rows_cap, int npw) {
-  const size_t kp = (size_t)tc_kpad(npw);
-  return sizeof(float) * kp * (4 * (size_t)rows_pad(rows_cap) + 2 * (size_t)npw) + 256;
-}
+size_t tc_bytes() { return 256; }
 
 cudaError_t tc_init(TcResources &r, void *mem, int rows_cap, int npw, int variant, bool real) {
   if (variant != 4 && variant != 5) return cudaErrorInvalidValue;
-  if (real && variant != 5) return cudaErrorInvalidValue;  // only the stacked kernel has a real form
+  if (real && variant != 5) return cudaErrorInvalidValue;
   r.variant = variant;
   r.real = real;
   r.rows_cap = rows_cap;
   r.npw = npw;
-  // real basis: K = n_pw (a multiple of the 32-element k block), at most the complex size
-  r.kpad = real ? ((npw + tc::BK - 1) / tc::BK) * tc::BK : tc_kpad(npw);
-  const int rp = rows_pad(rows_cap);
-  const size_t a = (size_t)rp * r.kpad, b = (size_t)npw * r.kpad;
-  float *f = static_cast<float *>(mem);
-  r.a1h = f; r.a1l = f + a; r.a2h = f + 2 * a; r.a2l = f + 3 * a;
-  r.bh = f + 4 * a; r.bl = f + 4 * a + b;
-  r.err = reinterpret_cast<int *>(f + 4 * a + 2 * b);
+  r.kpad = kpad_of(npw);
+  r.err = static_cast<int *>(mem);
+  const cudaError_t e = cudaFuncSetAttribute(tc::k_tc_cgemm_stacked, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::S_SMEM);
+  if (e != cudaSuccess) return e;
+  return cudaMemset(r.err, 0, sizeof(int));
+}
+
+// the transformed-state product's operands: stacked hi / lo rows of S^T and of P_r
+static size_t w_floats(int rows_cap, int npw) {
+  return (size_t)kpad_of(npw) * (4 * (size_t)rows_pad(rows_cap) + 2 * (size_t)npw);
+}
+static cudaError_t w_init(TcResources &r, float *f) {
+  const int rp = rows_pad(r.rows_cap);
+  const size_t a = (size_t)rp * r.kpad, b = (size_t)r.npw * r.kpad;
+  r.a1h = f;
+  r.a1l = f + 2 * a;
+  r.bh = f + 4 * a;
+  r.bl = f + 4 * a + b;
   tc::TcMaps *mp = new tc::TcMaps();
   int bad = 0;
-  if (variant == 5) {
-    // stacked operand: hi in a1h and lo in a1l, 2 rp rows each (spanning a1h..a2l)
-    r.a1l = f + 2 * a;
-    bad |= make_map(&mp->a1h, r.a1h, 2 * rp, r.kpad, 128, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-    bad |= make_map(&mp->a1l, r.a1l, 2 * rp, r.kpad, 128, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-    bad |= make_map(&mp->bh, r.bh, npw, r.kpad, tc::S_BN, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-    bad |= make_map(&mp->bl, r.bl, npw, r.kpad, tc::S_BN, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-  } else {
-    const int bn = tc_variant_bn(variant);
-    bad |= make_map(&mp->a1h, r.a1h, rows_cap, r.kpad, tc::BM) | make_map(&mp->a1l, r.a1l, rows_cap, r.kpad, tc::BM);
-    bad |= make_map(&mp->a2h, r.a2h, rows_cap, r.kpad, tc::BM) | make_map(&mp->a2l, r.a2l, rows_cap, r.kpad, tc::BM);
-    bad |= make_map(&mp->bh, r.bh, npw, r.kpad, bn) | make_map(&mp->bl, r.bl, npw, r.kpad, bn);
-  }
+  bad |= make_map(&mp->a1h, r.a1h, 2 * rp, r.kpad, 128);
+  bad |= make_map(&mp->a1l, r.a1l, 2 * rp, r.kpad, 128);
+  bad |= make_map(&mp->bh, r.bh, r.npw, r.kpad, tc::S_BN);
+  bad |= make_map(&mp->bl, r.bl, r.npw, r.kpad, tc::S_BN);
   if (bad) {
     delete mp;
     return cudaErrorInvalidValue;
   }
   r.maps = mp;
-  cudaError_t e = cudaFuncSetAttribute(tc::k_tc_cgemm_drain<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           tc::TcCfg<64, 2>::SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(tc::k_tc_cgemm_stacked, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::S_SMEM);
-  if (e != cudaSuccess) return e;
-  return cudaMemset(r.err, 0, sizeof(int));
+  return cudaSuccess;
 }
 
 void tc_release(TcResources &r) {
@@ -112,12 +109,10 @@ void tc_release(TcResources &r) {
   r.green = r.direct = false;   // their tensor maps are gone: set up again before any use
 }
 
-static int kpad_of(int k) { return ((k + tc::BK - 1) / tc::BK) * tc::BK; }
-
-size_t tc_green_bytes(int npw, int nv) {
+size_t tc_green_bytes(int rows_cap, int npw, int nv) {
   const size_t kp = (size_t)kpad_of(nv);
   const size_t arows = 2 * (size_t)rows_pad(((npw + 1) / 2 + 63) / 64 * 64);
-  return sizeof(float) * ((size_t)npw * nv + kp * (2 * arows + 2 * (size_t)npw)) + 1024;
+  return sizeof(float) * ((size_t)npw * nv + kp * (2 * arows + 2 * (size_t)npw) + w_floats(rows_cap, npw)) + 2048;
 }
 
 cudaError_t tc_green_init(TcResources &r, void *mem, const float *cv, int nv, cudaStream_t st) {
@@ -134,21 +129,22 @@ cudaError_t tc_green_init(TcResources &r, void *mem, const float *cv, int nv, cu
   r.gah = f; f += arows * kp;
   r.gal = f; f += arows * kp;
   r.gbh = f; f += (size_t)npw * kp;
-  r.gbl = f;
+  r.gbl = f; f += (size_t)npw * kp;
+  cudaError_t e = w_init(r, f);
+  if (e != cudaSuccess) return e;
   tc::TcMaps *mp = new tc::TcMaps();
   int bad = 0;
-  bad |= make_map(&mp->a1h, r.gah, (int)arows, r.kpad_v, 128, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-  bad |= make_map(&mp->a1l, r.gal, (int)arows, r.kpad_v, 128, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-  bad |= make_map(&mp->bh, r.gbh, npw, r.kpad_v, tc::S_BN, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-  bad |= make_map(&mp->bl, r.gbl, npw, r.kpad_v, tc::S_BN, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
+  bad |= make_map(&mp->a1h, r.gah, (int)arows, r.kpad_v, 128);
+  bad |= make_map(&mp->a1l, r.gal, (int)arows, r.kpad_v, 128);
+  bad |= make_map(&mp->bh, r.gbh, npw, r.kpad_v, tc::S_BN);
+  bad |= make_map(&mp->bl, r.gbl, npw, r.kpad_v, tc::S_BN);
   if (bad) {
     delete mp;
     return cudaErrorInvalidValue;
   }
   r.gmaps = mp;
   tc::k_transpose_f<<<dim3((npw + 31) / 32, (nv + 31) / 32), dim3(32, 8), 0, st>>>(nv, npw, cv, r.rvt);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   tc::k_pack_rows<<<dim3((r.kpad_v + 255) / 256, npw), 256, 0, st>>>(r.rvt, nv, r.kpad_v, r.gbh, r.gbl);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   r.green = r.use_green = true;
@@ -190,10 +186,10 @@ cudaError_t tc_direct_init(TcResources &r, void *mem, int no, int naux, int slot
   r.dc = reinterpret_cast<float2 *>(f);
   tc::TcMaps *mp = new tc::TcMaps();
   int bad = 0;
-  bad |= make_map(&mp->a1h, r.dah, (int)arows, r.dkpad, 128, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-  bad |= make_map(&mp->a1l, r.dal, (int)arows, r.dkpad, 128, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-  bad |= make_map(&mp->bh, r.dbh, (int)brows, r.dkpad, tc::S_BN, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
-  bad |= make_map(&mp->bl, r.dbl, (int)brows, r.dkpad, tc::S_BN, tc::S_BK, CU_TENSOR_MAP_SWIZZLE_64B);
+  bad |= make_map(&mp->a1h, r.dah, (int)arows, r.dkpad, 128);
+  bad |= make_map(&mp->a1l, r.dal, (int)arows, r.dkpad, 128);
+  bad |= make_map(&mp->bh, r.dbh, (int)brows, r.dkpad, tc::S_BN);
+  bad |= make_map(&mp->bl, r.dbl, (int)brows, r.dkpad, tc::S_BN);
   if (bad) {
     delete mp;
     return cudaErrorInvalidValue;
@@ -221,47 +217,23 @@ cudaError_t tc_direct(const TcResources &r, const void *mdiag, const float *v, i
 }
 
 cudaError_t tc_pack_b(const TcResources &r, const void *pt, cudaStream_t st) {
-  if (r.green_on()) {   // the pair-interleaved output of tc_green
-    tc::k_pack_b_pairs<<<dim3((r.kpad + 255) / 256, r.npw), 256, 0, st>>>(static_cast<const float2 *>(pt), r.npw,
-                                                                            r.kpad, r.bh, r.bl);
-    return cudaGetLastError();
-  }
-  if (r.real) {
-    tc::k_pack_b_real<<<dim3((r.kpad + 255) / 256, r.npw), 256, 0, st>>>(static_cast<const float *>(pt), r.npw,
-                                                                           r.kpad, r.bh, r.bl);
-    return cudaGetLastError();
-  }
-  tc::k_pack_b<<<dim3((r.kpad / 2 + 255) / 256, r.npw), 256, 0, st>>>(static_cast<const float2 *>(pt), r.npw,
-                                                                        r.kpad, r.bh, r.bl);
+  // the pair-interleaved output of tc_green
+  tc::k_pack_b_pairs<<<dim3((r.kpad + 255) / 256, r.npw), 256, 0, st>>>(static_cast<const float2 *>(pt), r.npw, r.kpad,
+                                                                        r.bh, r.bl);
   return cudaGetLastError();
 }
 
 cudaError_t tc_wgemm(const TcResources &r, const void *st_in, int rows, void *wt, cudaStream_t st) {
-  if (rows > r.rows_cap) return cudaErrorInvalidValue;
+  if (rows > r.rows_cap || !r.maps) return cudaErrorInvalidValue;
   const tc::TcMaps &m = *static_cast<const tc::TcMaps *>(r.maps);
-  const int variant = r.variant;
-  cudaError_t e;
-  if (variant == 5) {
-    const int r64 = ((rows + 63) / 64) * 64;   // zero-filled up to a whole 64-row block
-    if (r.real)
-      tc::k_pack_a_stacked_real<<<dim3((r.kpad + 255) / 256, r64), 256, 0, st>>>(
-          static_cast<const float2 *>(st_in), rows, r.npw, r.kpad, r.a1h, r.a1l);
-    else
-      tc::k_pack_a_stacked<<<dim3((r.kpad / 2 + 255) / 256, r64), 256, 0, st>>>(
-        static_cast<const float2 *>(st_in), rows, r.npw, r.kpad, r.a1h, r.a1l);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    dim3 grid((r.npw + tc::S_BN - 1) / tc::S_BN, r64 / 64);
-    tc::k_tc_cgemm_stacked<<<grid, 160, tc::S_SMEM, st>>>(m.a1h, m.a1l, m.bh, m.bl, rows, r.npw, r.kpad / tc::S_BK,
-                                                          static_cast<float2 *>(wt), r.npw, r.err);
-    return cudaGetLastError();
-  }
-  tc::k_pack_a<<<dim3((r.kpad / 2 + 255) / 256, rows), 256, 0, st>>>(static_cast<const float2 *>(st_in), rows,
-                                                                       r.npw, r.kpad, r.a1h, r.a1l, r.a2h, r.a2l);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  dim3 grid((r.npw + 63) / 64, (rows + tc::BM - 1) / tc::BM);
-  tc::k_tc_cgemm_drain<64><<<grid, 160, tc::TcCfg<64, 2>::SMEM_BYTES, st>>>(
-      m.a1h, m.a1l, m.a2h, m.a2l, m.bh, m.bl, rows, r.npw, r.kpad / tc::BK, static_cast<float2 *>(wt), r.npw,
-      r.err);
+  const int r64 = ((rows + 63) / 64) * 64;   // zero-filled up to a whole 64-row block
+  tc::k_pack_a_stacked_real<<<dim3((r.kpad + 255) / 256, r64), 256, 0, st>>>(static_cast<const float2 *>(st_in), rows,
+                                                                             r.npw, r.kpad, r.a1h, r.a1l);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  dim3 grid((r.npw + tc::S_BN - 1) / tc::S_BN, r64 / 64);
+  tc::k_tc_cgemm_stacked<<<grid, 160, tc::S_SMEM, st>>>(m.a1h, m.a1l, m.bh, m.bl, rows, r.npw, r.kpad / tc::S_BK,
+                                                        static_cast<float2 *>(wt), r.npw, r.err);
   return cudaGetLastError();
 }
 

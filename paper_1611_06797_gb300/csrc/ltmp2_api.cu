@@ -94,8 +94,7 @@ struct ltmp2_ctx {
   unsigned char *d_keep = nullptr;   // screened-pair mask and kept lists (learned form)
   int *d_keep_list = nullptr, *d_keep_count = nullptr;
   TcResources tc;
-  void *tc_mem = nullptr;   // operand buffers of the tensor-core GEMM (owned via allocs)
-  OzResources oz;           // FP64 path: slices of the tensor-core FP64 GEMM (memory owned via allocs)
+  OzResources oz;           // slices of the exact-slice products (memory owned via allocs)
   double ecut_aux = 0.0;               // E_aux of A (Hartree)
   std::vector<double> aux_g2;          // |G|^2 of A in internal order
   // internal cutoff extrapolation: level cutoffs, |A_n| (G != 0), device buffers
@@ -204,26 +203,29 @@ int upload_real_coeff(ltmp2_ctx *c, const ltmp2_system *sys, int row0, int rows,
   return cuda_status(cudaMemcpy(*dst, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
 }
 
-// R_v^T [n_pw][n_v] in the real basis, for the transformed states through the virtual space
-template <typename T>
-int upload_real_coeff_t(ltmp2_ctx *c, const ltmp2_system *sys, const std::vector<int> &order, void **dst) {
-  const int n_pw = sys->n_pw, no = sys->n_occ, nv = sys->n_orb - sys->n_occ;
-  const double r2 = 1.4142135623730950488016887242097;
-  std::vector<T> h((size_t)nv * n_pw);
-  for (int q = 0; q < n_pw; ++q) {
-    const int o = order[q];
-    const int *m = sys->miller + 3 * o;
-    const int kind = (m[0] == 0 && m[1] == 0 && m[2] == 0)
-                         ? 0
-                         : ((m[0] != 0 ? m[0] > 0 : (m[1] != 0 ? m[1] > 0 : m[2] > 0)) ? 1 : 2);
-    for (int a = 0; a < nv; ++a) {
-      const double *src = sys->coeff + ((size_t)(no + a) * n_pw + o) * 2;
-      h[(size_t)q * nv + a] = (T)(kind == 0 ? src[0] : (kind == 1 ? r2 * src[0] : r2 * src[1]));
-    }
-  }
-  int rc = dalloc_bytes(c, dst, h.size() * sizeof(T));
+// exact-slice tensor-core products of a context whose slabs have up to max_cols columns over nz
+// k points, and the virtuals by plane wave that they read (also the CUDA cores' virtual-space route)
+template <typename T> int setup_products(ltmp2_ctx *c, size_t max_cols, int nz, bool simt) {
+  Plan &p = c->p;
+  const int nk = nz;
+  if (p.n_v < 1) return LTMP2_OK;
+  void **vt = p.real_basis ? &p.rvt : &p.cvt;
+  int rc;
+  if (simt && !p.real_basis) return LTMP2_OK;
+  if ((rc = dalloc_bytes(c, vt, (p.real_basis ? sizeof(T) : sizeof(CT<T>)) * (size_t)nk * p.n_v * p.n_pw))) return rc;
+  cudaError_t e = Path<T>::transpose_virtuals(p, *vt, c->stream);
+  if (e != cudaSuccess || simt) return cuda_status(e);
+  const int slices = std::is_same<T, double>::value ? 8 : 4;
+  void *mem = nullptr;
+  const int rows = (int)(max_cols / nz);
+  rc = dalloc_bytes(c, &mem, oz_bytes(slices, rows, p.n_pw, p.n_v, nz, !p.real_basis));
+  if (rc == LTMP2_ERR_OOM) return LTMP2_OK;   // no room for the slices: the CUDA-core products
   if (rc) return rc;
-  return cuda_status(cudaMemcpy(*dst, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
+  e = oz_init(c->oz, mem, slices, rows, p.n_pw, p.n_v, nz, !p.real_basis);
+  if (e == cudaSuccess) e = oz_set_virtuals<T>(c->oz, p.cv, *vt, c->stream);
+  if (e != cudaSuccess) return cuda_status(e);
+  p.oz = &c->oz;
+  return LTMP2_OK;
 }
 
 // FP64: exponent tables of the fixed-point co-densities (the columns' one comes with the slab)
@@ -248,9 +250,6 @@ template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys,
   } else {
     if ((rc = upload_coeff<T>(c, sys->coeff, p.n_pw, p.n_occ, p.n_v, order, &p.cv))) return rc;
   }
-  // CUDA-core GEMMs in the real basis: R_v^T as well, for the large-tau transformed states
-  const bool simt = std::is_same<T, double>::value || (sys->flags & LTMP2_FLAG_SIMT_GEMM);
-  if (p.real_basis && simt && p.n_v > 0 && (rc = upload_real_coeff_t<T>(c, sys, order, &p.rvt))) return rc;
   void *cocc = nullptr;
   if ((rc = upload_coeff<T>(c, sys->coeff, p.n_pw, 0, p.n_occ, order, &cocc))) return rc;
   if ((rc = dalloc_bytes(c, &p.cgrid, cs * n3 * p.n_occ))) return rc;
@@ -290,8 +289,7 @@ template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys,
   if ((rc = dalloc(c, &p.yd, (size_t)p.max_prim * p.n_occ * p.n_occ))) return rc;
   if (std::is_same<T, float>::value && !(sys->flags & LTMP2_FLAG_SIMT_GEMM)) {
     void *tcmem = nullptr;
-    if ((rc = dalloc_bytes(c, &tcmem, tc_bytes((int)max_cols, p.n_pw)))) return rc;
-    c->tc_mem = tcmem;
+    if ((rc = dalloc_bytes(c, &tcmem, tc_bytes()))) return rc;
     e = tc_init(c->tc, tcmem, (int)max_cols, p.n_pw, 5, p.real_basis);
     if (e != cudaSuccess) return cuda_status(e);
     if (p.real_basis) {
@@ -304,15 +302,7 @@ template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys,
     }
     p.tc = &c->tc;
   }
-  if (std::is_same<T, double>::value && p.real_basis && !(sys->flags & LTMP2_FLAG_SIMT_GEMM)) {
-    // the transformed-state GEMM with FP64 accuracy on the tensor cores (exact integer slices)
-    void *omem = nullptr;
-    if ((rc = dalloc_bytes(c, &omem, oz_bytes((int)max_cols, p.n_pw, p.n_v)))) return rc;
-    e = oz_init(c->oz, omem, (int)max_cols, p.n_pw, p.n_v);
-    if (e == cudaSuccess) e = oz_split_cv(c->oz, (const double *)p.cv, c->stream);   // R_v, once
-    if (e != cudaSuccess) return cuda_status(e);
-    p.oz = &c->oz;
-  }
+  if ((rc = setup_products<T>(c, max_cols, 1, (sys->flags & LTMP2_FLAG_SIMT_GEMM) != 0))) return rc;
   e = Path<T>::setup_occupied(p, cocc, c->stream);
   if (e != cudaSuccess) return cuda_status(e);
   e = cudaStreamSynchronize(c->stream);
@@ -377,6 +367,7 @@ int setup_precision_k(ltmp2_ctx *c, const ltmp2_kpoint_system *sys, const std::v
   if ((rc = cuda_status(cudaMemset(p.mdiag, 0, mbytes)))) return rc;
   if ((rc = dalloc(c, &p.sx, (size_t)p.max_prim * p.n_occ * p.n_occ))) return rc;
   if ((rc = dalloc(c, &p.yd, (size_t)p.max_prim * p.n_occ * p.n_occ))) return rc;
+  if ((rc = setup_products<T>(c, max_cols, nk, false))) return rc;
   e = Path<T>::setup_occupied(p, c->k_cocc, c->stream);
   if (e != cudaSuccess) return cuda_status(e);
   return cuda_status(cudaStreamSynchronize(c->stream));
@@ -537,11 +528,7 @@ int apply_tuning(ltmp2_ctx *c, int slab, int variant, int plane_kernel, int plan
   c->p.max_prim = slab;
   c->p.plane_kernel = plane_kernel;
   c->p.plane_ib = plane_ib;
-  if (c->p.tc && variant >= 0 && variant != c->tc.variant) {
-    tc_release(c->tc);
-    cudaError_t e = tc_init(c->tc, c->tc_mem, c->tc.rows_cap, c->p.n_pw, variant, c->tc.real);
-    if (e != cudaSuccess) return cuda_status(e);
-  }
+  if (c->p.tc && variant >= 0) c->tc.variant = variant;
   return LTMP2_OK;
 }
 
@@ -561,8 +548,7 @@ template <typename T> int tune_ctx(ltmp2_ctx *c, int *slab_out, int *var_out) {
   }
   std::vector<int> slabs;
   for (int sl = std::min(c->slab_capacity, p.n_prim); sl >= 1 && slabs.size() < 4; sl /= 2) slabs.push_back(sl);
-  std::vector<int> variants =
-      p.tc ? (c->tc.real ? std::vector<int>{5} : std::vector<int>{5, 4}) : std::vector<int>{-1};
+  const std::vector<int> variants{p.tc ? 5 : -1};
   cudaEvent_t a = nullptr, b = nullptr;
   if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return LTMP2_ERR_CUDA;
   double best = 1e300;
@@ -1253,7 +1239,7 @@ int ltmp2_set_tuning(ltmp2_ctx *ctx, const int *values) {
   if (values[4] == 1 && !ctx->tc.green) {
     // first use: R_v^T and its split, once (the Green's function on the tensor cores)
     void *gmem = nullptr;
-    if ((rc = dalloc_bytes(ctx, &gmem, tc_green_bytes(p.n_pw, p.n_v)))) return rc;
+    if ((rc = dalloc_bytes(ctx, &gmem, tc_green_bytes(ctx->tc.rows_cap, p.n_pw, p.n_v)))) return rc;
     cudaError_t e = tc_green_init(ctx->tc, gmem, (const float *)p.cv, p.n_v, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_status(e);

@@ -144,6 +144,18 @@ cudaError_t Path<T>::setup_occupied(const Plan &p, const void *c_occ_dev, cudaSt
   return cudaGetLastError();
 }
 
+template <typename T> cudaError_t Path<T>::transpose_virtuals(const Plan &p, void *out, cudaStream_t st) {
+  const dim3 grid((p.n_pw + 31) / 32, (p.n_v + 31) / 32), block(32, 8);
+  const size_t n = (size_t)p.n_v * p.n_pw;
+  for (int k = 0; k < (p.nk > 0 ? p.nk : 1); ++k) {
+    if (p.real_basis) k_transpose<T><<<grid, block, 0, st>>>(p.n_v, p.n_pw, (const T *)p.cv, (T *)out);
+    else k_transpose<cpx<T>><<<grid, block, 0, st>>>(p.n_v, p.n_pw, (const cpx<T> *)p.cv + k * n, (cpx<T> *)out + k * n);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 template <typename T> cudaError_t Path<T>::overlap_setup(const Plan &p, cudaStream_t st) {
   // r_a transposed into pt ([n_pw][n_v]); pt is free on this route (no Green's function)
   k_transpose<T><<<dim3((p.n_pw + 31) / 32, (p.n_v + 31) / 32), dim3(32, 8), 0, st>>>(p.n_v, p.n_pw, (const T *)p.cv,
@@ -183,16 +195,13 @@ cudaError_t Path<T>::green(const Plan &p, double tau, cudaStream_t st, StageTime
     }
   }
   const int M = p.n_pw, N = p.n_pw, K = p.nv_tau > 0 ? p.nv_tau : p.n_v;
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
-  if constexpr (std::is_same<T, double>::value) {
-    if (p.oz && p.rvt && oz_green_fits(*p.oz)) {
-      // FP64 on the tensor cores: P_r = (R_v'^T D') R_v', then its slices for the W product
-      if ((e = oz_green(*p.oz, (const double *)p.rvt, (const double *)p.dscale + p.n_occ, K, (double *)p.pt, st)) !=
-          cudaSuccess)
-        return e;
-      return oz_split_b(*p.oz, (const double *)p.pt, st);
-    }
+  if (p.oz) {
+    // on the tensor cores by exact slices, then the result's own slices for the W product
+    const void *dv = (const T *)p.dscale + p.n_occ;
+    if ((e = oz_green<T>(*p.oz, p.real_basis ? p.rvt : p.cvt, dv, 0, K, p.pt, st)) != cudaSuccess) return e;
+    return oz_split_b<T>(*p.oz, p.pt, st);
   }
+  dim3 grid((N + 63) / 64, (M + 63) / 64);
   if (p.real_basis) {
     // P_r[q][p] = sum_a r_a(q) e^{-(e_a-mu)tau} r_a(p), r_a the real coordinates of a
     k_rgemm<T, T, false><<<grid, 256, 0, st>>>(M, N, K, (const T *)p.cv, p.n_pw, (const T *)p.cv, p.n_pw,
@@ -203,14 +212,7 @@ cudaError_t Path<T>::green(const Plan &p, double tau, cudaStream_t st, StageTime
                                                   (const cpx<T> *)p.cv, p.n_pw,
                                                   (const T *)p.dscale + p.n_occ, (cpx<T> *)p.pt, p.n_pw);
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if constexpr (std::is_same<T, float>::value) {
-    if (p.tc) return tc_pack_b(*p.tc, p.pt, st);  // split P into TF32 hi/lo operands
-  } else {
-    if (p.oz) return oz_split_b(*p.oz, (const double *)p.pt, st);   // exact integer slices of P_r
-  }
-  return cudaSuccess;
+  return cudaGetLastError();
 }
 
 template <typename T>
@@ -244,38 +246,32 @@ cudaError_t Path<T>::slab_pre(const Plan &p, int gp0, int np, cudaStream_t st, S
     } else if (p.w_virtual) {
       // X^T = (U S)^T R_v'^T [ncols][nv] in the z1 buffer (free until the z transform; it
       // holds n n_dorb >= n_pw > nv values per column), then W^T = X^T D' R_v'
-      if constexpr (std::is_same<T, double>::value) {
-        if (p.oz) {
-          if ((e = oz_virtual(*p.oz, p.st, ncols, (const double *)p.rvt, (const double *)p.dscale + p.n_occ, p.nv_tau,
-                              p.z1, p.wt, st)) != cudaSuccess)
-            return e;
-          done = true;
-        }
-      }
-    }
-    if (p.w_virtual && !done) {
       const int nv = p.nv_tau;
-      dim3 gx((nv + 63) / 64, (ncols + 63) / 64);
-      k_rgemm<T, cpx<T>, true><<<gx, 256, 0, st>>>(ncols, nv, p.n_pw, (const cpx<T> *)p.st, p.n_pw,
-                                                    (const T *)p.rvt, p.n_v, nullptr, (cpx<T> *)p.z1, nv);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      dim3 gw((p.n_pw + 63) / 64, (ncols + 63) / 64);
-      k_rgemm<T, cpx<T>, true><<<gw, 256, 0, st>>>(ncols, p.n_pw, nv, (const cpx<T> *)p.z1, nv, (const T *)p.cv,
-                                                    p.n_pw, (const T *)p.dscale + p.n_occ, (cpx<T> *)p.wt,
-                                                    p.n_pw);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      const T *dv = (const T *)p.dscale + p.n_occ;
+      if (p.oz) {
+        if ((e = oz_virtual<T>(*p.oz, p.st, ncols, dv, nv, p.z1, p.wt, st)) != cudaSuccess) return e;
+      } else {
+        dim3 gx((nv + 63) / 64, (ncols + 63) / 64);
+        k_rgemm<T, cpx<T>, true><<<gx, 256, 0, st>>>(ncols, nv, p.n_pw, (const cpx<T> *)p.st, p.n_pw,
+                                                      (const T *)p.rvt, p.n_v, nullptr, (cpx<T> *)p.z1, nv);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        dim3 gw((p.n_pw + 63) / 64, (ncols + 63) / 64);
+        k_rgemm<T, cpx<T>, true><<<gw, 256, 0, st>>>(ncols, p.n_pw, nv, (const cpx<T> *)p.z1, nv, (const T *)p.cv,
+                                                      p.n_pw, dv, (cpx<T> *)p.wt, p.n_pw);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      }
       done = true;
     }
     if constexpr (std::is_same<T, float>::value) {
-      if (p.tc && !done) {
+      // the opt-in 3xTF32 Green's function leaves its operands to the 3xTF32 product
+      if (!done && p.tc && p.tc->green_on()) {
         if ((e = tc_wgemm(*p.tc, p.st, ncols, p.wt, st)) != cudaSuccess) return e;
         done = true;
       }
-    } else {
-      if (p.oz && !done) {   // FP64-accurate products on the tensor cores
-        if ((e = oz_wgemm(*p.oz, p.st, ncols, p.wt, st)) != cudaSuccess) return e;
-        done = true;
-      }
+    }
+    if (p.oz && !done) {
+      if ((e = oz_wgemm<T>(*p.oz, p.st, ncols, p.wt, st)) != cudaSuccess) return e;
+      done = true;
     }
     if (!done) {
       dim3 grid((p.n_pw + 63) / 64, (ncols + 63) / 64);
@@ -385,6 +381,10 @@ template <typename T> cudaError_t Path<T>::green_k(const Plan &p, double tau, cu
   k_dscale_k<T><<<dim3((p.n_orb + 255) / 256, p.nk), 256, 0, st>>>(p, p.eps, p.mu, tau, (T *)p.dscale);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (p.oz) {
+    if ((e = oz_green<T>(*p.oz, p.cvt, (const T *)p.dscale + p.no_k, p.n_orb, p.n_v, p.pt, st)) != cudaSuccess) return e;
+    return oz_split_b<T>(*p.oz, p.pt, st);
+  }
   const size_t pw2 = (size_t)p.n_pw * p.n_pw;
   dim3 grid((p.n_pw + 63) / 64, (p.n_pw + 63) / 64);
   for (int k = 0; k < p.nk; ++k) {
@@ -414,7 +414,8 @@ cudaError_t Path<T>::slab_k(const Plan &p, int gp0, int np, double coef, cudaStr
     ScopedStage s(tm, kStageWGemm);
     const size_t pw2 = (size_t)p.n_pw * p.n_pw;
     dim3 grid((p.n_pw + 63) / 64, (rows_k + 63) / 64);
-    for (int kt = 0; kt < p.nk; ++kt) {
+    if (p.oz && (e = oz_wgemm<T>(*p.oz, p.st, rows_k, p.wt, st)) != cudaSuccess) return e;
+    for (int kt = 0; kt < p.nk && !p.oz; ++kt) {
       const size_t row0 = (size_t)kt * rows_k * p.n_pw;
       k_cgemm<T, true, false><<<grid, 256, 0, st>>>(rows_k, p.n_pw, p.n_pw, (const cpx<T> *)p.st + row0, p.n_pw,
                                                     (const cpx<T> *)p.pt + kt * pw2, p.n_pw, nullptr,

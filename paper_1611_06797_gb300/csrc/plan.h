@@ -6,18 +6,18 @@
 
 namespace ltmp2 {
 
-// Operands, tensor maps and error flag of the tcgen05 3xTF32 GEMM (precision form).
-struct OzResources;   // FP64 tensor-core GEMM resources (below)
+struct OzResources;   // exact-slice tensor-core products (below)
+// Operands, tensor maps and error flag of the tcgen05 3xTF32 GEMMs (precision form).
 struct TcResources {
   int rows_cap = 0, npw = 0, kpad = 0;
-  int variant = 5;         // 4 drained N=64, 5 stacked Re/Im rows (default; the only one for real orbitals)
-  bool real = false;       // real-basis Green's function: K = n_pw (variant 5 only)
-  float *a1h = nullptr, *a1l = nullptr, *a2h = nullptr, *a2l = nullptr, *bh = nullptr, *bl = nullptr;
+  int variant = 5;         // ltmp2_set_tuning's GEMM variant: 5, or 4 for general orbitals (one kernel serves both)
+  bool real = false;       // real orbitals
   int *err = nullptr;      // device flag: a bounded wait ran out
-  void *maps = nullptr;    // host copy of the six TMA tensor maps
-  // Green's function on the tensor cores (real basis): P_r = R_v^T D R_v with K = n_v,
-  // two real rows of R_v^T D per complex row of the stacked kernel
+  // Green's function on the tensor cores (real basis, opt-in): P_r = R_v^T D R_v with K = n_v,
+  // two real rows of R_v^T D per complex row of the stacked kernel, and the transformed states' product with it
   bool green = false;
+  float *a1h = nullptr, *a1l = nullptr, *bh = nullptr, *bl = nullptr;
+  void *maps = nullptr;    // host copy of the transformed-state product's tensor maps
   int nv = 0, kpad_v = 0, grows = 0;   // virtuals, padded K, complex rows ceil(n_pw / 2)
   float *rvt = nullptr;                // [n_pw][n_v] R_v^T
   float *gah = nullptr, *gal = nullptr, *gbh = nullptr, *gbl = nullptr;
@@ -34,17 +34,15 @@ struct TcResources {
   bool green_on() const { return green && use_green; }
   bool direct_on() const { return direct && use_direct; }
 };
-int tc_kpad(int npw);
-size_t tc_bytes(int rows_cap, int npw);
-cudaError_t tc_init(TcResources &r, void *mem, int rows_cap, int npw, int variant, bool real = false);
-int tc_variant_bn(int variant);
+size_t tc_bytes();
+cudaError_t tc_init(TcResources &r, void *mem, int rows_cap, int npw, int variant, bool real);
 void tc_release(TcResources &r);
-cudaError_t tc_pack_b(const TcResources &r, const void *pt, cudaStream_t st);
 // Green's function on the tensor cores: device bytes, set-up (transpose and split of the
 // virtuals' real coordinates cv [n_v][n_pw], once) and one build into pt (pair-interleaved)
-size_t tc_green_bytes(int npw, int nv);
+size_t tc_green_bytes(int rows_cap, int npw, int nv);
 cudaError_t tc_green_init(TcResources &r, void *mem, const float *cv, int nv, cudaStream_t st);
 cudaError_t tc_green(const TcResources &r, const float *dv, void *pt, cudaStream_t st);
+cudaError_t tc_pack_b(const TcResources &r, const void *pt, cudaStream_t st);
 // direct term on the tensor cores: bytes and set-up for up to `slots` primary G' per slab,
 // and the pair sums Y [np][n_o][n_o] of one slab from its diagonal co-densities
 size_t tc_direct_bytes(int no, int naux, int slots);
@@ -114,7 +112,7 @@ struct Plan {
   double *esum = nullptr;    // [4]: E_d, E_x, imag parts
   int max_prim = 0;          // primary G' per slab (capacity)
   TcResources *tc = nullptr; // precision form: tcgen05 GEMM resources (host pointer), or null
-  OzResources *oz = nullptr; // FP64 path: tensor-core FP64 GEMM resources (host pointer), or null
+  OzResources *oz = nullptr; // exact-slice tensor-core products (host pointer), or null: CUDA cores
   int plane_kernel = 2;      // 0: k_planes, 1: k_planes2, 2: k_planes3, 3: k_planes4 (set-up: 3 in FP32;
                              // the autotuner may change it)
   // screened exchange pairs (learned form); all null = every pair contracted
@@ -143,11 +141,12 @@ struct Plan {
   // e^{-(e_a - e_LUMO) tau} >= 2^-L are the first nv_tau of them; the others are left out
   // of the Green's function and of the transformed states (0 = all n_v).  With w_virtual
   // the transformed states go through the virtual space, W^T = ((U S)^T R_v'^T D') R_v'
-  // (real basis, CUDA-core GEMMs; rvt = R_v^T [n_pw][n_v]), which costs 4 n_pw nv_tau
+  // (real basis; rvt = R_v^T [n_pw][n_v]), which costs 4 n_pw nv_tau
   // multiply-adds per column against 2 n_pw^2 through P_r, and no Green's function is built.
   int nv_tau = 0;
   bool w_virtual = false;
   void *rvt = nullptr;
+  void *cvt = nullptr;       // general orbitals: the virtual coefficients by plane wave, cpx<T> [nk or 1][n_pw][n_v]
   // k-point sampling (Sec. II C-D), nk > 0: n_occ counts composite occupied orbitals
   // k n_o + i over the mesh, n_orb / n_v are per k, cv [nk][n_v][n_pw], pt [nk][n_pw][n_pw],
   // dscale [nk][n_orb]; the auxiliary set A (daux, aux_m) is the ball that holds every
@@ -163,35 +162,42 @@ struct Plan {
   int slots_per_prim() const { return (real_orb && nk == 0) ? 1 : 2; }
 };
 
-// FP64 products on the tensor cores by exact integer slices (gemm_f64tc.cuh): the FP64
-// path's transformed-state GEMM in the real basis, W^T = (U S)^T P_r.
+// Products on the tensor cores by exact integer slices (gemm_f64tc.cuh): the Green's function
+// and the transformed states, of FP64 accuracy from 8 slices per operand, of FP32 accuracy from 4.
+// Real basis: P_r and W^T = (U S)^T P_r; general orbitals: the complex P^T of each of nz k
+// points and W^T = S^T P^T, as real products over interleaved real and imaginary parts.
 struct OzResources {
-  int rows_cap = 0, npw = 0, kpad = 0, arows = 0;  // complex rows, K = n_pw, padded K, stacked rows
-  int nv = 0;                                      // virtuals (rows of the static slices bv)
-  // FP16 slices (integers of at most 8 bits) [8][arows][kpad], [8][npw][kpad]
-  void *a = nullptr, *b = nullptr;
-  void *bv = nullptr;                              // slices of R_v [8][nv][kpad], once per context
-  double *sa = nullptr, *sb = nullptr, *sbv = nullptr;  // row scales (powers of two)
+  int slices = 0, nz = 1;
+  bool cplx = false;
+  int rows_cap = 0, npw = 0, nv = 0;   // complex rows of a slab per product, plane waves, virtuals
+  int kpad = 0, arows = 0;             // padded K, rows per slice of A
+  // FP16 slices (integers of at most 8 bits) [slices][rows][kpad] and one exponent per row:
+  // a [arows] the left operand of the moment, b [nz npw] the Green's function of a tau, and
+  // once per context bt [nz npw] the virtuals' coefficients by plane wave, bv [nv] by virtual (real basis)
+  void *a = nullptr, *b = nullptr, *bt = nullptr, *bv = nullptr;
+  int *sa = nullptr, *sb = nullptr, *sbt = nullptr, *sbv = nullptr;
   int *err = nullptr;                              // device flag: a bounded wait ran out
-  void *maps = nullptr;                            // host copy of the three tensor maps
+  void *maps = nullptr;                            // host copy of the tensor maps
 };
-size_t oz_bytes(int rows_cap, int npw, int nv);
-cudaError_t oz_init(OzResources &r, void *mem, int rows_cap, int npw, int nv);
+size_t oz_bytes(int slices, int rows_cap, int npw, int nv, int nz, bool cplx);
+cudaError_t oz_init(OzResources &r, void *mem, int slices, int rows_cap, int npw, int nv, int nz, bool cplx);
 void oz_release(OzResources &r);
-// slices of the virtuals' real coordinates R_v (cv [nv][npw]), once
-cudaError_t oz_split_cv(const OzResources &r, const double *cv, cudaStream_t st);
-// the Green's function P_r = R_v'^T D' R_v' over the first nv virtuals (dv: their weights)
-// into pr [npw][npw]; needs oz_green_fits (n_pw rows fit the A slices)
-bool oz_green_fits(const OzResources &r);
-cudaError_t oz_green(const OzResources &r, const double *rvt, const double *dv, int nv, double *pr, cudaStream_t st);
-// W^T through the virtual space: X^T = S^T R_v'^T into x (complex [rows][nv]), then
+// slices of the virtuals, once: cv [nv][npw] real coordinates (real basis) and cvt, the same by
+// plane wave [npw][nv] (general orbitals: complex, [nz][npw][nv])
+template <typename T> cudaError_t oz_set_virtuals(const OzResources &r, const void *cv, const void *cvt, cudaStream_t st);
+// the Green's function over the first nv virtuals (dv: their weights, zscale apart per k point)
+// into pr: P_r = R_v'^T D' R_v' [npw][npw], or P^T [nz][npw][npw]
+template <typename T>
+cudaError_t oz_green(const OzResources &r, const void *cvt, const void *dv, int zscale, int nv, void *pr, cudaStream_t st);
+// W^T through the virtual space (real basis): X^T = S^T R_v'^T into x (complex [rows][nv]), then
 // W^T = X^T D' R_v' into wt (complex [rows][npw])
-cudaError_t oz_virtual(const OzResources &r, const void *st_in, int rows, const double *rvt, const double *dv, int nv,
-                       void *x, void *wt, cudaStream_t st);
-// slices of P_r (real symmetric [npw][npw]) as the B operand, once per tau
-cudaError_t oz_split_b(const OzResources &r, const double *pr, cudaStream_t st);
-// W^T (complex [rows][npw]) = S^T (complex [rows][npw]) P_r
-cudaError_t oz_wgemm(const OzResources &r, const void *st_in, int rows, void *wt, cudaStream_t st);
+template <typename T>
+cudaError_t oz_virtual(const OzResources &r, const void *st_in, int rows, const void *dv, int nv, void *x, void *wt,
+                       cudaStream_t st);
+// slices of the Green's function as the B operand, once per tau
+template <typename T> cudaError_t oz_split_b(const OzResources &r, const void *pr, cudaStream_t st);
+// W^T (complex [nz][rows][npw]) = S^T ([nz][rows][npw]) times the Green's function
+template <typename T> cudaError_t oz_wgemm(const OzResources &r, const void *st_in, int rows, void *wt, cudaStream_t st);
 // the bounded-wait flag: LTMP2_OK, or LTMP2_ERR_TIMEOUT (flag cleared), or LTMP2_ERR_CUDA
 int oz_check(const OzResources &r);
 
@@ -222,22 +228,20 @@ enum Stage {
 
 // Per-precision entry points (kernels_f64.cu / kernels_f32.cu)
 template <typename T> struct Path {
-  // kernel launches per Green's function build and per slab (the tcgen05 path of the
-  // precision form adds one operand-packing launch to each)
+  // kernel launches per Green's function build and per slab
   static int green_launches(const Plan &p) {
     if (p.route == 1 || p.w_virtual) return 1;
-    if (p.tc) return p.tc->green_on() ? 4 : 3;
-    if (p.oz) return oz_green_fits(*p.oz) && p.rvt ? 5 : 3;   // dscale, [split, split, product | product], split of P_r
-    return 2;
+    return p.oz || (p.tc && p.tc->green_on()) ? 4 : 2;   // dscale, split, product, split of the result
   }
   static int slab_launches(const Plan &p) {
     if (p.route == 1) return 7 + (p.precision == 0 ? 1 : 0) + (p.n_lev > 1 ? 1 : 0);   // no gather, CUDA-core product
-    // W: one product; FP64 on the tensor cores: split + product; through the virtual space:
-    // two products (CUDA cores) or split, product, split, split, product (tensor cores)
-    const int w = p.w_virtual ? (p.oz ? 5 : 2) : (p.oz ? 2 : 1);
-    return (p.tc ? 8 : 7) - 1 + (p.precision == 0 ? 1 : 0) + w + (p.real_basis ? 1 : 0) + (p.n_lev > 1 ? 1 : 0) +
+    // W: one product, on the tensor cores after a split; twice that through the virtual space
+    const int w = (p.w_virtual ? 2 : 1) * (p.oz ? 2 : 1);
+    return 6 + (p.precision == 0 ? 1 : 0) + w + (p.real_basis ? 1 : 0) + (p.n_lev > 1 ? 1 : 0) +
            (p.tc && p.tc->direct_on() && p.n_lev < 2 ? 2 : 0);   // direct term: pack, product, combine
   }
+  // setup: cv [nk or 1][n_v][n_pw] by plane wave, [nk or 1][n_pw][n_v]
+  static cudaError_t transpose_virtuals(const Plan &p, void *out, cudaStream_t st);
   // route 1 setup: the overlap densities of every primary G' into rt (uses st and pt as
   // scratch; pt holds the transposed virtual coordinates meanwhile)
   static cudaError_t overlap_setup(const Plan &p, cudaStream_t st);
@@ -274,8 +278,8 @@ template <typename T> struct Path {
   // one slab of primary supercell transfers Q' [gp0, gp0 + np)
   static cudaError_t green_k(const Plan &p, double tau, cudaStream_t st, StageTimer *tm);
   static cudaError_t slab_k(const Plan &p, int gp0, int np, double coef, cudaStream_t st, StageTimer *tm);
-  static int green_k_launches(const Plan &p) { return 1 + p.nk; }
-  static int slab_k_launches(const Plan &p) { return 6 + p.nk + (p.precision == 0 ? 1 : 0); }
+  static int green_k_launches(const Plan &p) { return p.oz ? 4 : 1 + p.nk; }
+  static int slab_k_launches(const Plan &p) { return 6 + (p.oz ? 2 : p.nk) + (p.precision == 0 ? 1 : 0); }
   // opposite-spin direct term of one slab (alpha plan pa, beta plan pb, same slab):
   // y [slab][na][nb] scratch, acc [na][nb] accumulated
   static cudaError_t direct_cross(const Plan &pa, const Plan &pb, int gp0, int np, double coef, double *y,
