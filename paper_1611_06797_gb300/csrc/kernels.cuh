@@ -62,6 +62,20 @@ template <> struct Codensity<double> {
   }
 };
 
+// column of a slab -> its orbital, the number of items i, and the item's place in tbuf: every
+// i (or the kept list), or i <= j in a pass of the pairs' symmetry (sym.cuh)
+__device__ __forceinline__ int cols_per_slot(const Plan &p) { return p.sym_nj ? p.sym_nj : p.n_occ; }
+__device__ __forceinline__ int col_orbital(const Plan &p, int col) {
+  return p.sym_nj ? p.sym_j0 + col % p.sym_nj : col % p.n_occ;
+}
+__device__ __forceinline__ int col_items(const Plan &p, int j) {
+  if (p.keep_count) return p.sym_nj ? p.keep_upto[j] : p.keep_count[j];
+  return p.sym_nj ? j + 1 : p.n_occ;
+}
+__device__ __forceinline__ size_t item_of(const Plan &p, int col, int i) {
+  return (size_t)col * (p.sym_nj ? p.sym_j0 + p.sym_nj : p.n_occ) + i;
+}
+
 // position in A of the G' carried by a slot of the current slab
 __device__ __forceinline__ int slot_aux(const Plan &p, int gp0, int np, int slot) {
   return slot < np ? p.prim[gp0 + slot] : p.aux_neg[p.prim[gp0 + slot - np]];
@@ -286,11 +300,11 @@ template <typename T> __device__ __forceinline__ cpx<T> from_real_basis(const in
 }
 
 // S^T in the real basis: row (slot, j) = U (e^{(e_j-mu)tau} e^{-iG'r} phi_j); unscaled
-// (factor 1) for the overlap densities of the paper's route
+// (factor 1) for the overlap densities of the paper's route and for the pairs' symmetry
 template <typename T>
 __global__ void k_gather_s_real(Plan p, int gp0, int np, cpx<T> *__restrict__ st, bool unscaled = false) {
   const int col = blockIdx.y;
-  const int slot = col / p.n_occ, j = col % p.n_occ;
+  const int slot = col / cols_per_slot(p), j = col_orbital(p, col);
   const int g = slot_aux(p, gp0, np, slot);
   const int gx = p.aux_m[3 * g], gy = p.aux_m[3 * g + 1], gz = p.aux_m[3 * g + 2];
   const T dj = unscaled ? T(1) : ((const T *)p.dscale)[j];
@@ -335,12 +349,12 @@ __global__ void k_transpose(int rows, int cols, const T *__restrict__ in, T *__r
 // S^T[(slot, j)][q] = e^{(e_j - mu) tau} c_j((G_q + G'_slot) mod grid): the plane-wave
 // coefficients of e^{-iG'r} phi_j restricted to the orbital sphere, scaled.
 template <typename T>
-__global__ void k_gather_s(Plan p, int gp0, int np, cpx<T> *__restrict__ st) {
+__global__ void k_gather_s(Plan p, int gp0, int np, cpx<T> *__restrict__ st, bool unscaled = false) {
   const int col = blockIdx.y;
-  const int slot = col / p.n_occ, j = col % p.n_occ;
+  const int slot = col / cols_per_slot(p), j = col_orbital(p, col);
   const int g = slot_aux(p, gp0, np, slot);
   const int gx = p.aux_m[3 * g], gy = p.aux_m[3 * g + 1], gz = p.aux_m[3 * g + 2];
-  const T dj = ((const T *)p.dscale)[j];
+  const T dj = unscaled ? T(1) : ((const T *)p.dscale)[j];
   const int n = p.n;
   const cpx<T> *cg = (const cpx<T> *)p.cgrid + (size_t)j * n * n * n;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < p.n_pw; q += gridDim.x * blockDim.x) {
@@ -435,8 +449,7 @@ __global__ void k_planes(Plan p, int ib, const cpx<T> *__restrict__ z1, cpx<T> *
   const cpx<T> *u = (const cpx<T> *)p.u;
   const int nxa = p.mxhi_aux - p.mxlo_aux + 1;
   // occupied i of this column: all, or the kept list when exchange pairs are screened
-  const int jcol = col % no;
-  const int ni = p.keep_count ? p.keep_count[jcol] : no;
+  const int jcol = col_orbital(p, col), ni = col_items(p, jcol);
   const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
   for (int i0 = 0; i0 < ni; i0 += ib) {
     const int nb = min(ib, ni - i0);
@@ -471,7 +484,7 @@ __global__ void k_planes(Plan p, int ib, const cpx<T> *__restrict__ z1, cpx<T> *
     for (int e = tid; e < nb * p.n_daux; e += nth) {
       const int il = e / p.n_daux, d = e % p.n_daux;
       const int4 c = p.daux[d];
-      const size_t item = (size_t)col * no + (ilist ? ilist[i0 + il] : i0 + il);
+      const size_t item = item_of(p, col, ilist ? ilist[i0 + il] : i0 + il);
       tbuf[(item * N + z) * p.n_daux + d] = wk[(il * N + wrapn(c.y, N)) * P + wrapn(c.x, N)];
     }
     __syncthreads();
@@ -510,8 +523,7 @@ __global__ void k_planes2(Plan p, int ib, const cpx<T> *__restrict__ z1, cpx<T> 
   plane_inverse<T, N>(p, z1 + ((size_t)col * N + z) * p.n_dorb, xp);   // ends with a barrier
   const cpx<T> *u = (const cpx<T> *)p.u;
   // occupied i of this column: all, or the kept list when exchange pairs are screened
-  const int jcol = col % no;
-  const int ni = p.keep_count ? p.keep_count[jcol] : no;
+  const int jcol = col_orbital(p, col), ni = col_items(p, jcol);
   const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
   for (int i0 = 0; i0 < ni; i0 += ib) {
     const int nb = min(ib, ni - i0);
@@ -553,7 +565,7 @@ __global__ void k_planes2(Plan p, int ib, const cpx<T> *__restrict__ z1, cpx<T> 
     __syncthreads();
     for (int e = tid; e < nb * nd; e += nth) {
       const int il = e / nd, d = e % nd;
-      const size_t item = (size_t)col * no + (ilist ? ilist[i0 + il] : i0 + il);
+      const size_t item = item_of(p, col, ilist ? ilist[i0 + il] : i0 + il);
       tbuf[(item * N + z) * nd + d] = ob[(size_t)il * nd + d];
     }
   }
@@ -591,8 +603,7 @@ __device__ __forceinline__ void planes3_body(const Plan &p, int ib, int z, int c
   plane_inverse<T, N>(p, z1 + ((size_t)col * N + z) * p.n_dorb, xp);   // ends with a barrier
   const cpx<T> *ut = (const cpx<T> *)p.ut;
   const T *utr = (const T *)p.utr;
-  const int jcol = col % no;
-  const int ni = p.keep_count ? p.keep_count[jcol] : no;
+  const int jcol = col_orbital(p, col), ni = col_items(p, jcol);
   const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
   for (int i0 = 0; i0 < ni; i0 += ib) {
     const int nb = min(ib, ni - i0);
@@ -635,7 +646,7 @@ __device__ __forceinline__ void planes3_body(const Plan &p, int ib, int z, int c
     }
     __syncthreads();
     for (int il = 0; il < nb; ++il) {
-      const size_t item = (size_t)col * no + (ilist ? ilist[i0 + il] : i0 + il);
+      const size_t item = item_of(p, col, ilist ? ilist[i0 + il] : i0 + il);
       cpx<T> *dst = tbuf + (item * N + z) * nd;
       const cpx<T> *src = wk + (size_t)il * Q;
       for (int d = tid; d < nd; d += nth) dst[d] = src[ytab[d]];
@@ -726,8 +737,7 @@ __device__ __forceinline__ void planes3_body_fx(const Plan &p, int ib, int z, in
   __syncthreads();
   const cpx<W> *ut = (const cpx<W> *)p.ut;
   const W *utr = (const W *)p.utr;
-  const int jcol = col % no;
-  const int ni = p.keep_count ? p.keep_count[jcol] : no;
+  const int jcol = col_orbital(p, col), ni = col_items(p, jcol);
   const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
   const int esh = p.wen3[col] - ew;   // >= 0 (a sentinel for a state that is not finite)
   for (int i0 = 0; i0 < ni; i0 += ib) {
@@ -773,7 +783,7 @@ __device__ __forceinline__ void planes3_body_fx(const Plan &p, int ib, int z, in
     __syncthreads();
     for (int il = 0; il < nb; ++il) {
       const int iocc = ilist ? ilist[i0 + il] : i0 + il;
-      const size_t item = (size_t)col * no + iocc;
+      const size_t item = item_of(p, col, iocc);
       cpx<W> *dst = tbuf + (item * N + z) * nd;
       const cpx<W> *src = wk + (size_t)il * Q;
       const int sh = min(62, esh + p.uen3[iocc] - p.uen[iocc * N + z]);
@@ -845,8 +855,7 @@ __global__ void __launch_bounds__(32 * kPlaneWarps) k_planes4(Plan p, int ib, co
   cpx<T> *wk = wk_all + (size_t)warp * ib * Q;
   const cpx<T> *ut = (const cpx<T> *)p.ut;
   const T *utr = (const T *)p.utr;
-  const int jcol = col % no;
-  const int ni = p.keep_count ? p.keep_count[jcol] : no;
+  const int jcol = col_orbital(p, col), ni = col_items(p, jcol);
   const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
   for (int i0 = warp * ib; i0 < ni; i0 += kPlaneWarps * ib) {
     const int nb = min(ib, ni - i0);
@@ -884,7 +893,7 @@ __global__ void __launch_bounds__(32 * kPlaneWarps) k_planes4(Plan p, int ib, co
     }
     __syncwarp();
     for (int il = 0; il < nb; ++il) {
-      const size_t item = (size_t)col * no + (ilist ? ilist[i0 + il] : i0 + il);
+      const size_t item = item_of(p, col, ilist ? ilist[i0 + il] : i0 + il);
       cpx<T> *dst = tbuf + (item * N + z) * nd;
       const cpx<T> *src = wk + (size_t)il * Q;
       for (int d = lane; d < nd; d += 32) dst[d] = src[ytab[d]];

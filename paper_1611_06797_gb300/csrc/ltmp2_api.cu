@@ -101,8 +101,11 @@ struct ltmp2_ctx {
   std::vector<double> lev_ecut;
   std::vector<int> lev_count;
   bool lev_alloc = false, lev_done = false;
+  // whole energies by the pairs' symmetry: the index set on the host, and room for its row groups
+  std::vector<int> sym_order;
+  int2 *d_sym_groups = nullptr;
   // spin-unrestricted pairing (this context as the alpha channel): opposite-spin scratch
-  double *d_cross_y = nullptr, *d_cross_acc = nullptr, *d_cross_sum = nullptr;
+  double *d_cross_y = nullptr, *d_cross_acc = nullptr, *d_cross_sum = nullptr, *d_cross_part = nullptr;
   int cross_nb = 0;
   int *d_selftest_err = nullptr;   // error word of the failure-path self-test
   unsigned long long fingerprint = 0;  // hash of the set-up inputs (ltmp2_fingerprint)
@@ -203,6 +206,97 @@ int upload_real_coeff(ltmp2_ctx *c, const ltmp2_system *sys, int row0, int rows,
   return cuda_status(cudaMemcpy(*dst, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
 }
 
+// ---------------------------------------------------------------- pairs' symmetry (sym.cuh)
+constexpr int kSymGroups = 304 + 2 * kMaxLevels;   // row groups of the direct term, at most
+
+// Row groups of the lower triangle, of about equal work, none across a level's boundary, and the
+// rows of each level (the rows are sorted by |G|^2, so a level is a prefix).
+int set_sym_rows(ltmp2_ctx *c, const std::vector<unsigned char> *lev) {
+  Plan &p = c->p;
+  if (!p.msym) return LTMP2_OK;
+  const int n = p.n_idx;
+  auto level = [&](int r) { return lev ? (int)(*lev)[c->sym_order[r]] : 1; };
+  for (int k = 0; k < kMaxLevels; ++k) {
+    int rows = 0;
+    while (rows < n && level(rows) >= k + 1) ++rows;
+    p.lev_rows[k] = rows;
+  }
+  const double total = 0.5 * n * (n + 1.0);
+  const double target = total / std::min(304.0, std::max(1.0, total / 1024.0));
+  std::vector<int2> g;
+  int first = 0;
+  double work = 0.0;
+  for (int r = 0; r < n; ++r) {
+    work += r + 1;
+    if (r + 1 == n || work >= target || level(r + 1) != level(r)) {
+      g.push_back(make_int2(first, r + 1));
+      first = r + 1;
+      work = 0.0;
+    }
+  }
+  if ((int)g.size() > kSymGroups) return LTMP2_ERR_INVALID_ARG;
+  p.n_groups = (int)g.size();
+  return cuda_status(cudaMemcpy(c->d_sym_groups, g.data(), g.size() * sizeof(int2), cudaMemcpyHostToDevice));
+}
+
+// Index set and matrices of the pairs' symmetry, where they take at most a quarter of the free
+// memory and their rows fit the column kernel's shared memory; else the energies go by slabs of G'.
+template <typename T>
+int setup_sym(ltmp2_ctx *c, const std::vector<int> &prim, const std::vector<int> &aux_neg) {
+  Plan &p = c->p;
+  const size_t cs = sizeof(CT<T>);
+  const int planes = p.real_orb ? 2 : 1, n = p.real_orb ? p.n_prim : 2 * p.n_prim, no = p.n_occ;
+  if (n < 1 || (size_t)planes * n * cs > 200 * 1024) return LTMP2_OK;
+  const size_t pair = (size_t)planes * n * n * cs;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return LTMP2_ERR_CUDA;
+  // orbitals per pass: a slab's columns, and at most 12 GB of pairs
+  int nj = std::min(no, std::max(1, p.max_prim * p.slots_per_prim() * no / n));
+  while (nj > 1 && (size_t)nj * no * pair > ((size_t)12 << 30)) --nj;
+  const size_t pairs = (size_t)nj * no - (size_t)nj * (nj - 1) / 2;
+  if ((pairs + no) * pair > free_b / 4) return LTMP2_OK;
+  std::vector<int> order(prim), pos(p.n_aux, -1);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return c->aux_g2[a] < c->aux_g2[b]; });
+  if (!p.real_orb) {
+    std::vector<int> both;
+    for (int g : order) {
+      both.push_back(g);
+      both.push_back(aux_neg[g]);
+    }
+    order.swap(both);
+  }
+  for (int r = 0; r < n; ++r) {
+    pos[order[r]] = r;
+    if (p.real_orb) pos[aux_neg[order[r]]] = n + r;   // second plane: S(-p, g')
+  }
+  int rc;
+  int *d_order = nullptr, *d_pos = nullptr;
+  void *m = nullptr, *md = nullptr;
+  double *rows = nullptr, *part = nullptr;
+  if ((rc = dalloc(c, &d_order, (size_t)n)) || (rc = dalloc(c, &d_pos, (size_t)p.n_aux)) ||
+      (rc = dalloc(c, &c->d_sym_groups, (size_t)kSymGroups)) || (rc = dalloc_bytes(c, &m, pairs * pair)) ||
+      (rc = dalloc_bytes(c, &md, (size_t)no * pair)) || (rc = dalloc(c, &rows, pairs * n)) ||
+      (rc = dalloc(c, &part, (size_t)kSymGroups * no * no)))
+    return rc == LTMP2_ERR_OOM ? LTMP2_OK : rc;
+  if ((rc = cuda_status(cudaMemcpy(d_order, order.data(), n * sizeof(int), cudaMemcpyHostToDevice))) ||
+      (rc = cuda_status(cudaMemcpy(d_pos, pos.data(), p.n_aux * sizeof(int), cudaMemcpyHostToDevice))))
+    return rc;
+  p.n_idx = n;
+  p.sym_planes = planes;
+  p.sym_order = d_order;
+  p.sym_pos = d_pos;
+  p.sym_groups = c->d_sym_groups;
+  p.sym_rows = rows;
+  p.sym_part = part;
+  p.sym_nj_cap = nj;
+  p.mdsym = md;
+  p.msym = m;
+  c->sym_order = order;
+  return set_sym_rows(c, nullptr);
+}
+// every G' at the Gamma point, by the Green's-function route
+bool use_sym(const Plan &p) { return p.msym && p.nk == 0 && p.route == 0; }
+
 // exact-slice tensor-core products of a context whose slabs have up to max_cols columns over nz
 // k points, and the virtuals by plane wave that they read (also the CUDA cores' virtual-space route)
 template <typename T> int setup_products(ltmp2_ctx *c, size_t max_cols, int nz, bool simt) {
@@ -238,7 +332,8 @@ template <typename T> int dalloc_exponents(ltmp2_ctx *c) {
   return dalloc(c, &p.uen3, (size_t)p.n_occ);
 }
 
-template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys, const std::vector<int> &order) {
+template <typename T>
+int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys, const std::vector<int> &order, const HostPlan &hp) {
   Plan &p = c->p;
   cudaError_t e = Path<T>::init_device();
   if (e != cudaSuccess) return cuda_status(e);
@@ -303,6 +398,7 @@ template <typename T> int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys,
     p.tc = &c->tc;
   }
   if ((rc = setup_products<T>(c, max_cols, 1, (sys->flags & LTMP2_FLAG_SIMT_GEMM) != 0))) return rc;
+  if ((rc = setup_sym<T>(c, hp.prim, hp.aux_neg))) return rc;
   e = Path<T>::setup_occupied(p, cocc, c->stream);
   if (e != cudaSuccess) return cuda_status(e);
   e = cudaStreamSynchronize(c->stream);
@@ -426,6 +522,10 @@ int enqueue_energy(ltmp2_ctx *c, cudaStream_t stream, int n_tau, const double *t
     if (e != cudaSuccess) return cuda_status(e);
     *launches += p.nk > 0 ? Path<T>::green_k_launches(p) : Path<T>::green_launches(p);
     const double coef = w[k] / (nk * nk * nk * p.omega * p.omega * nfft * nfft);
+    if (gp_begin == 0 && gp_end == p.n_prim && use_sym(p)) {
+      if ((e = Path<T>::sym_tau(p, coef, stream, tm, launches)) != cudaSuccess) return cuda_status(e);
+      continue;
+    }
     for (int g0 = gp_begin; g0 < gp_end; g0 += p.max_prim) {
       const int np = std::min(p.max_prim, gp_end - g0);
       e = p.nk > 0 ? Path<T>::slab_k(p, g0, np, coef, stream, tm) : Path<T>::slab(p, g0, np, coef, stream, tm);
@@ -835,6 +935,14 @@ int enqueue_uhf(ltmp2_ctx *a, ltmp2_ctx *b, int n_tau, const double *tau, const 
     if ((e = Path<T>::green(pb, tau[k], st, nullptr)) != cudaSuccess) return cuda_status(e);
     *launches += Path<T>::green_launches(pa) + Path<T>::green_launches(pb);
     const double coef = w[k] / (pa.omega * pa.omega * nfft * nfft);
+    if (a->d_cross_part && use_sym(pa) && use_sym(pb)) {
+      if ((e = Path<T>::sym_tau(pa, coef, st, nullptr, launches)) != cudaSuccess ||
+          (e = Path<T>::sym_tau(pb, coef, st, nullptr, launches)) != cudaSuccess ||
+          (e = Path<T>::sym_cross(pa, pb, coef, a->d_cross_part, a->d_cross_acc, st)) != cudaSuccess)
+        return cuda_status(e);
+      *launches += 2;
+      continue;
+    }
     for (int g0 = 0; g0 < pa.n_prim; g0 += pa.max_prim) {
       const int np = std::min(pa.max_prim, pa.n_prim - g0);
       // each channel: its exchange and same-spin direct sums, and its diagonal co-densities
@@ -914,7 +1022,9 @@ int ltmp2_setup(const ltmp2_system *sys, ltmp2_ctx **out) {
   if (!rc && p.real_basis) rc = up(&p.pw_pair, hp.pw_pair);   // internal position of -G_q
   if (!rc) rc = up(&p.aux_m, hp.aux_m);
   if (!rc) rc = up(&p.aux_neg, hp.aux_neg);
-  if (!rc) rc = up(&p.prim, hp.prim);
+  int *d_prim = nullptr;
+  if (!rc) rc = up(&d_prim, hp.prim);
+  p.prim = d_prim;
   if (!rc) rc = up(&p.v_aux64, hp.v64);
   if (!rc) rc = up(&p.v_aux32, hp.v32);
   if (!rc) rc = up(&p.eps, heps);
@@ -925,8 +1035,8 @@ int ltmp2_setup(const ltmp2_system *sys, ltmp2_ctx **out) {
   if (!rc) rc = dalloc(c, &p.edi, no2);
   if (!rc) rc = dalloc(c, &p.esum, 4);
   if (!rc)
-    rc = (sys->precision == LTMP2_FP64) ? setup_precision<double>(c, sys, order)
-                                        : setup_precision<float>(c, sys, order);
+    rc = (sys->precision == LTMP2_FP64) ? setup_precision<double>(c, sys, order, hp)
+                                        : setup_precision<float>(c, sys, order, hp);
   if (rc) {
     cudaGetLastError();
     return rc;
@@ -1157,6 +1267,7 @@ int ltmp2_set_pair_mask(ltmp2_ctx *ctx, const unsigned char *keep) {
     p.pair_keep = nullptr;
     p.keep_list = nullptr;
     p.keep_count = nullptr;
+    p.keep_upto = nullptr;
     ctx->mask_hash = 0;
     return LTMP2_OK;
   }
@@ -1171,14 +1282,17 @@ int ltmp2_set_pair_mask(ltmp2_ctx *ctx, const unsigned char *keep) {
   if (!ctx->d_keep) {
     if ((rc = dalloc(ctx, &ctx->d_keep, (size_t)no * no))) return rc;
     if ((rc = dalloc(ctx, &ctx->d_keep_list, (size_t)no * no))) return rc;
-    if ((rc = dalloc(ctx, &ctx->d_keep_count, (size_t)no))) return rc;
+    if ((rc = dalloc(ctx, &ctx->d_keep_count, 2 * (size_t)no))) return rc;
   }
   std::vector<unsigned char> k01((size_t)no * no);
-  std::vector<int> list((size_t)no * no, 0), count(no, 0);
+  std::vector<int> list((size_t)no * no, 0), count(2 * (size_t)no, 0);   // kept i, and kept i <= j
   for (int j = 0; j < no; ++j)
     for (int i = 0; i < no; ++i) {
       k01[(size_t)i * no + j] = keep[(size_t)i * no + j] ? 1 : 0;
-      if (keep[(size_t)i * no + j]) list[(size_t)j * no + count[j]++] = i;
+      if (keep[(size_t)i * no + j]) {
+        list[(size_t)j * no + count[j]++] = i;
+        if (i <= j) ++count[no + j];
+      }
     }
   if (cudaMemcpy(ctx->d_keep, k01.data(), k01.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->d_keep_list, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -1187,6 +1301,7 @@ int ltmp2_set_pair_mask(ltmp2_ctx *ctx, const unsigned char *keep) {
   p.pair_keep = ctx->d_keep;
   p.keep_list = ctx->d_keep_list;
   p.keep_count = ctx->d_keep_count;
+  p.keep_upto = ctx->d_keep_count + no;
   // the mask changes the exchange energy, so it enters the fingerprint
   unsigned long long h = 0xcbf29ce484222325ull;
   for (unsigned char b : k01) h = (h ^ b) * 0x100000001b3ull;
@@ -1427,6 +1542,8 @@ int ltmp2_energy_uhf(ltmp2_ctx *alpha, ltmp2_ctx *beta, int n_tau, const double 
     if ((rc = dalloc(alpha, &alpha->d_cross_y, (size_t)alpha->slab_capacity * nab))) return rc;
     if ((rc = dalloc(alpha, &alpha->d_cross_acc, nab))) return rc;
     if ((rc = dalloc(alpha, &alpha->d_cross_sum, 1))) return rc;
+    alpha->d_cross_part = nullptr;
+    if (use_sym(pa) && use_sym(pb) && (rc = dalloc(alpha, &alpha->d_cross_part, (size_t)kSymGroups * nab))) return rc;
     alpha->cross_nb = pb.n_occ;
   }
   pa.max_prim = pb.max_prim = slab;
@@ -1509,6 +1626,10 @@ int ltmp2_set_extrapolation(ltmp2_ctx *ctx, int n_c, double alpha) {
   Plan &p = ctx->p;
   ctx->lev_done = false;
   if (n_c <= 1) {
+    DeviceGuard g(ctx->device);
+    if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return LTMP2_ERR_CUDA;
+    const int rc = set_sym_rows(ctx, nullptr);
+    if (rc) return rc;
     p.n_lev = 0;
     ctx->lev_ecut.clear();
     ctx->lev_count.clear();
@@ -1566,6 +1687,7 @@ int ltmp2_set_extrapolation(ltmp2_ctx *ctx, int n_c, double alpha) {
   if (e == cudaSuccess)
     e = cudaMemcpy((void *)p.lev_start, start.data(), (n_c + 1) * sizeof(int), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_status(e);
+  if ((rc = set_sym_rows(ctx, &lev))) return rc;
   p.n_lev = n_c;
   ctx->lev_ecut = ecut;
   ctx->lev_count = count;

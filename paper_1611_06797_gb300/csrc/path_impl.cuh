@@ -1,11 +1,13 @@
 // Launchers of the hot path for one real type T.  Included once per precision by
 // kernels_f64.cu / kernels_f32.cu, which explicitly instantiate Path<T>.
 #pragma once
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
 #include "kernels.cuh"
 #include "sized.h"
+#include "sym.cuh"
 
 namespace ltmp2 {
 
@@ -218,15 +220,15 @@ cudaError_t Path<T>::green(const Plan &p, double tau, cudaStream_t st, StageTime
 template <typename T>
 cudaError_t Path<T>::slab_pre(const Plan &p, int gp0, int np, cudaStream_t st, StageTimer *tm) {
   const int n = p.n, no = p.n_occ;
-  const int nslots = np * p.slots_per_prim();
-  const int ncols = nslots * no;
+  const bool sym = p.sym_nj > 0;   // the columns of the pass's orbitals, without the occupied factors
+  const int ncols = sym ? np * p.sym_nj : np * p.slots_per_prim() * no;
   cudaError_t e;
   if (p.route != 1) {
     ScopedStage s(tm, kStageGatherZ);
     if (p.real_basis)
-      k_gather_s_real<T><<<dim3((p.n_pw + 255) / 256, ncols), 256, 0, st>>>(p, gp0, np, (cpx<T> *)p.st);
+      k_gather_s_real<T><<<dim3((p.n_pw + 255) / 256, ncols), 256, 0, st>>>(p, gp0, np, (cpx<T> *)p.st, sym);
     else
-      k_gather_s<T><<<dim3((p.n_pw + 255) / 256, ncols), 256, 0, st>>>(p, gp0, np, (cpx<T> *)p.st);
+      k_gather_s<T><<<dim3((p.n_pw + 255) / 256, ncols), 256, 0, st>>>(p, gp0, np, (cpx<T> *)p.st, sym);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   {
@@ -374,6 +376,69 @@ cudaError_t Path<T>::slab_post(const Plan &p, int gp0, int np, double coef, cuda
     }
   }
   return cudaSuccess;
+}
+
+// pair slots of a pass over sym_nj orbitals from sym_j0
+static int sym_pairs(const Plan &p) { return p.sym_nj * p.sym_j0 + p.sym_nj * (p.sym_nj + 1) / 2; }
+
+template <typename T>
+cudaError_t Path<T>::sym_tau(const Plan &p0, double coef, cudaStream_t st, StageTimer *tm, long long *launches) {
+  Plan p = p0;
+  p.prim = p.sym_order;   // the slots of a pass: every G' of the index set, in its order
+  const int n_idx = p.n_idx, no = p.n_occ;
+  // columns per pass as of a slab; whole orbitals j if they fit, else one j in several parts
+  const int budget = p.max_prim * p.slots_per_prim() * no;
+  const int nj = std::max(1, std::min(std::min(budget / n_idx, no), p.sym_nj_cap));
+  const int np_max = std::max(1, std::min(n_idx, budget / nj));
+  const size_t smem = (size_t)p.sym_planes * n_idx * sizeof(cpx<T>);
+  const int threads = std::min(256, ((p.n_daux + 31) / 32) * 32);
+  cudaError_t e;
+  for (p.sym_j0 = 0; p.sym_j0 < no; p.sym_j0 += nj) {
+    p.sym_nj = std::min(nj, no - p.sym_j0);
+    for (int g0 = 0; g0 < n_idx; g0 += np_max) {
+      const int np = std::min(np_max, n_idx - g0), ncols = np * p.sym_nj;
+      if ((e = slab_pre(p, g0, np, st, tm)) != cudaSuccess) return e;
+      {
+        ScopedStage s(tm, kStagePlane);
+        if ((e = launch_planes<T>(p, ncols, p.plane_kernel, p.plane_ib, st)) != cudaSuccess) return e;
+      }
+      {
+        ScopedStage s(tm, kStageColumn);
+        if (!with_size(p.n, [&](auto c) { Sized<T, decltype(c)::value>::zsym(p, g0, ncols, threads, smem, st); }))
+          return cudaErrorInvalidValue;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      }
+      *launches += pre_launches(p) + 2;
+    }
+    ScopedStage s(tm, kStageColumn);
+    const int pairs = sym_pairs(p);
+    k_xsym<T><<<dim3(pairs, (n_idx + 31) / 32), 256, 0, st>>>(p, p.sym_rows);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // real orbitals: the rows are the primary G', each standing for -G' too
+    k_xsym_sum<T><<<pairs, 128, 0, st>>>(p, p.sym_rows, (p.real_orb ? 2.0 : 1.0) * coef);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    *launches += 2;
+  }
+  {
+    ScopedStage s(tm, kStageDirect);
+    const int t = (no + 3) / 4;
+    k_dsym<T><<<dim3(p.n_groups, t * (t + 1) / 2), 256, 0, st>>>(p, p, true, p.sym_part);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_dsym_sum<T><<<(no * no + 3) / 4, 128, 0, st>>>(p, p, true, p.sym_part, (p.real_orb ? -4.0 : -2.0) * coef, p.ed,
+                                                     p.edl);
+    *launches += 2;
+  }
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t Path<T>::sym_cross(const Plan &pa, const Plan &pb, double coef, double *part, double *acc, cudaStream_t st) {
+  k_dsym<T><<<dim3(pa.n_groups, ((pa.n_occ + 3) / 4) * ((pb.n_occ + 3) / 4)), 256, 0, st>>>(pa, pb, false, part);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_dsym_sum<T><<<(pa.n_occ * pb.n_occ + 3) / 4, 128, 0, st>>>(pa, pb, false, part, (pa.real_orb ? -2.0 : -1.0) * coef, acc,
+                                                               nullptr);
+  return cudaGetLastError();
 }
 
 template <typename T> cudaError_t Path<T>::green_k(const Plan &p, double tau, cudaStream_t st, StageTimer *tm) {

@@ -80,7 +80,7 @@ struct Plan {
   int *pw_pair = nullptr;    // [n_pw] internal position of -G_q (real basis only)
   int *aux_m = nullptr;      // [n_aux * 3]
   int *aux_neg = nullptr;    // [n_aux] position of -G in A
-  int *prim = nullptr;       // [n_prim] position in A of each primary G'
+  const int *prim = nullptr; // [n_prim] position in A of each primary G'
   double *v_aux64 = nullptr; // [n_aux] 4 pi / |G|^2
   float *v_aux32 = nullptr;
   double *eps = nullptr;     // [n_orb] (device)
@@ -119,6 +119,7 @@ struct Plan {
   const unsigned char *pair_keep = nullptr;  // [n_occ][n_occ] 1 = contract, symmetric, diagonal kept
   const int *keep_list = nullptr;            // [n_occ][n_occ] kept i for each j (first keep_count[j])
   const int *keep_count = nullptr;           // [n_occ]
+  const int *keep_upto = nullptr;            // [n_occ] kept i <= j (the lists ascend)
   int plane_ib = 0;          // occupied planes per plane-kernel block, 0 = kernel default
   // internal auxiliary-cutoff extrapolation (Sec. III D): nested spheres A_1 = A, ...,
   // A_n = {G : |G|^2/2 <= E_aux / alpha^(n-1)}; every G- and G'-sum is also kept per level.
@@ -147,6 +148,17 @@ struct Plan {
   bool w_virtual = false;
   void *rvt = nullptr;
   void *cvt = nullptr;       // general orbitals: the virtual coefficients by plane wave, cpx<T> [nk or 1][n_pw][n_v]
+  // Whole energies by the pairs' exchange symmetry (sym.cuh); msym null: not set up
+  int n_idx = 0, sym_planes = 0;       // index set, planes (2: real orbitals, 1: general)
+  const int *sym_order = nullptr;      // [n_idx] aux positions by |G|^2 (general: G and -G side by side)
+  const int *sym_pos = nullptr;        // [n_aux] plane n_idx + index, or -1 (G = 0)
+  void *msym = nullptr, *mdsym = nullptr;   // S_ij of a pass's pairs i < j, S_jj of every j: [planes][n_idx g'][n_idx p]
+  double *sym_rows = nullptr, *sym_part = nullptr;   // exchange sums per pair and row, direct sums per row group
+  const int2 *sym_groups = nullptr;    // [n_groups] row ranges, none across a level's boundary
+  int n_groups = 0;
+  int sym_nj_cap = 0;                  // orbitals j per pass that msym holds
+  int lev_rows[16] = {0};              // level n: rows in A_{n+1}
+  int sym_nj = 0, sym_j0 = 0;          // during a pass: columns (slot, j) of sym_nj orbitals j >= sym_j0, items i <= j
   // k-point sampling (Sec. II C-D), nk > 0: n_occ counts composite occupied orbitals
   // k n_o + i over the mesh, n_orb / n_v are per k, cv [nk][n_v][n_pw], pt [nk][n_pw][n_pw],
   // dscale [nk][n_orb]; the auxiliary set A (daux, aux_m) is the ball that holds every
@@ -233,12 +245,16 @@ template <typename T> struct Path {
     if (p.route == 1 || p.w_virtual) return 1;
     return p.oz || (p.tc && p.tc->green_on()) ? 4 : 2;   // dscale, split, product, split of the result
   }
-  static int slab_launches(const Plan &p) {
-    if (p.route == 1) return 7 + (p.precision == 0 ? 1 : 0) + (p.n_lev > 1 ? 1 : 0);   // no gather, CUDA-core product
+  // gather, product, map from the real basis, norms (FP64), z transform
+  static int pre_launches(const Plan &p) {
     // W: one product, on the tensor cores after a split; twice that through the virtual space
     const int w = (p.w_virtual ? 2 : 1) * (p.oz ? 2 : 1);
-    return 6 + (p.precision == 0 ? 1 : 0) + w + (p.real_basis ? 1 : 0) + (p.n_lev > 1 ? 1 : 0) +
-           (p.tc && p.tc->direct_on() && p.n_lev < 2 ? 2 : 0);   // direct term: pack, product, combine
+    return 2 + w + (p.real_basis ? 1 : 0) + (p.precision == 0 ? 1 : 0);
+  }
+  static int slab_launches(const Plan &p) {
+    const int tail = 4 + (p.n_lev > 1 ? 1 : 0);   // plane, column, direct, accumulate (and the levels')
+    if (p.route == 1) return 3 + (p.precision == 0 ? 1 : 0) + tail;   // no gather, CUDA-core product
+    return pre_launches(p) + tail + (p.tc && p.tc->direct_on() && p.n_lev < 2 ? 2 : 0);   // direct term: pack, product, combine
   }
   // setup: cv [nk or 1][n_v][n_pw] by plane wave, [nk or 1][n_pw][n_v]
   static cudaError_t transpose_virtuals(const Plan &p, void *out, cudaStream_t st);
@@ -255,6 +271,10 @@ template <typename T> struct Path {
   // one slab of primary G' [gp0, gp0 + np): everything up to the pair sums, then accumulate
   static cudaError_t slab(const Plan &p, int gp0, int np, double coef, cudaStream_t st,
                           StageTimer *tm);
+  // one tau of a whole energy by the pairs' symmetry: every G', exchange and direct sums
+  static cudaError_t sym_tau(const Plan &p, double coef, cudaStream_t st, StageTimer *tm, long long *launches);
+  // opposite-spin direct term of a tau from the channels' S_jj: acc [na][nb] accumulated (part: scratch)
+  static cudaError_t sym_cross(const Plan &pa, const Plan &pb, double coef, double *part, double *acc, cudaStream_t st);
   // the slab in phases: up to w in real space (gather, transformed-state GEMM, z transform),
   // and after the co-density FFTs (direct term, accumulation); the batching form runs the
   // FFT stages of every system in between as shared persistent launches

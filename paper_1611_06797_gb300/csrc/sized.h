@@ -19,6 +19,7 @@ template <typename T, int N> struct Sized {
   static void planes_store(const Plan &p, const void *z1, cudaStream_t st);
   static void planes(const Plan &p, int cols, int kernel, int ib, int threads, size_t smem, cudaStream_t st);
   static void zcol(const Plan &p, int gp0, int np, int npairs, int threads, size_t smem, bool lev, cudaStream_t st);
+  static void zsym(const Plan &p, int gp0, int cols, int threads, size_t smem, cudaStream_t st);
   static void zcol_k(const Plan &p, int gp0, int np, int npairs, int threads, size_t smem, cudaStream_t st);
 };
 

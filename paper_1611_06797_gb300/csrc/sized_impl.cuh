@@ -2,6 +2,7 @@
 #pragma once
 #include "kernels.cuh"
 #include "sized.h"
+#include "sym.cuh"
 
 namespace ltmp2 {
 
@@ -19,6 +20,7 @@ template <typename T, int N> cudaError_t Sized<T, N>::init() {
   limit(k_zcol<T, N, false>);
   limit(k_zcol<T, N, true>);
   limit(k_zcol_k<T, N>);
+  limit(k_zsym<T, N>);
   return e;
 }
 
@@ -48,6 +50,11 @@ template <typename T, int N>
 void Sized<T, N>::zcol(const Plan &p, int gp0, int np, int npairs, int threads, size_t smem, bool lev, cudaStream_t st) {
   if (lev) k_zcol<T, N, true><<<npairs, threads, smem, st>>>(p, gp0, np, p.tbuf, (cpx<T> *)p.mdiag, p.sx);
   else k_zcol<T, N, false><<<npairs, threads, smem, st>>>(p, gp0, np, p.tbuf, (cpx<T> *)p.mdiag, p.sx);
+}
+
+template <typename T, int N>
+void Sized<T, N>::zsym(const Plan &p, int gp0, int cols, int threads, size_t smem, cudaStream_t st) {
+  k_zsym<T, N><<<dim3(p.sym_j0 + p.sym_nj, cols), threads, smem, st>>>(p, gp0);
 }
 
 template <typename T, int N>
