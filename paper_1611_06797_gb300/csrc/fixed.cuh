@@ -73,15 +73,18 @@ template <long long C> __host__ __device__ __forceinline__ long long fx_mulc(lon
     return p + p + (t >> 31);
   }
 }
-// a * b * 2^-62 for |a| <= 2^62, |b| <= 2^61; of the low x low product only the upper 16 x 16 bits
-__host__ __device__ __forceinline__ long long fx_mul62(long long a, long long b) {
-  const int ah = (int)(a >> 32), bh = (int)(b >> 32);
-  const unsigned al = (unsigned)a, bl = (unsigned)b;
-  const long long t = (long long)ah * (long long)(unsigned long long)bl +
-                      (long long)bh * (long long)(unsigned long long)al +
-                      ((long long)((al >> 16) * (bl >> 16)) + (1ll << 29));
-  const long long p = (long long)ah * bh;
-  return (p << 2) + (t >> 30);
+// A fixed-point value v, |v| <= 2^61, as v = hi 2^31 + lo with lo in [-2^30, 2^30): both halves are
+// signed, so a product of two split values is three signed 32 x 32 -> 64 bit products.
+struct alignas(8) fx2 { int lo, hi; };
+__host__ __device__ __forceinline__ fx2 fx_split(long long v) {
+  const int hi = (int)((v + (1ll << 30)) >> 31);
+  return {(int)(v - ((long long)hi << 31)), hi};
+}
+// a * b * 2^-61, rounded; the product of the low halves is dropped (at most half a unit, mean zero)
+__host__ __device__ __forceinline__ long long fx_mul61(fx2 a, fx2 b) {
+  const long long t = (long long)a.hi * b.lo + ((long long)a.lo * b.hi + (1ll << 29));
+  const long long q = (long long)a.hi * b.hi;
+  return q + q + (t >> 30);
 }
 // x / 2^s rounded to nearest, 0 <= s < 63
 __host__ __device__ __forceinline__ long long fx_shr(long long x, int s) {

@@ -668,13 +668,18 @@ __device__ __forceinline__ double block_sum(double v) {
   return s;
 }
 
+struct alignas(16) cpx2 { fx2 x, y; };   // complex, both parts split
 // FP64 form of planes3_body on 64-bit fixed point (fixed.cuh).  The FP64 pipe bound the same
 // passes in double (85 % of its issue rate); a launch of 3488 columns of 32 occupied on 24^3 took
-// 62.3 ms in double and takes 11.5 ms on integers (with the column kernel, 14.1 -> 4.2 ms).
+// 62.3 ms in double, 11.5 ms on integers with a full 64 x 64 bit product, and takes 9.8 ms with
+// split halves and one copy of the transform (the column kernel: 14.1 -> 4.2 ms).  Now bound by the
+// issue of its 2,500 instructions a plane (half of the issue slots) at three warps per scheduler,
+// which its registers (4 per point and thread) allow.
 //  w plane: scaled by 2^(61 - e), 2^e > ||w||_2 of the plane (n ||z1||_2 by Parseval), inverse
 //           transformed in fixed point; every partial sum of the transform is at most
 //           sum |z1| <= sqrt(n_dorb) ||z1||_2 < ||w||_2;
-//  x pass : phi_i comes as phi 2^(62 - uen), 2^uen > ||phi_i||_2 of the plane, so the product
+//  x pass : phi_i comes as phi 2^(61 - uen), 2^uen > ||phi_i||_2 of the plane, and phi and w as
+//           two signed halves (fx_split), which makes their product three IMAD.WIDE; the product
 //           is conj(phi_i) w 2^(61 - uen - e), and every partial sum of its forward transform
 //           is at most ||phi_i||_2 ||w||_2 (Cauchy-Schwarz): below 2^61;
 //  y pass, copy: as in planes3_body; the copy shifts to the item's scale 2^(61 - uen3 - wen3), from
@@ -716,71 +721,81 @@ __device__ __forceinline__ void planes3_body_fx(const Plan &p, int ib, int z, in
   }
   __syncthreads();
   const int nxo = p.mxhi_orb - p.mxlo_orb + 1;
-  for (int t = tid; t < nxo; t += nth) {
-    const int x = wrapn(p.mxlo_orb + t, N);
-    cpx<W> a[N];
-#pragma unroll
-    for (int k = 0; k < N; ++k) a[k] = xp[k * P + x];
-    LineFFT<W, N, +1>::run(a);
-#pragma unroll
-    for (int k = 0; k < N; ++k) xp[k * P + x] = a[k];
-  }
-  __syncthreads();
-  for (int t = tid; t < N; t += nth) {
-    cpx<W> a[N];
-#pragma unroll
-    for (int k = 0; k < N; ++k) a[k] = xp[t * P + k];
-    LineFFT<W, N, +1>::run(a);
-#pragma unroll
-    for (int k = 0; k < N; ++k) xp[t * P + k] = a[k];
-  }
-  __syncthreads();
-  const cpx<W> *ut = (const cpx<W> *)p.ut;
-  const W *utr = (const W *)p.utr;
+  const cpx2 *ut = (const cpx2 *)p.ut;
+  const fx2 *utr = (const fx2 *)p.utr;
   const int jcol = col_orbital(p, col), ni = col_items(p, jcol);
   const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
   const int esh = p.wen3[col] - ew;   // >= 0 (a sentinel for a state that is not finite)
-  for (int i0 = 0; i0 < ni; i0 += ib) {
-    const int nb = min(ib, ni - i0);
-    for (int t = tid; t < nb * N; t += nth) {
-      const int il = t / N, y = t - il * N;
-      const int iocc = ilist ? ilist[i0 + il] : i0 + il;
+  // Passes: 0 inverse y, 1 inverse x (w, then split), then 2 product and forward x, 3 forward y of each
+  // block of ib occupied.  One copy of the line transform serves them all (an inverse transform is
+  // the forward one between two swaps of real and imaginary parts): with a copy per pass the code
+  // outgrew the instruction caches (one issue in six waited for an instruction).
+  const int npass = 2 + 2 * ((ni + ib - 1) / ib);
+  for (int pass = 0; pass < npass; ++pass) {
+    const int mode = pass < 2 ? pass : 2 + (pass & 1);
+    const int i0 = ((pass - 2) >> 1) * ib, nb = min(ib, ni - i0);
+    const int count = mode == 0 ? nxo : mode == 1 ? N : mode == 2 ? nb * N : nb * nxa;
+    for (int t = tid; t < count; t += nth) {
       cpx<W> a[N];
-      const size_t urow = ((size_t)iocc * N + z) * N * N + y;
-      const cpx<W> *wr = xp + y * P;
-      if (utr) {
+      // the line in shared memory: modes 0, 1, 3 in place, mode 2's output row
+      cpx<W> *line;
+      int stride;
+      if (mode == 2) {
+        const int il = t / N, y = t - il * N;
+        const int iocc = ilist ? ilist[i0 + il] : i0 + il;
+        // row y of phi_i from the transposed plane: element x at x N + y, so the threads of a warp
+        // read consecutive addresses.  Real orbitals: two real products per point.
+        const size_t urow = ((size_t)iocc * N + z) * N * N + y;
+        const cpx2 *wr = reinterpret_cast<const cpx2 *>(xp + y * P);
+        if (utr) {
 #pragma unroll
-        for (int k = 0; k < N; ++k) {
-          const W u = utr[urow + k * N];
-          a[k] = {fx_mul62(u, wr[k].x), fx_mul62(u, wr[k].y)};
+          for (int k = 0; k < N; ++k) {
+            const fx2 u = utr[urow + k * N];
+            const cpx2 w = wr[k];
+            a[k] = {fx_mul61(u, w.x), fx_mul61(u, w.y)};
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < N; ++k) {
+            const cpx2 u = ut[urow + k * N], w = wr[k];
+            a[k] = {fx_mul61(u.x, w.x) + fx_mul61(u.y, w.y), fx_mul61(u.x, w.y) - fx_mul61(u.y, w.x)};
+          }
         }
+        line = wk + (size_t)il * Q + y * nxa - mlo;   // line[m] for m in [mlo, mhi]
+        stride = 1;
       } else {
+        if (mode == 3) {
+          const int il = (int)(((unsigned)t * inv_nxa) >> 20);   // t / nxa, exact for t < 2^12
+          line = wk + (size_t)il * Q + (t - il * nxa);
+          stride = nxa;
+        } else {
+          line = mode == 0 ? xp + wrapn(p.mxlo_orb + t, N) : xp + t * P;
+          stride = mode == 0 ? P : 1;
+        }
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-          const cpx<W> u = ut[urow + k * N], w = wr[k];
-          a[k] = {fx_mul62(u.x, w.x) + fx_mul62(u.y, w.y), fx_mul62(u.x, w.y) - fx_mul62(u.y, w.x)};
+          const cpx<W> v = line[k * stride];
+          a[k] = mode == 3 ? v : cpx<W>{v.y, v.x};
         }
       }
       LineFFT<W, N, -1>::run(a);
-      cpx<W> *row = wk + (size_t)il * Q + y * nxa - mlo;   // row[m] for m in [mlo, mhi]
+      if (mode == 2) {
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
-        const int m = freq_of<N>(k);
-        if (m >= mlo && m <= mhi) row[m] = a[k];
+        for (int k = 0; k < N; ++k) {
+          const int m = freq_of<N>(k);
+          if (m >= mlo && m <= mhi) line[m] = a[k];
+        }
+      } else if (mode == 1) {
+        cpx2 *row = reinterpret_cast<cpx2 *>(line);   // w split in place
+#pragma unroll
+        for (int k = 0; k < N; ++k) row[k] = {fx_split(a[k].y), fx_split(a[k].x)};
+      } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) line[k * stride] = mode == 3 ? a[k] : cpx<W>{a[k].y, a[k].x};
       }
     }
     __syncthreads();
-    for (int t = tid; t < nb * nxa; t += nth) {
-      const int il = (int)(((unsigned)t * inv_nxa) >> 20), xa = t - il * nxa;   // t / nxa, exact for t < 2^12
-      cpx<W> *src = wk + (size_t)il * Q + xa;
-      cpx<W> b[N];
-#pragma unroll
-      for (int k = 0; k < N; ++k) b[k] = src[k * nxa];
-      LineFFT<W, N, -1>::run(b);
-#pragma unroll
-      for (int k = 0; k < N; ++k) src[k * nxa] = b[k];
-    }
-    __syncthreads();
+    if (mode != 3) continue;
     for (int il = 0; il < nb; ++il) {
       const int iocc = ilist ? ilist[i0 + il] : i0 + il;
       const size_t item = item_of(p, col, iocc);
@@ -905,7 +920,7 @@ __global__ void __launch_bounds__(32 * kPlaneWarps) k_planes4(Plan p, int ib, co
 // setup: real-space occupied orbitals u[j][z][y][x] from z1 (cols = occupied orbitals)
 // (and the plane-transposed copy outt[j][z][x][y] that the plane kernel reads row-wise).
 // FP64: the transposed copy (outr's real part where it is given, else outt) is fixed point,
-// phi 2^(62 - uen[j][z]), and un2[j][z] keeps the plane's square norm.
+// phi 2^(61 - uen[j][z]) in split form, and un2[j][z] keeps the plane's square norm.
 template <typename T, int N>
 __global__ void k_planes_store(Plan p, const cpx<T> *__restrict__ z1, cpx<T> *__restrict__ out,
                                void *__restrict__ outt, void *__restrict__ outr) {
@@ -928,13 +943,14 @@ __global__ void k_planes_store(Plan p, const cpx<T> *__restrict__ z1, cpx<T> *__
       p.un2[col * N + z] = s2;
     }
     if (eu == kFxNotFinite) eu = 0;
-    const double f = fx_pow2(kFxBits + 1 - eu);
+    const double f = fx_pow2(kFxBits - eu);
     for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
       const int y = e / N, x = e % N;
       if (out) out[base + e] = xp[y * P + x];
       const cpx<double> v = xp[x * P + y];   // e = x' N + y' with x' = y, y' = x
-      if (outr) ((long long *)outr)[base + e] = __double2ll_rn(v.x * f);
-      else ((cpx<long long> *)outt)[base + e] = {__double2ll_rn(v.x * f), __double2ll_rn(v.y * f)};
+      const fx2 re = fx_split(__double2ll_rn(v.x * f));
+      if (outr) ((fx2 *)outr)[base + e] = re;
+      else ((cpx2 *)outt)[base + e] = {re, fx_split(__double2ll_rn(v.y * f))};
     }
   } else {
     for (int e = threadIdx.x; e < N * N; e += blockDim.x) {

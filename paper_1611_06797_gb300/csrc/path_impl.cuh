@@ -46,6 +46,14 @@ template <typename T> static int plane_ib_default(const Plan &p, int kernel) {
   } else if (kernel == 0) {
     ib = (int)((96 * 1024) / plane) - 1;   // about 96 KB of shared memory
     if (ib > 8) ib = 8;
+  } else if (kernel == 2 && std::is_same<T, double>::value) {
+    // fixed point: blocks of two warps whose lanes the n ib lines of the x pass fill, or of three
+    // where they fill those better by 15 % (two warps keep more blocks resident).  One Laplace point's
+    // plane pass: 20^3 with 3 of 4 planes 9.9 against 11.8 ms, 18^3 4.2 against 4.9, 27^3 with 2 of 4
+    // 19.8 against 21.9, 32^3 18.5 against 20.2; 24^3 with 4 (three warps) 9.8 against 11.5 with 2
+    const int two = 64 / n, three = 96 / n;
+    ib = two > 0 && 1.15 * two * n / 64.0 >= three * n / 96.0 ? two : three;
+    while (ib > 1 && plane + (sizeof(int) * p.n_daux + 64) + (size_t)ib * plane_stride(n, nxa) * sizeof(cpx<T>) > 100 * 1024) --ib;
   } else if (kernel == 2) {
     // four planes per block: small blocks, many resident per SM (best on the 24^3 workload
     // in both precisions among 2..16)

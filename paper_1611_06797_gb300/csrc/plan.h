@@ -94,7 +94,7 @@ struct Plan {
                              // (the orbitals are real in real space), else null
   // FP64: exponents of the fixed-point co-densities (fixed.cuh): 2^uen bounds the 2-norm of
   // plane z of orbital i, 2^uen3 that of the orbital, 2^wen3 that of a transformed state; ut (or utr
-  // where the orbitals are real) holds phi 2^(62 - uen) as integers
+  // where the orbitals are real) holds phi 2^(61 - uen) as split integers
   int *uen = nullptr;        // [n_occ][n]
   int *uen3 = nullptr;       // [n_occ]
   int *wen3 = nullptr;       // [max_cols]

@@ -67,21 +67,24 @@ int main() {
       tw = std::fmax(tw, (double)std::fabs((long double)fxc::sinn(e, n) / 4611686018427387904.0L - std::sin(t)));
     }
   std::printf("const 0 %.3e\n", tw);
-  double mean = 0, worst = 0;
+  // products: |x|, |y| <= 2^61 of every magnitude, and the ends of the range
+  double mean = 0, worst = 0, back = 0;
   const int n = 200000;
+  auto err = [&](long long x, long long y) {
+    const fx2 a = fx_split(x), b = fx_split(y);
+    back = std::fmax(back, std::fabs((double)(((__int128)a.hi << 31) + a.lo - x)));
+    return (double)(((__int128)fx_mul61(a, b) << 61) - (__int128)x * y) / 2305843009213693952.0;
+  };
   for (int i = 0; i < n; ++i) {
     const int sa = (int)(next() % 40), sb = (int)(next() % 40);
-    const long long x = ((long long)next() >> 1) >> sa, y = ((long long)next() >> 2) >> sb;   // |x| <= 2^62, |y| <= 2^61
-    const double d = (double)(((__int128)fx_mul62(x, y) << 62) - (__int128)x * y) / 4611686018427387904.0;
+    const double d = err(((long long)next() >> 2) >> sa, ((long long)next() >> 2) >> sb);
     mean += d / n;
     worst = std::fmax(worst, std::fabs(d));
   }
-  const long long top = 1ll << 62, half = 1ll << 61;
-  for (long long x : {top, -top, top - 1, 0ll})
-    for (long long y : {half, -half, half - 1, 0ll}) {
-      const double d = (double)(((__int128)fx_mul62(x, y) << 62) - (__int128)x * y) / 4611686018427387904.0;
-      worst = std::fmax(worst, std::fabs(d));
-    }
-  std::printf("mul %.4f %.4f\n", mean, worst);
+  const long long top = 1ll << 61;
+  for (long long x : {top, -top, top - 1, 0ll, (1ll << 30) - 1, 1ll << 30, -(1ll << 30)})
+    for (long long y : {top, -top, top - 1, 0ll, (1ll << 30) - 1, 1ll << 30, -(1ll << 30)})
+      worst = std::fmax(worst, std::fabs(err(x, y)));
+  std::printf("mul %.4f %.4f %.1f\n", mean, worst, back);
   return 0;
 }
