@@ -1161,9 +1161,11 @@ __global__ void __launch_bounds__(256) k_zcol(Plan p, int gp0, int np, const voi
 }
 
 // ---------------------------------------------------------------- direct term
-// Y_ij(G') = sum_G v(G) M_ii(G;G') M_jj(-G;-G')  (general)  or  M_ii(G;G') conj(M_jj(G;G')) (real)
-template <typename T, bool LEV>
-__global__ void k_direct(Plan p, int np, const cpx<T> *__restrict__ mdiag, double2 *__restrict__ yd) {
+// Y_ij(G') = sum_G v(G) M_ii(G;G') M_jj(-G;-G')  (general)  or  M_ii(G;G') conj(M_jj(G;G')) (real),
+// on every nested sphere: groups from the innermost level outwards, so that the running sum is the
+// sum over A_n
+template <typename T>
+__global__ void k_direct_lev(Plan p, int np, const cpx<T> *__restrict__ mdiag, double2 *__restrict__ yd) {
   const int gpl = blockIdx.x, i = blockIdx.y;
   const int no = p.n_occ;
   const int slotA = gpl, slotB = p.real_orb ? gpl : gpl + np;
@@ -1171,41 +1173,150 @@ __global__ void k_direct(Plan p, int np, const cpx<T> *__restrict__ mdiag, doubl
   const cpx<T> *MA = mdiag + (size_t)slotA * p.n_aux * no;
   const cpx<T> *MB = mdiag + (size_t)slotB * p.n_aux * no;
   for (int j = threadIdx.x; j < no; j += blockDim.x) {
-    if constexpr (LEV) {
-      // groups from the innermost level outwards; the running sum is the sum over A_n
-      double ax = 0, ay = 0;
-      for (int n = p.n_lev - 1; n >= 0; --n) {
-        T cx = T(0), cy = T(0);
-        int cnt = 0;
-        for (int k = p.lev_start[n]; k < p.lev_start[n + 1]; ++k) {
-          const int g = p.lev_order[k];
-          const cpx<T> x = MA[(size_t)g * no + i];
-          cpx<T> prod;
-          if (!p.real_orb) prod = cmul(x, MB[(size_t)p.aux_neg[g] * no + j]);
-          else prod = cmulconj(x, MB[(size_t)g * no + j]);
-          cx += v[g] * prod.x;
-          cy += v[g] * prod.y;
-          if ((++cnt & 31) == 0) { ax += (double)cx; ay += (double)cy; cx = cy = T(0); }
-        }
-        ax += (double)cx; ay += (double)cy;
-        double2 *base = n == 0 ? yd : p.ydl + (size_t)n * p.lev_stride;
-        base[((size_t)gpl * no + i) * no + j] = make_double2(ax, ay);
-      }
-      continue;
-    }
     double ax = 0, ay = 0;
-    T cx = T(0), cy = T(0);
-    for (int g = 0; g < p.n_aux; ++g) {
-      const cpx<T> x = MA[(size_t)g * no + i];
-      cpx<T> prod;
-      if (!p.real_orb) prod = cmul(x, MB[(size_t)p.aux_neg[g] * no + j]);
-      else prod = cmulconj(x, MB[(size_t)g * no + j]);
-      cx += v[g] * prod.x;
-      cy += v[g] * prod.y;
-      if ((g & 31) == 31) { ax += (double)cx; ay += (double)cy; cx = cy = T(0); }
+    for (int n = p.n_lev - 1; n >= 0; --n) {
+      T cx = T(0), cy = T(0);
+      int cnt = 0;
+      for (int k = p.lev_start[n]; k < p.lev_start[n + 1]; ++k) {
+        const int g = p.lev_order[k];
+        const cpx<T> x = MA[(size_t)g * no + i];
+        cpx<T> prod;
+        if (!p.real_orb) prod = cmul(x, MB[(size_t)p.aux_neg[g] * no + j]);
+        else prod = cmulconj(x, MB[(size_t)g * no + j]);
+        cx += v[g] * prod.x;
+        cy += v[g] * prod.y;
+        if ((++cnt & 31) == 0) { ax += (double)cx; ay += (double)cy; cx = cy = T(0); }
+      }
+      ax += (double)cx; ay += (double)cy;
+      double2 *base = n == 0 ? yd : p.ydl + (size_t)n * p.lev_stride;
+      base[((size_t)gpl * no + i) * no + j] = make_double2(ax, ay);
     }
-    ax += (double)cx; ay += (double)cy;
-    yd[((size_t)gpl * no + i) * no + j] = make_double2(ax, ay);
+  }
+}
+
+// v[q] summed over the warp's lanes, into lane 2 q (16 values; each step halves the values a lane
+// keeps, 16 additions instead of 80)
+template <typename X> __device__ __forceinline__ X warp_sum16(X (&v)[16]) {
+  const int lane = threadIdx.x % 32;
+#pragma unroll
+  for (int h = 8; h > 0; h >>= 1) {
+    const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+    for (int q = 0; q < h; ++q) {
+      const X keep = up ? v[q + h] : v[q], give = up ? v[q] : v[q + h];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * h);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// Warp-level sums of the direct term: block (G' of the slab, 4 x 4 block of (i, j)), 4 warps with
+// their lanes over G, no padding to tiles (in FP64, with 2 FMA per clock and SM, products are what
+// counts: one thread per (i, j) with a serial sum over G took 2.3 ms for 109 G' of 32 occupied and
+// 1742 G, this form 0.5 ms).  load(g, x, y): the 4 weighted left and the 4 right factors.  CPLX: real and imaginary part,
+// else the real part alone.
+template <typename T, bool CPLX, typename F>
+__device__ __forceinline__ void direct_block(int naux, int ni, int nj, F &&load, double2 (&red)[4][16]) {
+  constexpr int B = 4, kP = CPLX ? 2 : 1;
+  constexpr bool kComp = std::is_same<T, float>::value;   // FP32: 32 products, then compensated
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  T s[kP][B * B], hi[kComp ? kP : 1][B * B], low[kComp ? kP : 1][B * B];
+  auto zero = [](T *q) {
+#pragma unroll
+    for (int a = 0; a < B * B; ++a) q[a] = T(0);
+  };
+#pragma unroll
+  for (int c = 0; c < kP; ++c) {
+    zero(s[c]);
+    if (kComp) { zero(hi[c]); zero(low[c]); }
+  }
+  auto carry = [&] {
+#pragma unroll
+    for (int c = 0; c < kP; ++c)
+#pragma unroll
+      for (int q = 0; q < B * B; ++q) {
+        kadd(hi[c][q], low[c][q], s[c][q]);
+        s[c][q] = T(0);
+      }
+  };
+  int count = 0;
+  for (int g = warp * 32 + lane; g < naux; g += 128) {
+    cpx<T> x[B], y[B];
+    load(g, x, y);
+#pragma unroll
+    for (int a = 0; a < B; ++a) {
+      if (a >= ni) continue;
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        if (b >= nj) continue;
+        T &sx = s[0][a * B + b], &sy = s[kP - 1][a * B + b];
+        sx = fma(x[a].x, y[b].x, fma(-x[a].y, y[b].y, sx));
+        if (CPLX) sy = fma(x[a].x, y[b].y, fma(x[a].y, y[b].x, sy));
+      }
+    }
+    if (kComp && (++count & 31) == 0) carry();
+  }
+  if (kComp) carry();
+  double h[kP];
+#pragma unroll
+  for (int c = 0; c < kP; ++c) {
+    double d[B * B];
+#pragma unroll
+    for (int q = 0; q < B * B; ++q) d[q] = kComp ? (double)hi[c][q] - (double)low[c][q] : (double)s[c][q];
+    h[c] = warp_sum16(d);
+  }
+  const double hx = h[0], hy = CPLX ? h[kP - 1] : 0.0;
+  if (lane % 2 == 0) red[warp][lane / 2] = make_double2(hx, hy);
+  __syncthreads();
+}
+// block index -> 4 x 4 block (bi, bj) of nb x nb, upper triangle only if asked
+__device__ __forceinline__ void block_pair(int t, int nb, bool upper, int &bi, int &bj) {
+  bi = 0;
+  if (!upper) {
+    bi = t / nb;
+    bj = t - bi * nb;
+    return;
+  }
+  while (t >= nb - bi) t -= nb - bi++;
+  bj = bi + t;
+}
+
+// The direct term without levels; real orbitals: Re Y_ij = Re Y_ji alone enters the energy
+template <typename T> __global__ void __launch_bounds__(128) k_direct_w(Plan p, int np, const cpx<T> *__restrict__ mdiag,
+                                                                        double2 *__restrict__ yd) {
+  __shared__ double2 red[4][16];
+  const int no = p.n_occ, nb = (no + 3) / 4, blocks = p.real_orb ? nb * (nb + 1) / 2 : nb * nb;
+  const int gpl = blockIdx.x / blocks;
+  int bi, bj;
+  block_pair(blockIdx.x - gpl * blocks, nb, p.real_orb, bi, bj);
+  const int i0 = 4 * bi, j0 = 4 * bj;
+  const T *v = vtab<T>(p);
+  const cpx<T> *MA = mdiag + (size_t)gpl * p.n_aux * no + i0;
+  const cpx<T> *MB = mdiag + (size_t)(p.real_orb ? gpl : gpl + np) * p.n_aux * no + j0;
+  auto load = [&](int g, cpx<T>(&x)[4], cpx<T>(&y)[4]) {
+    const T w = v[g];
+    const size_t ra = (size_t)g * no, rb = (size_t)(p.real_orb ? g : p.aux_neg[g]) * no;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[k] = i0 + k < no ? cscale(MA[ra + k], w) : cpx<T>{T(0), T(0)};
+      y[k] = j0 + k < no ? MB[rb + k] : cpx<T>{T(0), T(0)};
+      if (p.real_orb) y[k].y = -y[k].y;
+    }
+  };
+  const int ni = no - i0, nj = no - j0;
+  if (p.real_orb) direct_block<T, false>(p.n_aux, ni, nj, load, red);
+  else direct_block<T, true>(p.n_aux, ni, nj, load, red);
+  if (threadIdx.x < 16) {
+    const int a = threadIdx.x / 4, b = threadIdx.x % 4, i = i0 + a, j = j0 + b;
+    if (a >= ni || b >= nj || (p.real_orb && j < i)) return;
+    double2 s = red[0][threadIdx.x];
+    for (int w = 1; w < 4; ++w) {
+      s.x += red[w][threadIdx.x].x;
+      s.y += red[w][threadIdx.x].y;
+    }
+    double2 *y = yd + (size_t)gpl * no * no;
+    y[i * no + j] = s;
+    if (p.real_orb && i != j) y[j * no + i] = s;
   }
 }
 
@@ -1352,6 +1463,12 @@ __device__ __forceinline__ int kp_class(const Plan &p, const int *d) {
   return ((d[0] + p.mesh[0] - 1) * (2 * p.mesh[1] - 1) + (d[1] + p.mesh[1] - 1)) * (2 * p.mesh[2] - 1) +
          (d[2] + p.mesh[2] - 1);
 }
+// column of the auxiliary set at (m1, m2), or -1
+__device__ __forceinline__ int kp_column(const Plan &p, int m1, int m2) {
+  const int n = p.n;
+  if (2 * abs(m1) >= n || 2 * abs(m2) >= n) return -1;
+  return p.kcol[wrapn(m2, n) * n + wrapn(m1, n)];
+}
 // position in the auxiliary set of the integer vector g, or -1
 __device__ __forceinline__ int kp_lut(const Plan &p, int g0, int g1, int g2) {
   const int n = p.n;
@@ -1459,7 +1576,10 @@ __global__ void __launch_bounds__(256) k_zcol_k(Plan p, int gp0, int np, const v
   T accx = T(0), accy = T(0);
   for (int d = tid; d < nd; d += nth) {
     const int4 c = p.daux[d];
-    const int off = p.daux_off[d];
+    // the partners of a column lie in one column: position pq - m of A for m3 in [pc.z, pc.w]
+    const int pd = kp_column(p, -c.x + del[0], -c.y + del[1]);
+    const int4 pc = pd >= 0 ? p.daux[pd] : make_int4(0, 0, 1, 0);
+    const int pq = pd >= 0 ? p.daux_off[pd] - pc.z + del[2] : 0;
     const cpx<W> *src = tbuf + itemB * N * nd + d;
     cpx<W> a[N];
 #pragma unroll
@@ -1474,8 +1594,8 @@ __global__ void __launch_bounds__(256) k_zcol_k(Plan p, int gp0, int np, const v
           const int q = kp_lut(p, c.x + cB[0], c.y + cB[1], m + cB[2]);
           if (q >= 0) mdiag[((size_t)(gpl + np) * p.n_aux + q) * NO + I] = cscale(x, scB);
         }
-        const int qa = kp_lut(p, -c.x + del[0], -c.y + del[1], -m + del[2]);
-        if (qa >= 0) {
+        if (del[2] - m >= pc.z && del[2] - m <= pc.w) {
+          const int qa = pq - m;
           const T v = vA[qa];
           const cpx<T> prod = cmul(MA[qa], x);
           accx += v * prod.x;
@@ -1488,12 +1608,16 @@ __global__ void __launch_bounds__(256) k_zcol_k(Plan p, int gp0, int np, const v
                         (double)scB);
 }
 
-// Direct term per (primary slot, I): Y_IJ = sum_{g_c} v(g_c - kappa'/n) M_II(g_c; Q') M_JJ(-g_c + e; -Q'),
+// Direct term per primary slot: Y_IJ = sum_{g_c} v(g_c - kappa'/n) M_II(g_c; Q') M_JJ(-g_c + e; -Q'),
 // e = [kappa' != 0] per axis, from the canonically stored diagonal co-densities
 template <typename T>
-__global__ void k_direct_k(Plan p, int np, int gp0, const cpx<T> *__restrict__ mdiag, double2 *__restrict__ yd) {
-  const int gpl = blockIdx.x, I = blockIdx.y;
-  const int NO = p.n_occ;
+__global__ void __launch_bounds__(128) k_direct_k(Plan p, int np, int gp0, const cpx<T> *__restrict__ mdiag,
+                                                  double2 *__restrict__ yd) {
+  __shared__ double2 red[4][16];
+  const int NO = p.n_occ, nb = (NO + 3) / 4, gpl = blockIdx.x / (nb * nb);
+  int bi, bj;
+  block_pair(blockIdx.x - gpl * nb * nb, nb, false, bi, bj);
+  const int i0 = 4 * bi, j0 = 4 * bj;
   int M[3], e[3], dd[3];
   kp_slot(p, gp0, np, gpl, M);
   for (int a = 0; a < 3; ++a) {
@@ -1502,24 +1626,27 @@ __global__ void k_direct_k(Plan p, int np, int gp0, const cpx<T> *__restrict__ m
     dd[a] = -ks;
   }
   const T *v = vtab_k<T>(p) + (size_t)kp_class(p, dd) * p.n_aux;
-  const cpx<T> *MA = mdiag + (size_t)gpl * p.n_aux * NO;
-  const cpx<T> *MB = mdiag + (size_t)(gpl + np) * p.n_aux * NO;
-  for (int J = threadIdx.x; J < NO; J += blockDim.x) {
-    double ax = 0, ay = 0;
-    T cx = T(0), cy = T(0);
-    int cnt = 0;
-    for (int g = 0; g < p.n_aux; ++g) {
-      const T vg = v[g];
-      if (vg == T(0)) continue;
-      const int qb = kp_lut(p, e[0] - p.aux_m[3 * g], e[1] - p.aux_m[3 * g + 1], e[2] - p.aux_m[3 * g + 2]);
-      if (qb < 0) continue;
-      const cpx<T> prod = cmul(MA[(size_t)g * NO + I], MB[(size_t)qb * NO + J]);
-      cx += vg * prod.x;
-      cy += vg * prod.y;
-      if ((++cnt & 31) == 0) { ax += (double)cx; ay += (double)cy; cx = cy = T(0); }
+  const cpx<T> *MA = mdiag + (size_t)gpl * p.n_aux * NO + i0;
+  const cpx<T> *MB = mdiag + (size_t)(gpl + np) * p.n_aux * NO + j0;
+  const int ni = NO - i0, nj = NO - j0;
+  direct_block<T, true>(p.n_aux, ni, nj, [&](int g, cpx<T>(&x)[4], cpx<T>(&y)[4]) {
+    const T w = v[g];
+    const int qb = w == T(0) ? -1 : kp_lut(p, e[0] - p.aux_m[3 * g], e[1] - p.aux_m[3 * g + 1], e[2] - p.aux_m[3 * g + 2]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[k] = k < ni && qb >= 0 ? cscale(MA[(size_t)g * NO + k], w) : cpx<T>{T(0), T(0)};
+      y[k] = k < nj && qb >= 0 ? MB[(size_t)qb * NO + k] : cpx<T>{T(0), T(0)};
     }
-    ax += (double)cx; ay += (double)cy;
-    yd[((size_t)gpl * NO + I) * NO + J] = make_double2(ax, ay);
+  }, red);
+  if (threadIdx.x < 16) {
+    const int a = threadIdx.x / 4, b = threadIdx.x % 4;
+    if (a >= ni || b >= nj) return;
+    double2 s = red[0][threadIdx.x];
+    for (int w = 1; w < 4; ++w) {
+      s.x += red[w][threadIdx.x].x;
+      s.y += red[w][threadIdx.x].y;
+    }
+    yd[((size_t)gpl * NO + i0 + a) * NO + j0 + b] = s;
   }
 }
 
@@ -1527,11 +1654,11 @@ __global__ void k_direct_k(Plan p, int np, int gp0, const cpx<T> *__restrict__ m
 static __global__ void k_accum_k(Plan p, int gp0, int np, double coef, const double2 *__restrict__ sx,
                                  const double2 *__restrict__ yd) {
   const int no = p.n_occ;
-  const int ij = blockIdx.x * blockDim.x + threadIdx.x;
+  const int ij = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
   if (ij >= no * no) return;
   const int i = ij / no, j = ij % no;
   double ex = 0, exi = 0, ed = 0, edi = 0;
-  for (int gpl = 0; gpl < np; ++gpl) {
+  for (int gpl = lane; gpl < np; gpl += 32) {
     const double vv = coef * p.vprim[gp0 + gpl];
     const double2 a = sx[((size_t)gpl * no + i) * no + j], b = sx[((size_t)gpl * no + j) * no + i];
     const double2 c = yd[((size_t)gpl * no + i) * no + j], d = yd[((size_t)gpl * no + j) * no + i];
@@ -1540,6 +1667,13 @@ static __global__ void k_accum_k(Plan p, int gp0, int np, double coef, const dou
     ed += -2.0 * vv * (c.x + d.x);
     edi += -2.0 * vv * (c.y + d.y);
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    ex += __shfl_xor_sync(0xffffffffu, ex, o);
+    exi += __shfl_xor_sync(0xffffffffu, exi, o);
+    ed += __shfl_xor_sync(0xffffffffu, ed, o);
+    edi += __shfl_xor_sync(0xffffffffu, edi, o);
+  }
+  if (lane != 0) return;
   p.ex[ij] += ex;
   p.exi[ij] += exi;
   p.ed[ij] += ed;
@@ -1548,15 +1682,16 @@ static __global__ void k_accum_k(Plan p, int gp0, int np, double coef, const dou
 
 // ---------------------------------------------------------------- accumulation (FP64)
 //   e^x_ij += coef v(G') (X_ij + X_ji),   e^d_ij += -2 coef v(G') (Y_ij + Y_ji)
-// coef = w_k / (Omega^2 N_FFT^2); the sum over the slab runs in a fixed order.
+// coef = w_k / (Omega^2 N_FFT^2); the sum over the slab runs in a fixed order, one warp per (i, j)
+// (one thread per (i, j) left a chain of loads as long as the slab: 40 us for 128 G').
 static __global__ void k_accum(Plan p, int gp0, int np, double coef, const double2 *__restrict__ sx,
                         const double2 *__restrict__ yd) {
   const int no = p.n_occ;
-  const int ij = blockIdx.x * blockDim.x + threadIdx.x;
+  const int ij = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
   if (ij >= no * no) return;
   const int i = ij / no, j = ij % no;
   double ex = 0, exi = 0, ed = 0, edi = 0;
-  for (int gpl = 0; gpl < np; ++gpl) {
+  for (int gpl = lane; gpl < np; gpl += 32) {
     const double vv = coef * p.v_aux64[p.prim[gp0 + gpl]];
     const double2 a = sx[((size_t)gpl * no + i) * no + j], b = sx[((size_t)gpl * no + j) * no + i];
     const double2 c = yd[((size_t)gpl * no + i) * no + j], d = yd[((size_t)gpl * no + j) * no + i];
@@ -1565,6 +1700,13 @@ static __global__ void k_accum(Plan p, int gp0, int np, double coef, const doubl
     ed += -2.0 * vv * (c.x + d.x);
     edi += -2.0 * vv * (c.y + d.y);
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    ex += __shfl_xor_sync(0xffffffffu, ex, o);
+    exi += __shfl_xor_sync(0xffffffffu, exi, o);
+    ed += __shfl_xor_sync(0xffffffffu, ed, o);
+    edi += __shfl_xor_sync(0xffffffffu, edi, o);
+  }
+  if (lane != 0) return;
   p.ex[ij] += ex;
   p.exi[ij] += exi;
   p.ed[ij] += ed;

@@ -222,7 +222,7 @@ int set_sym_rows(ltmp2_ctx *c, const std::vector<unsigned char> *lev) {
     p.lev_rows[k] = rows;
   }
   const double total = 0.5 * n * (n + 1.0);
-  const double target = total / std::min(304.0, std::max(1.0, total / 1024.0));
+  const double target = total / std::min(304.0, std::max(1.0, total / 64.0));
   std::vector<int2> g;
   int first = 0;
   double work = 0.0;
@@ -1077,7 +1077,12 @@ int ltmp2_setup_kpoints(const ltmp2_kpoint_system *sys, ltmp2_ctx **out) {
       return cuda_status(cudaMemcpy(*dptr, vec.data(), vec.size() * sizeof(X), cudaMemcpyHostToDevice));
     };
     std::vector<double> heps(sys->eps, sys->eps + (size_t)p.nk * p.n_orb);
-    int *d_prim = nullptr, *d_lut = nullptr;
+    int *d_prim = nullptr, *d_lut = nullptr, *d_kcol = nullptr;
+    std::vector<int> kcol((size_t)p.n * p.n, -1);
+    for (size_t q = 0; q < hp.daux.size(); ++q) {
+      const int m1 = (hp.daux[q].x + p.n) % p.n, m2 = (hp.daux[q].y + p.n) % p.n;
+      kcol[(size_t)m2 * p.n + m1] = (int)q;
+    }
     double *d_vprim = nullptr, *d_vc64 = nullptr, *d_eps = nullptr;
     float *d_vc32 = nullptr;
     if (!rc) rc = up(&p.dorb, hp.dorb);
@@ -1091,12 +1096,14 @@ int ltmp2_setup_kpoints(const ltmp2_kpoint_system *sys, ltmp2_ctx **out) {
     if (!rc) rc = up(&d_vc64, kh.vcls64);
     if (!rc) rc = up(&d_vc32, kh.vcls32);
     if (!rc) rc = up(&d_lut, kh.lut);
+    if (!rc) rc = up(&d_kcol, kcol);
     if (!rc) rc = up(&d_eps, heps);
     p.prim_m = d_prim;
     p.vprim = d_vprim;
     p.vcls64 = d_vc64;
     p.vcls32 = d_vc32;
     p.lut = d_lut;
+    p.kcol = d_kcol;
     p.eps = d_eps;
     const size_t no2 = (size_t)p.n_occ * p.n_occ;
     if (!rc) rc = dalloc(c, &p.ex, no2);

@@ -354,8 +354,8 @@ cudaError_t Path<T>::slab_post(const Plan &p, int gp0, int np, double coef, cuda
   {
     ScopedStage s(tm, kStageDirect);
     int th = no < 128 ? ((no + 31) / 32) * 32 : 128;
-    // FP32: the shared-memory tiled kernel (1.6x faster on the 24^3 workload); FP64 is
-    // bound by the FP64 pipe either way and the one-warp-per-(G', i) kernel is 12 % faster
+    // FP32: the shared-memory tiled kernel; FP64 is bound by the FP64 pipe, and the warp-level
+    // sums pad nothing and take the real part alone where only that enters
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
       if (!lev && p.tc && p.tc->direct_on()) {   // real orbitals: one tensor-core product per G'
@@ -365,18 +365,19 @@ cudaError_t Path<T>::slab_post(const Plan &p, int gp0, int np, double coef, cuda
     }
     if (done) {
     } else if (lev) {
-      k_direct<T, true><<<dim3(np, no), th, 0, st>>>(p, np, (const cpx<T> *)p.mdiag, p.yd);
+      k_direct_lev<T><<<dim3(np, no), th, 0, st>>>(p, np, (const cpx<T> *)p.mdiag, p.yd);
     } else if (std::is_same<T, float>::value) {
       const int t = (no + 31) / 32;
       k_direct_tiled<T><<<dim3(np, t, t), 256, 0, st>>>(p, np, (const cpx<T> *)p.mdiag, p.yd);
     } else {
-      k_direct<T, false><<<dim3(np, no), th, 0, st>>>(p, np, (const cpx<T> *)p.mdiag, p.yd);
+      const int t = (no + 3) / 4;
+      k_direct_w<T><<<np * (p.real_orb ? t * (t + 1) / 2 : t * t), 128, 0, st>>>(p, np, (const cpx<T> *)p.mdiag, p.yd);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   {
     ScopedStage s(tm, kStageAccum);
-    k_accum<<<(no * no + 127) / 128, 128, 0, st>>>(p, gp0, np, coef, p.sx, p.yd);
+    k_accum<<<(no * no + 3) / 4, 128, 0, st>>>(p, gp0, np, coef, p.sx, p.yd);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (lev) {
       k_accum_lev<<<dim3((no * no + 31) / 32, p.n_lev - 1), 32, 0, st>>>(p, gp0, np, coef);
@@ -522,13 +523,13 @@ cudaError_t Path<T>::slab_k(const Plan &p, int gp0, int np, double coef, cudaStr
   }
   {
     ScopedStage s(tm, kStageDirect);
-    const int th = NO < 128 ? ((NO + 31) / 32) * 32 : 128;
-    k_direct_k<T><<<dim3(np, NO), th, 0, st>>>(p, np, gp0, (const cpx<T> *)p.mdiag, p.yd);
+    const int t = (NO + 3) / 4;
+    k_direct_k<T><<<np * t * t, 128, 0, st>>>(p, np, gp0, (const cpx<T> *)p.mdiag, p.yd);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   {
     ScopedStage s(tm, kStageAccum);
-    k_accum_k<<<(NO * NO + 127) / 128, 128, 0, st>>>(p, gp0, np, coef, p.sx, p.yd);
+    k_accum_k<<<(NO * NO + 3) / 4, 128, 0, st>>>(p, gp0, np, coef, p.sx, p.yd);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

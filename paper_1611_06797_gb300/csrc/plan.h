@@ -171,6 +171,7 @@ struct Plan {
   const double *vcls64 = nullptr;      // [n_cls][n_aux] 4 pi / |g + delta/n|^2 inside the sphere, else 0
   const float *vcls32 = nullptr;
   const int *lut = nullptr;            // [n^3] position in A of the grid point, -1 if absent
+  const int *kcol = nullptr;           // [n m2][n m1] column of A, -1 if absent
   int slots_per_prim() const { return (real_orb && nk == 0) ? 1 : 2; }
 };
 

@@ -2,11 +2,14 @@
 times its transpose) against the slabs of the outer G' loop, which every partial range takes, at
 the sizes of passes where they can go wrong: one column, ragged parts of one orbital, several
 orbitals with a ragged last pass, everything in one; with cutoff levels and a pair mask."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 
 import paper_1611_06797_gb300 as L
 from oracle import OracleSystem, denominator_range, sinc_laplace_quadrature
+from synth import SPECS, build_model_solid
 from tests.conftest import solid
 
 pytestmark = pytest.mark.gpu
@@ -68,4 +71,19 @@ def test_levels_of_the_symmetric_passes(real):
     L.ltmp2_set_extrapolation(ctx, 1)
     e = L.ltmp2_energy(ctx, tau, w)
     assert abs(e[0] - plain[0]) < 1e-14 * abs(plain[0])
+    L.ltmp2_destroy(ctx)
+
+
+@pytest.mark.parametrize("n_occ", [1, 3, 5, 9])
+@pytest.mark.parametrize("real", [True, False], ids=["real", "general"])
+def test_direct_blocks(n_occ, real):
+    """The direct term's 4 x 4 blocks of (i, j) at ragged orbital counts: the slabs' against the
+    symmetric passes' (another kernel, with its own order of the sum)."""
+    s = build_model_solid(replace(SPECS["tiny2"], wells=n_occ, n_occ=n_occ), random_phases=not real)
+    tau, w = sinc_laplace_quadrature(2, *denominator_range(OracleSystem.from_solid(s)))
+    ctx = L.setup_from_solid(s, precision=L.FP64, real=real)
+    ed, ex, ep = _halves(ctx, tau, w, L.ltmp2_num_primary_gprime(ctx))
+    e = L.ltmp2_energy(ctx, tau, w)
+    tol = 1e-13 * abs(ed)   # FP64 sums of 1e5 terms in another order
+    assert abs(e[0] - ed) < tol and abs(e[1] - ex) < tol and np.abs(e[2] - ep).max() < tol
     L.ltmp2_destroy(ctx)
