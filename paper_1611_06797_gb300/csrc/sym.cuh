@@ -87,42 +87,48 @@ __global__ void __launch_bounds__(256) k_zsym(Plan p, int gp0) {
 // tile are summed in FP32, tiles in FP64.  Bound by reading S once (12.7 GB per Laplace point of the
 // 24^3 system in FP64).
 template <typename T> __global__ void __launch_bounds__(256) k_xsym(Plan p, double *__restrict__ rows) {
-  __shared__ cpx<T> tile[32][33];
+  __shared__ cpx<T> tile[2][32][33];
   const int nt = (p.n_idx + 31) / 32, R = nt - 1 - (int)blockIdx.y, pair = blockIdx.x;
   const int n = p.n_idx;
   int i, j;
   sym_pair(p, pair, i, j);
   if (sym_screened(p, i, j)) return;
   const cpx<T> *S = sym_matrix<T>(p, i, j);
+  const size_t n2 = (size_t)n * n;
+  const bool two = p.sym_planes == 2;
   const T *v = vtab<T>(p);
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   double acc[4] = {0, 0, 0, 0};
   for (int C = 0; C <= R; ++C) {
     const int col = C * 32 + tx;
     const T vc = col < n ? v[p.sym_order[col]] : T(0);
-    T part[4] = {T(0), T(0), T(0), T(0)};
-    for (int pl = 0; pl < p.sym_planes; ++pl) {
-      const cpx<T> *P = S + (size_t)pl * n * n;
-      cpx<T> x[4];
+    cpx<T> x[2][4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int r = C * 32 + ty + 8 * k, c = R * 32 + tx;     // the transposed tile's rows
-        tile[ty + 8 * k][tx] = r < n && c < n ? P[(size_t)r * n + c] : cpx<T>{T(0), T(0)};
-        const int row = R * 32 + ty + 8 * k;
-        x[k] = row < n && col < n ? P[(size_t)row * n + col] : cpx<T>{T(0), T(0)};
+    for (int k = 0; k < 4; ++k) {
+      const int r = C * 32 + ty + 8 * k, c = R * 32 + tx;     // the transposed tile's rows
+      const int row = R * 32 + ty + 8 * k;
+      const bool in_t = r < n && c < n, in_x = row < n && col < n;
+      const cpx<T> zero{T(0), T(0)};
+      tile[0][ty + 8 * k][tx] = in_t ? S[(size_t)r * n + c] : zero;
+      x[0][k] = in_x ? S[(size_t)row * n + col] : zero;
+      if (two) {
+        tile[1][ty + 8 * k][tx] = in_t ? S[n2 + (size_t)r * n + c] : zero;
+        x[1][k] = in_x ? S[n2 + (size_t)row * n + col] : zero;
       }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int row = R * 32 + ty + 8 * k;
-        const cpx<T> y = tile[tx][ty + 8 * k];
-        const T t = pl == 0 ? x[k].x * y.x + x[k].y * y.y : x[k].x * y.x - x[k].y * y.y;
-        if (col <= row) part[k] += col < row ? t + t : t;
-      }
-      __syncthreads();
     }
+    __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] += (double)(vc * part[k]);
+    for (int k = 0; k < 4; ++k) {
+      const int row = R * 32 + ty + 8 * k;
+      const cpx<T> y = tile[0][tx][ty + 8 * k];
+      T t = x[0][k].x * y.x + x[0][k].y * y.y;
+      if (two) {
+        const cpx<T> z = tile[1][tx][ty + 8 * k];
+        t += x[1][k].x * z.x - x[1][k].y * z.y;
+      }
+      if (col <= row) acc[k] += (double)(vc * (col < row ? t + t : t));
+    }
+    __syncthreads();
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -159,7 +165,7 @@ template <typename T> __global__ void k_xsym_sum(Plan p, const double *__restric
 // rows g' of v(g') sum_{p <= g'} c v(p) Re[S_ii conj S_jj] (general orbitals: Re[S_ii(p, g')
 // S_jj(-p, -g')], whose index is the neighbour's; c = 1 within the pair of rows g', -g').  p and q: the
 // two channels' plans (the same one for a closed shell; then only blocks with j >= i are there).
-// A warp takes every eighth row of the group, its lanes the columns: no product is padded, which in
+// The warps take the rows' 32-column chunks in turn, a lane a column: no product is padded, which in
 // FP64 (2 FMA per clock and SM) is what counts: 32 x 32 tiles through shared memory took 1.7 ms
 // per Laplace point on the 8^3 system with 2 occupied.  FP32 sums are compensated.
 template <typename T>
@@ -188,12 +194,15 @@ __global__ void __launch_bounds__(256) k_dsym(Plan p, Plan q, bool triangle, dou
     for (int b = 0; b < B; ++b) acc[a][b] = hi[a][b] = cmp[a][b] = T(0);
   const int2 rows = p.sym_groups[blockIdx.x];
   const cpx<T> *Ma = (const cpx<T> *)p.mdsym + i0 * stride, *Mb = (const cpx<T> *)q.mdsym + j0 * stride;
-  for (int g = rows.x + warp; g < rows.y; g += 8) {
+  // the rows' 32-column chunks go round the warps
+  int chunk = 0, count = 0;
+  for (int g = rows.x; g < rows.y; ++g) {
     const T vg = v[p.sym_order[g]];
     const int end = gen ? (g | 1) + 1 : g + 1;            // columns of the lower triangle
     const int gj = gen ? g ^ 1 : g, twice = gen ? (g & ~1) : g;
-    int count = 0;
-    for (int c = lane; c < end; c += 32) {
+    for (int c0 = ((warp - chunk) & 7) * 32; c0 < end; c0 += 256) {
+      const int c = c0 + lane;
+      if (c >= end) continue;
       const T w = v[p.sym_order[c]] * vg * (c < twice ? T(2) : T(1));
       const int cj = gen ? c ^ 1 : c;
       for (int pl = 0; pl < p.sym_planes; ++pl) {
@@ -213,7 +222,7 @@ __global__ void __launch_bounds__(256) k_dsym(Plan p, Plan q, bool triangle, dou
             if (j0 + b < nj) acc[a][b] = fma(xr, y[b].x, fma(xi, y[b].y, acc[a][b]));
         }
       }
-      if (kComp && (++count & 15) == 0) {   // at most 64 products in plain FP32
+      if (kComp && (++count & 15) == 0) {   // at most 64 products in plain FP32 (a lane past the end skips a turn)
 #pragma unroll
         for (int a = 0; a < B; ++a)
 #pragma unroll
@@ -223,24 +232,18 @@ __global__ void __launch_bounds__(256) k_dsym(Plan p, Plan q, bool triangle, dou
           }
       }
     }
-    if (kComp) {
-#pragma unroll
-      for (int a = 0; a < B; ++a)
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-          kadd(hi[a][b], cmp[a][b], acc[a][b]);
-          acc[a][b] = T(0);
-        }
-    }
+    chunk += (end + 31) / 32;
   }
+  double sum[B * B];
 #pragma unroll
   for (int a = 0; a < B; ++a)
 #pragma unroll
     for (int b = 0; b < B; ++b) {
-      double s = kComp ? (double)hi[a][b] - (double)cmp[a][b] : (double)acc[a][b];
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) red[warp][a * B + b] = s;
+      if (kComp) kadd(hi[a][b], cmp[a][b], acc[a][b]);
+      sum[a * B + b] = kComp ? (double)hi[a][b] - (double)cmp[a][b] : (double)acc[a][b];
     }
+  const double s = warp_sum16(sum);
+  if (lane % 2 == 0) red[warp][lane / 2] = s;
   __syncthreads();
   if (threadIdx.x < B * B) {
     double s = 0.0;
