@@ -191,10 +191,11 @@ int ltmp2_autotune(ltmp2_ctx *ctx, int *slab, int *gemm_variant);
 
 /* Settings in effect for ctx: values[0] slab size, [1] tensor-core GEMM layout (5, or 4 for general orbitals; one kernel serves both; -1 in
  * FP64 or with LTMP2_FLAG_SIMT_GEMM), [2] plane FFT kernel (0 full-plane passes,
- * 1 compacted passes, 2 product in registers with a compact intermediate, 3 the same with
- * every warp on its own occupied planes and no block barriers; set-up chooses 3 in
- * LTMP2_FP32 and 2 in LTMP2_FP64), [3] occupied planes per plane-kernel block, for
- * kernel 3 per warp step (0 = default), [4] the precision form's
+ * 1 compacted passes, 2 product in registers with a compact intermediate, in LTMP2_FP32 on
+ * pairs of columns, 3 every warp on its own occupied planes and no block barriers; set-up
+ * chooses 3 in LTMP2_FP32 on grids above 27^3, else 2; LTMP2_FP64 has one kernel, which
+ * every value runs), [3] occupied planes per plane-kernel block, for
+ * kernel 3 per warp step (0 = default; a launch takes no more than fit), [4] the precision form's
  * Green's function and transformed states in 3xTF32 (1; set up at first use) or from
  * exact slices (0, the default: the 3xTF32 build's plain FP32 sums over K = n_v left
  * 4x the error in E_d on the 36^3 workload), [5] its direct-term

@@ -131,7 +131,7 @@ template <int DIR> struct Radix<long long, 5, DIR> {
 
 // v * exp(DIR * 2 pi i E / NT): eighths of a turn take two products, other angles three
 // shears (tan(t/2), sin t, tan(t/2)) after a quarter turn that brings |t| to at most 1/8 turn
-template <int NT, int E, int DIR> __host__ __device__ __forceinline__ cpx<long long> fx_twiddle(cpx<long long> v) {
+template <int NT, int E, int DIR> __host__ __device__ __forceinline__ cpx<long long> ct_twiddle(cpx<long long> v) {
   constexpr int e = E % NT;
   if constexpr ((4 * e) % NT == 0) {
     constexpr int q = (4 * e) / NT;
@@ -142,11 +142,11 @@ template <int NT, int E, int DIR> __host__ __device__ __forceinline__ cpx<long l
   } else if constexpr (8 * e > NT) {
     // turn by a quarter and go on with what is left, in (-1/8, 1/8] of a turn
     constexpr int quarters = (8 * e + NT) / (2 * NT);          // nearest number of quarter turns
-    const cpx<long long> u = fx_twiddle<4, quarters % 4, DIR>(v);
+    const cpx<long long> u = ct_twiddle<4, quarters % 4, DIR>(v);
     constexpr int rest = 4 * e - quarters * NT;                // of 4 NT
     if constexpr (rest == 0) return u;
-    else if constexpr (rest > 0) return fx_twiddle<4 * NT, rest, DIR>(u);
-    else return fx_twiddle<4 * NT, -rest, -DIR>(u);
+    else if constexpr (rest > 0) return ct_twiddle<4 * NT, rest, DIR>(u);
+    else return ct_twiddle<4 * NT, -rest, -DIR>(u);
   } else if constexpr (8 * e == NT) {
     constexpr long long r2 = (long long)fxc::sinn(1, 8);
     return DIR > 0 ? cpx<long long>{fx_mulc<r2>(v.x - v.y), fx_mulc<r2>(v.x + v.y)}
@@ -172,9 +172,10 @@ template <typename F, int... I> __host__ __device__ __forceinline__ void fx_each
   (f(std::integral_constant<int, I>{}), ...);
 }
 
-// The line FFT on fixed-point values: the splits of LineFFT with compile-time twiddles
-template <int N, int DIR, int NT> struct LineFFT<long long, N, DIR, NT> {
-  typedef cpx<long long> C;
+// The line FFT with compile-time twiddles, by the splits of LineFFT: fixed-point values V (and the
+// packed pairs of pair.cuh, which bring their own ct_twiddle)
+template <typename V, int N, int DIR> struct CtLineFFT {
+  typedef cpx<V> C;
   static __host__ __device__ __forceinline__ void run(C (&a)[N]) {
     constexpr int P1 = pfa_n1(N);
     if constexpr (P1 > 0) {
@@ -186,7 +187,7 @@ template <int N, int DIR, int NT> struct LineFFT<long long, N, DIR, NT> {
         C v[N1];
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) v[n1] = a[(N2 * n1 + N1 * n2) % N];
-        LineFFT<long long, N1, DIR, N1>::run(v);
+        CtLineFFT<V, N1, DIR>::run(v);
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) t[k1 * N2 + n2] = v[k1];
       }
@@ -195,7 +196,7 @@ template <int N, int DIR, int NT> struct LineFFT<long long, N, DIR, NT> {
         C u[N2];
 #pragma unroll
         for (int n2 = 0; n2 < N2; ++n2) u[n2] = t[k1 * N2 + n2];
-        LineFFT<long long, N2, DIR, N2>::run(u);
+        CtLineFFT<V, N2, DIR>::run(u);
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) a[(N2 * A * k1 + N1 * B * k2) % N] = u[k2];
       }
@@ -208,10 +209,10 @@ template <int N, int DIR, int NT> struct LineFFT<long long, N, DIR, NT> {
         C v[R];
 #pragma unroll
         for (int n1 = 0; n1 < R; ++n1) v[n1] = a[M * n1 + n2];
-        Radix<long long, R, DIR>::run(v);
+        Radix<V, R, DIR>::run(v);
         fx_each([&](auto k1c) {
           constexpr int k1 = decltype(k1c)::value;
-          t[M * k1 + n2] = fx_twiddle<N, n2 * k1, DIR>(v[k1]);
+          t[M * k1 + n2] = ct_twiddle<N, n2 * k1, DIR>(v[k1]);
         }, std::make_integer_sequence<int, R>{});
       }, std::make_integer_sequence<int, M>{});
 #pragma unroll
@@ -219,12 +220,13 @@ template <int N, int DIR, int NT> struct LineFFT<long long, N, DIR, NT> {
         C u[M];
 #pragma unroll
         for (int n2 = 0; n2 < M; ++n2) u[n2] = t[M * k1 + n2];
-        if constexpr (M > 1) LineFFT<long long, M, DIR, M>::run(u);
+        if constexpr (M > 1) CtLineFFT<V, M, DIR>::run(u);
 #pragma unroll
         for (int k2 = 0; k2 < M; ++k2) a[k1 + R * k2] = u[k2];
       }
     }
   }
 };
+template <int N, int DIR, int NT> struct LineFFT<long long, N, DIR, NT> : CtLineFFT<long long, N, DIR> {};
 
 }  // namespace ltmp2

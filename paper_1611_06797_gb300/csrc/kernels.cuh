@@ -9,7 +9,7 @@
 #include <type_traits>
 
 #include "fft.cuh"
-#include "fixed.cuh"
+#include "pair.cuh"
 #include "plan.h"
 
 namespace ltmp2 {
@@ -64,7 +64,7 @@ template <> struct Codensity<double> {
 
 // column of a slab -> its orbital, the number of items i, and the item's place in tbuf: every
 // i (or the kept list), or i <= j in a pass of the pairs' symmetry (sym.cuh)
-__device__ __forceinline__ int cols_per_slot(const Plan &p) { return p.sym_nj ? p.sym_nj : p.n_occ; }
+__host__ __device__ __forceinline__ int cols_per_slot(const Plan &p) { return p.sym_nj ? p.sym_nj : p.n_occ; }
 __device__ __forceinline__ int col_orbital(const Plan &p, int col) {
   return p.sym_nj ? p.sym_j0 + col % p.sym_nj : col % p.n_occ;
 }
@@ -571,64 +571,100 @@ __global__ void k_planes2(Plan p, int ib, const cpx<T> *__restrict__ z1, cpx<T> 
   }
 }
 
-// Same result as k_planes, with the product formed in registers.  Per block of ib
-// occupied i:
+// FP32: the block takes the planes z of two columns (slots 2 pair and 2 pair + 1 of the same j, whose
+// items are the same occupied i), the two lines of a pair side by side in one thread (f2):
+//  inverse: the orbital-disk values of the two planes to w_j(x, y, z), as in plane_inverse;
+//  then per block of ib occupied i:
 //  x pass : thread (i, y) loads row y of phi_i (from the plane-transposed copy, coalesced
-//           across the warp, L2 resident) and of w_j^{G'} (shared), multiplies conj(phi_i) w
-//           in registers, transforms, and keeps only the m1 of the aux range: a compact
-//           [ib][N][nxa] intermediate (nxa is odd, so the row pitch spreads the banks);
+//           across the warp, L2 resident) and of both w (shared), forms conj(phi_i) w in registers,
+//           transforms, and keeps only the m1 of the aux range: a compact [i][N][nxa]
+//           intermediate of 16-byte elements (nxa is odd, so the row pitch spreads the banks);
 //  y pass : thread (i, m1) transforms its column and writes it back in place (consecutive
 //           threads, consecutive addresses);
 //  copy   : the aux-disk entries gathered through a per-block table (consecutive disk
 //           columns of one m1 are nxa apart: no bank conflicts) and written coalesced to
 //           tbuf[(col, i)][z][d_aux].
-template <typename T, int N>
-__device__ __forceinline__ void planes3_body(const Plan &p, int ib, int z, int col, const cpx<T> *__restrict__ z1,
-                                             cpx<T> *__restrict__ tbuf, unsigned char *smem_raw) {
-  constexpr int P = N + 1;
-  cpx<T> *xp = reinterpret_cast<cpx<T> *>(smem_raw);
+// Pairs issue half the instructions of k_planes4 (8.7e8 -> 5.0e8 for 3484 columns of 24^3) and two thirds
+// of its shared-memory wavefronts (1.85e8 -> 1.39e8).  Now bound by latency: 44 % of the issue slots and 60 %
+// of the L1 rate at 12 warps per SM, which the registers of a pair of lines (162) allow; blocks of 64 threads
+// lose the least at the barriers (24^3, ib = 4: 82.6 ms per energy, 93.2 ms with 96 threads; k_planes4 97.2).
+template <int N>
+__device__ __forceinline__ void planes3_body_pair(const Plan &p, int ib, int z, int colA, int colB,
+                                                  const cpx<float> *__restrict__ z1, cpx<float> *__restrict__ tbuf,
+                                                  unsigned char *smem_raw) {
+  constexpr int P = N | 1;   // an odd pitch of 16-byte elements spreads the banks
+  cpx<f2> *xp = reinterpret_cast<cpx<f2> *>(smem_raw);
   const int nxa = p.mxhi_aux - p.mxlo_aux + 1;   // odd: the aux sphere is symmetric
   const int nd = p.n_daux;
   const int Q = plane_stride(N, nxa);
-  cpx<T> *wk = xp + N * P;                    // [ib] planes of [N][nxa], Q elements apart
+  cpx<f2> *wk = xp + N * P;                      // [ib] planes of [N][nxa], Q elements apart
   int *ytab = reinterpret_cast<int *>(wk + (size_t)ib * Q);   // [nd] position of disk column d in a plane of wk
   const int tid = threadIdx.x, nth = blockDim.x;
   const int no = p.n_occ;
   const int mlo = p.mxlo_aux, mhi = p.mxhi_aux;
   const unsigned inv_nxa = ((1u << 20) + nxa - 1) / nxa;   // ceil(2^20 / nxa)
+  const cpx<float> *za = z1 + ((size_t)colA * N + z) * p.n_dorb, *zb = z1 + ((size_t)colB * N + z) * p.n_dorb;
   for (int d = tid; d < nd; d += nth) {
     const int4 c = p.daux[d];
     ytab[d] = wrapn(c.y, N) * nxa + (c.x - mlo);
   }
-  plane_inverse<T, N>(p, z1 + ((size_t)col * N + z) * p.n_dorb, xp);   // ends with a barrier
-  const cpx<T> *ut = (const cpx<T> *)p.ut;
-  const T *utr = (const T *)p.utr;
-  const int jcol = col_orbital(p, col), ni = col_items(p, jcol);
+  for (int e = tid; e < N * P; e += nth) f2_store(xp + e, {{0}, {0}});
+  __syncthreads();
+  for (int d = tid; d < p.n_dorb; d += nth) {
+    const int4 c = p.dorb[d];
+    const cpx<float> u = za[d], v = zb[d];
+    f2_store(xp + wrapn(c.y, N) * P + wrapn(c.x, N), {f2_make(u.x, v.x), f2_make(u.y, v.y)});
+  }
+  __syncthreads();
+  const int nxo = p.mxhi_orb - p.mxlo_orb + 1;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int t = tid; t < (pass == 0 ? nxo : N); t += nth) {
+      cpx<f2> *line = pass == 0 ? xp + wrapn(p.mxlo_orb + t, N) : xp + t * P;
+      const int stride = pass == 0 ? P : 1;
+      cpx<f2> a[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) a[k] = f2_load(line + k * stride);
+      LineFFT<f2, N, +1>::run(a);
+#pragma unroll
+      for (int k = 0; k < N; ++k) f2_store(line + k * stride, a[k]);
+    }
+    __syncthreads();
+  }
+  const cpx<float> *ut = (const cpx<float> *)p.ut;
+  const float *utr = (const float *)p.utr;
+  const int jcol = col_orbital(p, colA), ni = col_items(p, jcol);
   const int *ilist = p.keep_count ? p.keep_list + (size_t)jcol * no : nullptr;
   for (int i0 = 0; i0 < ni; i0 += ib) {
     const int nb = min(ib, ni - i0);
     for (int t = tid; t < nb * N; t += nth) {
       const int il = t / N, y = t - il * N;
       const int iocc = ilist ? ilist[i0 + il] : i0 + il;
-      cpx<T> a[N];
+      cpx<f2> a[N];
       // row y of phi_i from the transposed plane: element x at x N + y, so the threads of
       // a warp (consecutive y) read consecutive addresses.  Real orbitals: phi_i is real,
       // so conj(phi_i) w is two real products per point and half the bytes are read.
       const size_t urow = ((size_t)iocc * N + z) * N * N + y;
-      const cpx<T> *wr = xp + y * P;
+      const cpx<f2> *wr = xp + y * P;
       if (utr) {
 #pragma unroll
-        for (int k = 0; k < N; ++k) a[k] = cscale(wr[k], utr[urow + k * N]);
+        for (int k = 0; k < N; ++k) {
+          const float u = utr[urow + k * N];
+          a[k] = cscale(f2_load(wr + k), f2_make(u, u));
+        }
       } else {
 #pragma unroll
-        for (int k = 0; k < N; ++k) a[k] = cmul(cconj(ut[urow + k * N]), wr[k]);
+        for (int k = 0; k < N; ++k) {
+          const cpx<float> u = ut[urow + k * N];
+          const cpx<f2> w = f2_load(wr + k);
+          a[k] = {f2_fma(u.x, w.x, f2_mul(u.y, w.y)), f2_fma(u.x, w.y, f2_mul(-u.y, w.x))};
+        }
       }
-      LineFFT<T, N, -1>::run(a);
-      cpx<T> *row = wk + (size_t)il * Q + y * nxa - mlo;   // row[m] for m in [mlo, mhi]
+      LineFFT<f2, N, -1>::run(a);
+      cpx<f2> *row = wk + (size_t)il * Q + y * nxa - mlo;   // row[m] for m in [mlo, mhi]
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         const int m = freq_of<N>(k);
-        if (m >= mlo && m <= mhi) row[m] = a[k];
+        if (m < 0 ? m >= mlo : m <= mhi) f2_store(row + m, a[k]);
       }
     }
     __syncthreads();
@@ -636,20 +672,27 @@ __device__ __forceinline__ void planes3_body(const Plan &p, int ib, int z, int c
       // t / nxa by an exact multiply-shift: t < 2^12 and nxa < 2^7 keep the rounding of the
       // reciprocal below one part in nxa
       const int il = (int)(((unsigned)t * inv_nxa) >> 20), xa = t - il * nxa;
-      cpx<T> *src = wk + (size_t)il * Q + xa;
-      cpx<T> b[N];
+      cpx<f2> *src = wk + (size_t)il * Q + xa;
+      cpx<f2> b[N];
 #pragma unroll
-      for (int k = 0; k < N; ++k) b[k] = src[k * nxa];
-      LineFFT<T, N, -1>::run(b);
+      for (int k = 0; k < N; ++k) b[k] = f2_load(src + k * nxa);
+      LineFFT<f2, N, -1>::run(b);
 #pragma unroll
-      for (int k = 0; k < N; ++k) src[k * nxa] = b[k];
+      for (int k = 0; k < N; ++k) f2_store(src + k * nxa, b[k]);
     }
     __syncthreads();
     for (int il = 0; il < nb; ++il) {
-      const size_t item = item_of(p, col, ilist ? ilist[i0 + il] : i0 + il);
-      cpx<T> *dst = tbuf + (item * N + z) * nd;
-      const cpx<T> *src = wk + (size_t)il * Q;
-      for (int d = tid; d < nd; d += nth) dst[d] = src[ytab[d]];
+      const int iocc = ilist ? ilist[i0 + il] : i0 + il;
+      cpx<float> *da = tbuf + (item_of(p, colA, iocc) * N + z) * nd, *db = tbuf + (item_of(p, colB, iocc) * N + z) * nd;
+      const cpx<f2> *src = wk + (size_t)il * Q;
+      for (int d = tid; d < nd; d += nth) {
+        const cpx<f2> v = f2_load(src + ytab[d]);
+        cpx<float> a, b;
+        f2_get(v.x, a.x, b.x);
+        f2_get(v.y, a.y, b.y);
+        da[d] = a;
+        db[d] = b;
+      }
     }
     __syncthreads();
   }
@@ -825,19 +868,31 @@ static __global__ void k_wnorm(Plan p, const cpx<double> *__restrict__ w) {
   if (threadIdx.x == 0) p.wen3[blockIdx.x] = fx_exponent(s2 * ((double)p.n * p.n * p.n * (1.0 + 1e-9)));
 }
 
+// column of the q-th pair of columns' first slot
+__device__ __forceinline__ int first_of_pair(const Plan &p, int q) {
+  const int cps = cols_per_slot(p), pair = q / cps;
+  return 2 * pair * cps + (q - pair * cps);
+}
+
+// Plane z of column col (FP32: of a pair of slots' columns, taken at the first of the two) of ncols
 template <typename T, int N>
-__device__ __forceinline__ void planes3_any(const Plan &p, int ib, int z, int col, const void *z1, void *tbuf,
+__device__ __forceinline__ void planes3_any(const Plan &p, int ib, int z, int col, int ncols, const void *z1, void *tbuf,
                                             unsigned char *smem_raw) {
-  if constexpr (std::is_same<T, double>::value)
+  if constexpr (std::is_same<T, double>::value) {
     planes3_body_fx<N>(p, ib, z, col, (const cpx<double> *)z1, (cpx<long long> *)tbuf, smem_raw);
-  else
-    planes3_body<T, N>(p, ib, z, col, (const cpx<T> *)z1, (cpx<T> *)tbuf, smem_raw);
+  } else {
+    const int cps = cols_per_slot(p);
+    if ((col / cps) & 1) return;
+    planes3_body_pair<N>(p, ib, z, col, col + cps < ncols ? col + cps : col, (const cpx<float> *)z1, (cpx<float> *)tbuf,
+                         smem_raw);
+  }
 }
 
 template <typename T, int N>
-__global__ void k_planes3(Plan p, int ib, const void *__restrict__ z1, void *__restrict__ tbuf) {
+__global__ void k_planes3(Plan p, int ib, int ncols, const void *__restrict__ z1, void *__restrict__ tbuf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  planes3_any<T, N>(p, ib, blockIdx.x, blockIdx.y, z1, tbuf, smem_raw);
+  const int col = std::is_same<T, double>::value ? (int)blockIdx.y : first_of_pair(p, blockIdx.y);
+  planes3_any<T, N>(p, ib, blockIdx.x, col, ncols, z1, tbuf, smem_raw);
 }
 
 // Same result as k_planes3 with no block barrier after the w plane is transformed: each of

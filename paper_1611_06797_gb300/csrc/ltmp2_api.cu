@@ -998,9 +998,10 @@ int ltmp2_setup(const ltmp2_system *sys, ltmp2_ctx **out) {
   }
   Plan &p = c->p;
   p = hp.p;
-  // plane kernel: FP32, the warp-autonomous one (fastest on the 24^3 and 36^3 workloads);
-  // FP64, the block-synchronous one (FP64-issue bound either way, and 17 % faster)
-  p.plane_kernel = sys->precision == LTMP2_FP32 ? 3 : 2;
+  // plane kernel: FP64 has one; FP32 on lines up to 27, pairs of columns by blocks (24^3: 82.6 against
+  // 97.2 ms, 27^3: 50.5 against 54.4 ms per pass, 18^3 and 20^3: 5 to 25 % faster); longer lines hold
+  // too many registers in pairs, and the warp-autonomous kernel is 5 to 20 % faster
+  p.plane_kernel = sys->precision == LTMP2_FP32 && p.n > 27 ? 3 : 2;
   std::memcpy(c->lattice, sys->lattice, sizeof(c->lattice));
   c->ecut_aux = hp.ecut_aux;
   c->aux_g2 = hp.aux_g2;

@@ -29,7 +29,9 @@ template <typename F> static bool with_size(int n, F &&f) {
 // 2 = k_planes3 (product in registers, compact intermediate), 3 = k_planes4 (as 2, each
 // warp on its own occupied planes without block barriers).
 // ib = occupied planes per block (kernel 3: per warp step); 0 picks the default of each kernel.
-// FP64 has one plane kernel, 2 in fixed point: the others are accepted and run it.
+// FP64 has one plane kernel, 2 in fixed point: the others are accepted and run it.  In FP32 kernel 2
+// takes pairs of columns.
+template <typename T> static size_t plane_smem(const Plan &p, int kernel, int ib);
 template <typename T> static int plane_ib_default(const Plan &p, int kernel) {
   const int n = p.n;
   const size_t plane = (size_t)n * (n + 1) * sizeof(cpx<T>);
@@ -55,11 +57,18 @@ template <typename T> static int plane_ib_default(const Plan &p, int kernel) {
     ib = two > 0 && 1.15 * two * n / 64.0 >= three * n / 96.0 ? two : three;
     while (ib > 1 && plane + (sizeof(int) * p.n_daux + 64) + (size_t)ib * plane_stride(n, nxa) * sizeof(cpx<T>) > 100 * 1024) --ib;
   } else if (kernel == 2) {
-    // four planes per block: small blocks, many resident per SM (best on the 24^3 workload
-    // in both precisions among 2..16)
-    const size_t per = (size_t)n * nxa * sizeof(cpx<T>);
-    ib = (int)((100 * 1024 - plane - sizeof(int) * p.n_daux - 64) / per);
-    if (ib > 4) ib = 4;
+    // blocks of 64 threads: the fewest steps of 64 lines per occupied (x pass and y pass), weighed against
+    // the shared memory above what six blocks per SM (the registers' limit) have
+    ib = 1;
+    double best = 1e9;
+    for (int k = 1; k <= 8; ++k) {
+      const double steps = (double)((k * n + 63) / 64 + (k * nxa + 63) / 64) / k;
+      const double score = steps * std::max(1.0, (double)plane_smem<T>(p, 2, k) / 36864.0);
+      if (score < 0.99 * best) {
+        best = score;
+        ib = k;
+      }
+    }
   } else {
     const size_t per = plane + (size_t)p.n_daux * sizeof(cpx<T>);
     ib = (int)((100 * 1024 - plane - 3 * sizeof(int) * (n + 1) - 64) / per);
@@ -76,7 +85,7 @@ template <typename T> static size_t plane_smem(const Plan &p, int kernel, int ib
   const int nxa = p.mxhi_aux - p.mxlo_aux + 1;
   if (kernel == 0) return plane * (1 + ib);
   const size_t q = (size_t)plane_stride(n, nxa);
-  if (kernel == 2) return plane + (size_t)ib * q * sizeof(cpx<T>) + sizeof(int) * p.n_daux;
+  if (kernel == 2) return 16 * ((size_t)n * (n + 1) + (size_t)ib * q) + sizeof(int) * p.n_daux;
   if (kernel == 3) return plane + (size_t)kPlaneWarps * ib * q * sizeof(cpx<T>) + sizeof(int) * p.n_daux;
   return plane * (1 + ib) + (size_t)ib * p.n_daux * sizeof(cpx<T>) + 3 * sizeof(int) * nxa;
 }
@@ -86,12 +95,13 @@ template <typename T> static cudaError_t launch_planes(const Plan &p, int ncols,
   if (std::is_same<T, double>::value) {
     kernel = 2;
     if (ib > 256 / p.n) ib = 256 / p.n;   // registers: at most 256 threads of up to 255
-    while (ib > 1 && plane_smem<T>(p, kernel, ib) > 200 * 1024) --ib;
   }
   if (ib <= 0) ib = plane_ib_default<T>(p, kernel);
+  if (kernel == 2)
+    while (ib > 1 && plane_smem<T>(p, kernel, ib) > 200 * 1024) --ib;
   const size_t smem = plane_smem<T>(p, kernel, ib);
   int threads = kernel == 3 ? 32 * kPlaneWarps : ib * p.n;
-  if (threads < 64) threads = 64;
+  if (threads < 64 || (kernel == 2 && std::is_same<T, float>::value)) threads = 64;
   if (threads > 1024 || smem > 200 * 1024) return cudaErrorInvalidValue;
   if (!with_size(p.n, [&](auto n) { Sized<T, decltype(n)::value>::planes(p, ncols, kernel, ib, threads, smem, st); }))
     return cudaErrorInvalidValue;
@@ -102,7 +112,10 @@ template <typename T> bool Path<T>::plane_feasible(const Plan &p, int kernel, in
   if (kernel < 0 || kernel > 3 || ib < 0) return false;
   if (ib == 0) ib = plane_ib_default<T>(p, kernel);
   const int threads = kernel == 3 ? 32 * kPlaneWarps : ib * p.n;
-  return threads <= 1024 && plane_smem<T>(p, kernel, ib) <= 200 * 1024;
+  size_t smem = plane_smem<T>(p, kernel, ib);
+  // FP32 pairs: as many planes as fit unpaired are accepted, and a launch takes as many pairs as fit
+  if (kernel == 2 && std::is_same<T, float>::value) smem = smem / 2 + 2 * p.n_daux;
+  return threads <= 1024 && smem <= 200 * 1024;
 }
 
 template <typename T>

@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(kPersistThreads) k_planes_persist(const Plan *
     switch (p.n) {
 #define LTMP2_CASE(NN)                                                                                        \
   case NN:                                                                                                    \
-    planes3_any<T, NN>(p, sr.ib[e], z, col, p.z1, p.tbuf, smem_raw);                                         \
+    planes3_any<T, NN>(p, sr.ib[e], z, col, (sr.first[e + 1] - sr.first[e]) / NN, p.z1, p.tbuf, smem_raw);   \
     break;
       LTMP2_FOR_EACH_N(LTMP2_CASE)
 #undef LTMP2_CASE

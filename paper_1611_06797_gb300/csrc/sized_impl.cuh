@@ -43,7 +43,10 @@ void Sized<T, N>::planes(const Plan &p, int cols, int kernel, int ib, int thread
     else if (kernel == 1) k_planes2<T, N><<<grid, threads, smem, st>>>(p, ib, z1, tbuf);
     else if (kernel == 3) k_planes4<T, N><<<grid, threads, smem, st>>>(p, ib, z1, tbuf);
   }
-  if (kernel == 2) k_planes3<T, N><<<grid, threads, smem, st>>>(p, ib, p.z1, p.tbuf);
+  if (kernel == 2) {
+    const int cps = cols_per_slot(p), cols2 = std::is_same<T, double>::value ? cols : (cols / cps + 1) / 2 * cps;
+    k_planes3<T, N><<<dim3(N, cols2), threads, smem, st>>>(p, ib, cols, p.z1, p.tbuf);
+  }
 }
 
 template <typename T, int N>

@@ -37,3 +37,22 @@ def test_fixed_point_line_ffts_match_the_exact_dft(tmp_path):
     mean, worst, back = map(float, next(r for r in rows if r[0] == "mul")[1:])
     # rounding to nearest (half a unit) and the dropped product of the low halves (half a unit)
     assert worst < 1.01 and abs(mean) < 0.01 and back == 0
+
+
+def test_packed_line_ffts_match_the_dft(tmp_path):
+    """The FP32 transforms of two lines at once (csrc/pair.cuh), compiled for the host."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    exe = tmp_path / "fft_pair"
+    subprocess.run([nvcc, "-std=c++17", "--expt-relaxed-constexpr", "-O2",
+                    "-gencode", "arch=compute_103a,code=sm_103a",
+                    "-I", os.path.join(ROOT, "paper_1611_06797_gb300", "csrc"), "-x", "cu",
+                    os.path.join(ROOT, "tests", "native", "fft_pair.cu"), "-o", str(exe)],
+                   check=True, capture_output=True, timeout=600)
+    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True, timeout=120).stdout
+    rows = [line.split() for line in out.strip().splitlines()]
+    assert {int(r[0]) for r in rows} == {8, 10, 12, 16, 18, 20, 24, 25, 27, 30, 32, 36, 40} and len(rows) == 26
+    for n, d, err in rows:
+        # at most log2(n) butterfly stages of at most 4 roundings (2^-24 each) on a value
+        assert float(err) <= 4 * 2.0 ** -24 * int(n).bit_length(), (n, d, err)
