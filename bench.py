@@ -61,8 +61,8 @@ def measured_peaks():
 # Source files that define each stage's kernel, its launch configuration and the data it
 # reads: a stored DRAM measurement holds only while these are unchanged.
 STAGE_SOURCES = {
-    "plane_fft": ["kernels.cuh", "fft.cuh", "fixed.cuh", "plan.h", "path_impl.cuh", "sized_impl.cuh"],
-    "column_fft_contract": ["kernels.cuh", "fft.cuh", "fixed.cuh", "plan.h", "path_impl.cuh", "sized_impl.cuh"],
+    "plane_fft": ["kernels.cuh", "fft.cuh", "fixed.cuh", "pair.cuh", "plan.h", "path_impl.cuh", "sized_impl.cuh"],
+    "column_fft_contract": ["kernels.cuh", "fft.cuh", "fixed.cuh", "sym.cuh", "plan.h", "path_impl.cuh", "sized_impl.cuh"],
     "w_gemm": ["kernels.cuh", "plan.h", "path_impl.cuh", "tcgen05.cuh", "gemm_tc.cuh", "gemm_tc.cu",
                "gemm_f64tc.cuh", "gemm_f64tc.cu"],
 }
@@ -211,7 +211,7 @@ def oracle_check(cb, e_pair):
 
 
 # ------------------------------------------------------------------ cost model
-def stage_costs(sizes, n_prim, real, reps, nxa, nv_tau, w_virtual, n_v, green_full=False):
+def stage_costs(sizes, n_prim, real, reps, nxa, nv_tau, w_virtual, n_v, green_full=False, pairs_sym=False):
     """Algorithmic work of `reps` ltmp2_energy calls, by stage (flops).
 
     Real orbitals use the real cos/sin basis: the Green's function is a real product
@@ -222,7 +222,8 @@ def stage_costs(sizes, n_prim, real, reps, nxa, nv_tau, w_virtual, n_v, green_fu
     Green's function is built, else the Green's function sums over nv_tau[k] virtuals (all
     n_v on the tensor cores: green_full) and one product with it follows.  The plane FFT
     pass counts 5 n log2 n flops per line of n points: per (column, occupied i) it
-    transforms n rows and nxa columns (the aux m1 range) on each of the n planes."""
+    transforms n rows and nxa columns (the aux m1 range) on each of the n planes; with
+    pairs_sym (whole energies by the pairs' exchange symmetry) only for i <= j."""
     n_pw, n_occ, n = sizes["n_pw"], sizes["n_occ"], sizes["grid"]
     spp = 1 if real else 2
     ncols = n_prim * spp * n_occ
@@ -233,7 +234,8 @@ def stage_costs(sizes, n_prim, real, reps, nxa, nv_tau, w_virtual, n_v, green_fu
     return {
         "green_gemm": {"flops": reps * green},
         "w_gemm": {"flops": reps * wgemm},
-        "plane_fft": {"flops": reps * len(nv_tau) * ncols * n_occ * n * (n + nxa) * line},
+        "plane_fft": {"flops": reps * len(nv_tau) * ncols * (0.5 * (n_occ + 1) if pairs_sym else n_occ)
+                      * n * (n + nxa) * line},
     }
 
 
@@ -256,13 +258,16 @@ def _stage_bound(stage, st, costs, precision, simt, peaks, peak_kind, alu):
     if stage in costs:
         work = costs[stage]["flops"] / st[stage]["launches"]
         if not simt and (stage == "w_gemm" or (stage == "green_gemm" and precision == 0)):
-            # tensor products per real product: 3xTF32 in the precision form; in the FP64 path
-            # the 36 slice products (orders s + t < 8 of 8 x 7-bit slices per operand)
+            # counted as TF32-rate work, 3 products per FP32 product and 36 per FP64 product, so that
+            # the figures of earlier builds compare; the kernels form 10 (4 exact slices) and 36
+            # (8 exact slices) FP16 products, whose rate is the bf16 one
             work *= 3.0 if precision != 0 else 36.0
             peak = peaks["bf16_tflops"] * TF32_OVER_BF16
-            bound, pk = "tensor", f"tf32 = {peak_kind} bf16 {peaks['bf16_tflops']} x nominal 1.1/2.25"
+            bound, pk = "tensor", (f"tf32 = {peak_kind} bf16 {peaks['bf16_tflops']} x nominal 1.1/2.25; the products "
+                                   "are FP16 slices")
         elif precision == 0:
-            peak, bound, pk = alu["fp64"], "alu", "FP64 FMA rate " + alu["kind"]
+            peak, bound, pk = alu["fp64"], "alu", ("FP64 FMA rate " + alu["kind"] + "; the transforms run in 64-bit "
+                                                   "fixed point on the integer units, so this rate does not bound them")
         else:
             peak, bound, pk = alu["fp32"], "alu", "FP32 FMA rate " + alu["kind"]
         achieved = work / (per_launch_ms / 1e3) / 1e12
@@ -469,7 +474,7 @@ def main():
             b0, e0 = gprime_share(n_prim, rank, world)
             n_prim = e0 - b0
         costs = stage_costs(r["sizes"], n_prim, True, args.steps, aux_nxa(spec), r["nv_tau"], r["w_virtual"],
-                            s.n_orb - s.n_occ, r["green_full"])
+                            s.n_orb - s.n_occ, r["green_full"], pairs_sym=dist is None)
         return (roofline_of(r["stages"], costs, precision, simt, peaks, peak_kind, alu),
                 stage_rooflines(r["stages"], costs, precision, simt, peaks, peak_kind, alu))
 
@@ -497,8 +502,9 @@ def main():
                    "n_occ": sizes["n_occ"], "grid": sizes["grid"], "n_tau": n_tau, "pairs": pairs,
                    "form": "plain FP64" if primary == L.FP64 else "precision (FP32 FFT, split GEMM)",
                    "gemm": ("FP64-accurate products on tcgen05: rows scaled by powers of two, 8 exact 7-bit "
-                            "slices per operand, 36 slice products accumulated exactly in FP32 tensor memory, "
-                            "FP64 sums" if primary == L.FP64 else "tcgen05 3xTF32, FP32 sums per k block"),
+                            "slices per operand, 36 FP16 slice products accumulated exactly in FP32 tensor memory, "
+                            "integer sums" if primary == L.FP64 else "tcgen05, 4 exact 7-bit slices per operand, "
+                            "10 FP16 slice products, integer sums"),
                    "time_reversal": True, "l2": "flushed (256 MiB write) before every timed step",
                    "laplace_max_rel_err": qerr,
                    "parallelism": (f"outer G' loop split over {world} GPUs (contiguous balanced shares), one "
@@ -538,7 +544,7 @@ def main():
             "value": pairs * n_tau / (ms_o / 1e3), "s_per_E_MP2": ms_o / 1e3,
             "speedup_vs_fp64": (ms_step / ms_o) if other == L.FP32 else (ms_o / ms_step),
             "err_vs_fp64_meV_per_atom": err, "within_0.1_meV_per_atom": max(err.values()) <= 0.1,
-            "gemm": "tcgen05 3xTF32" if other == L.FP32 else "tcgen05, FP64-accurate exact slices",
+            "gemm": "tcgen05, FP32-accurate exact slices" if other == L.FP32 else "tcgen05, FP64-accurate exact slices",
             "roofline": ro_roof,
             "stage_rooflines": ro_stages,
             "stages": {k: {"ms_per_step": v["ms"] / args.steps} for k, v in so.items()},
@@ -798,7 +804,7 @@ def run_learned(args, local):
 
 def form_cfg3(L, torch, local, steps, warmup, alu=None):
     """Precision form on its own workload: 64 wells, 36^3 grid, 10059 plane waves, 128
-    occupied orbitals, 10 Laplace points (FP32 FFTs, 3xTF32 tcgen05 GEMM, FP64 sums).
+    occupied orbitals, 10 Laplace points (FP32 FFTs, exact-slice tcgen05 GEMM, FP64 sums).
     A full FP64 evaluation of this system takes about 45 minutes on one GB300, so the
     error against the FP64 path is measured on the same inputs over four spread ranges
     of the outer G' loop (ltmp2_energy_partial, 24 of 2724 primary G'), where both paths
@@ -848,7 +854,7 @@ def form_cfg3(L, torch, local, steps, warmup, alu=None):
     tuning = L.ltmp2_get_tuning(ctx)
     nv_tau, w_virtual = L.ltmp2_tau_virtuals(ctx, tau)
     costs = stage_costs(sizes, n_prim, True, steps, aux_nxa(spec), nv_tau, w_virtual, s.n_orb - s.n_occ,
-                        tuning["green_tc"] == 1)
+                        tuning["green_tc"] == 1, pairs_sym=True)
     roof = roofline_of(st, costs, L.FP32, False, peaks, peak_kind, alu)
     stage_roofs = stage_rooflines(st, costs, L.FP32, False, peaks, peak_kind, alu)
     # FP32 vs FP64 on the same inputs, over sampled G' ranges
@@ -879,7 +885,7 @@ def form_cfg3(L, torch, local, steps, warmup, alu=None):
         "data": "synthetic: seeded Gaussian-well model solid, orbitals from dense diagonalisation",
         "config": {"workload": _workload_desc(spec), "n_pw": sizes["n_pw"], "n_aux": sizes["n_aux"],
                    "n_occ": sizes["n_occ"], "grid": sizes["grid"], "n_tau": n_tau, "pairs": pairs,
-                   "form": "precision (FP32 FFT, 3xTF32 tcgen05 GEMM, FP64 sums)", "time_reversal": True,
+                   "form": "precision (FP32 FFT, exact-slice tcgen05 GEMM, FP64 sums)", "time_reversal": True,
                    "l2": "flushed (256 MiB write) before every timed step; inputs exceed L2",
                    "laplace_max_rel_err": qerr, "tuning": tuning},
         "energy": {"E_d": ed, "E_x": ex, "E": ed + ex, "meV_per_atom": (ed + ex) * per_atom},
@@ -1119,7 +1125,7 @@ def run_fftcmp(args, local):
             "shape": [rows, npw, npw], "cublas": "DGEMM" if prec == L.FP64 else "SGEMM (TF32 off)",
             "cublas_ms": ms, "cublas_tflops": 2.0 * rows * npw * npw / ms / 1e9,
             "ours_ms_per_launch": st["ms"] / max(1, st["launches"]),
-            "ours": "k_rgemm FP64 (SIMT)" if prec == L.FP64 else "tcgen05 3xTF32 (k_tc_cgemm_stacked + packing)"}
+            "ours": "tcgen05 exact slices (k_dgemm_oz + slicing)"}
         del A, B, C
     return out
 

@@ -446,7 +446,8 @@ int ltmp2_num_primary_gprime(const ltmp2_ctx *ctx);
 int ltmp2_sizes(const ltmp2_ctx *ctx, int *n_aux, int *n_pw, int *n_occ, int *grid_n);
 
 /* Imaginary residues of the last ltmp2_energy* call: the exact sums are real, so
- * these measure rounding (and, for LTMP2_FLAG_REAL_ORBITALS, the symmetry).       */
+ * these measure rounding (and, for LTMP2_FLAG_REAL_ORBITALS, the symmetry); 0 where a
+ * sum over (i, j) and (j, i) is taken as real.                                       */
 int ltmp2_last_imag(const ltmp2_ctx *ctx, double *im_direct, double *im_exchange);
 
 /* Per-stage device timing.  When enabled (on != 0), every later ltmp2_energy*
