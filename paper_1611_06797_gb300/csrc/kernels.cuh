@@ -698,11 +698,12 @@ __device__ __forceinline__ void planes3_body_pair(const Plan &p, int ib, int z, 
   }
 }
 
-// sum of v over the block's threads (blockDim.x a multiple of 32 or below 1024), in every thread
+// sum of v over the block's threads, in every thread.  blockDim.x is a multiple of 32: every lane of a
+// warp is read, and one that was not launched has no value.
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double red[32];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x / 32, nw = (blockDim.x + 31) / 32;
+  const int w = threadIdx.x / 32, nw = blockDim.x / 32;
   __syncthreads();
   if (threadIdx.x % 32 == 0) red[w] = v;
   __syncthreads();

@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "plane_block.h"
 #include "sized.h"
 #include "sym.cuh"
 
@@ -92,16 +93,15 @@ template <typename T> static size_t plane_smem(const Plan &p, int kernel, int ib
 
 // launch the plane kernel for the ncols columns of the current slab (z1 -> tbuf)
 template <typename T> static cudaError_t launch_planes(const Plan &p, int ncols, int kernel, int ib, cudaStream_t st) {
-  if (std::is_same<T, double>::value) {
-    kernel = 2;
-    if (ib > 256 / p.n) ib = 256 / p.n;   // registers: at most 256 threads of up to 255
-  }
+  constexpr bool kFp64 = std::is_same<T, double>::value;
+  if (kFp64) kernel = 2;
   if (ib <= 0) ib = plane_ib_default<T>(p, kernel);
+  if (kFp64) ib = plane_block_f64(p.n, ib).ib;
   if (kernel == 2)
     while (ib > 1 && plane_smem<T>(p, kernel, ib) > 200 * 1024) --ib;
   const size_t smem = plane_smem<T>(p, kernel, ib);
-  int threads = kernel == 3 ? 32 * kPlaneWarps : ib * p.n;
-  if (threads < 64 || (kernel == 2 && std::is_same<T, float>::value)) threads = 64;
+  int threads = kernel == 3 ? 32 * kPlaneWarps : kFp64 ? plane_block_f64(p.n, ib).threads : ib * p.n;
+  if (threads < 64 || (kernel == 2 && !kFp64)) threads = 64;
   if (threads > 1024 || smem > 200 * 1024) return cudaErrorInvalidValue;
   if (!with_size(p.n, [&](auto n) { Sized<T, decltype(n)::value>::planes(p, ncols, kernel, ib, threads, smem, st); }))
     return cudaErrorInvalidValue;
