@@ -218,7 +218,8 @@ typedef struct ltmp2_batch ltmp2_batch; /* opaque; a captured, instantiated grap
 /* Capture the full energy evaluation of n distinct contexts (each with its own
  * quadrature: n_tau[i], tau[i][*], w[i][*], host arrays copied into the graph) into one
  * CUDA graph.  The contexts must stay alive, on one device and with unchanged slab /
- * tuning settings, until ltmp2_batch_destroy.  Nothing runs yet.
+ * tuning settings, until ltmp2_batch_destroy; the cutoff levels may change (the batch
+ * keeps those of its creation).  Nothing runs yet.
  * Errors: INVALID_ARG (NULL, duplicate ctx, bad tau), OOM, CUDA.                     */
 int ltmp2_batch_create(ltmp2_ctx *const *ctxs, int n, const int *n_tau, const double *const *tau,
                        const double *const *w, ltmp2_batch **out);

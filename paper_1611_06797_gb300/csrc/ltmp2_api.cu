@@ -724,6 +724,9 @@ struct ltmp2_batch {
   int device = 0;
   bool persistent = false;        // shared persistent FFT stages per round (else one branch per system)
   void *d_plans = nullptr;        // persistent mode: the systems' plans on the device
+  // branches: the graph's own copies of the tables that ltmp2_set_extrapolation rewrites (a captured
+  // launch has their sizes fixed)
+  std::vector<void *> tables;
   int *d_counters = nullptr;      // persistent mode: the two work-queue counters
   std::vector<ltmp2_ctx *> ctxs;
   std::vector<long long> launches;
@@ -735,6 +738,7 @@ struct ltmp2_batch {
   ~ltmp2_batch() {
     cudaFree(d_plans);
     cudaFree(d_counters);
+    for (void *t : tables) cudaFree(t);
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
     for (auto e : events) cudaEventDestroy(e);
@@ -809,6 +813,29 @@ int pair_descriptors(ltmp2_ctx *ctx, double *desc) {
       f[7] = dist / (spread[i] + spread[j] + 1e-3);
     }
   return LTMP2_OK;
+}
+}  // namespace
+
+// A captured branch's plan: the context's, with the row groups of the symmetric passes and the level
+// tables as they are now in the batch's own memory
+namespace {
+int own_tables(ltmp2_batch *b, Plan &p) {
+  auto copy = [&](auto *&ptr, size_t count) {
+    void *t = nullptr;
+    const size_t bytes = count * sizeof(*ptr);
+    if (cudaMalloc(&t, bytes) != cudaSuccess) return LTMP2_ERR_OOM;
+    b->tables.push_back(t);
+    const int rc = cuda_status(cudaMemcpy(t, ptr, bytes, cudaMemcpyDeviceToDevice));
+    ptr = static_cast<typename std::remove_reference<decltype(ptr)>::type>(t);
+    return rc;
+  };
+  int rc = LTMP2_OK;
+  if (use_sym(p)) rc = copy(p.sym_groups, (size_t)p.n_groups);
+  if (!rc && p.n_lev > 1) rc = copy(p.aux_lev, (size_t)p.n_aux);
+  if (!rc && p.n_lev > 1) rc = copy(p.lev_order, (size_t)p.n_aux);
+  if (!rc && p.n_lev > 1) rc = copy(p.lev_start, (size_t)p.n_lev + 1);
+  if (!rc) rc = cuda_status(cudaStreamSynchronize(nullptr));   // device copies return before they are done
+  return rc;
 }
 }  // namespace
 
@@ -1430,7 +1457,17 @@ int ltmp2_batch_create(ltmp2_ctx *const *ctxs, int n, const int *n_tau, const do
     *out = b;
     return LTMP2_OK;
   }
+  std::vector<Plan> plans(n);
+  for (int i = 0; i < n; ++i) {
+    plans[i] = ctxs[i]->p;
+    if (const int trc = own_tables(b, plans[i])) return fail(trc);
+  }
+  // the capture records the batch's tables in place of the contexts'
+  auto swap_plans = [&] {
+    for (int i = 0; i < n; ++i) std::swap(ctxs[i]->p, plans[i]);
+  };
   if (cudaStreamBeginCapture(b->origin, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return fail(LTMP2_ERR_CUDA);
+  swap_plans();
   int rc = cuda_status(cudaEventRecord(b->events[n], b->origin));
   for (int i = 0; i < n && !rc; ++i) {
     ltmp2_ctx *c = ctxs[i];
@@ -1444,6 +1481,7 @@ int ltmp2_batch_create(ltmp2_ctx *const *ctxs, int n, const int *n_tau, const do
     if (!rc) rc = cuda_status(cudaEventRecord(b->events[i], b->streams[i]));
     if (!rc) rc = cuda_status(cudaStreamWaitEvent(b->origin, b->events[i], 0));
   }
+  swap_plans();
   const cudaError_t ec = cudaStreamEndCapture(b->origin, &b->graph);
   if (rc) return fail(rc);
   if (ec != cudaSuccess) return fail(LTMP2_ERR_CUDA);
