@@ -5,11 +5,11 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "../../include/ltmp2.h"
 #include "fft.cuh"
 #include "gemm_f64tc.cuh"
+#include "once_device.h"
 #include "plan.h"
 
 namespace ltmp2 {
@@ -39,14 +39,16 @@ template <typename T> cudaError_t attributes_of() {
   return e;
 }
 
+// of the current device: a function's attributes belong to one device
 cudaError_t set_attributes() {
-  static std::once_flag once;
-  static cudaError_t e = cudaSuccess;
-  std::call_once(once, [] {
-    e = attributes_of<double>();
-    if (e == cudaSuccess) e = attributes_of<float>();
+  static OncePerDevice once;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return once.run(dev, [] {
+    const cudaError_t a = attributes_of<double>();
+    return a == cudaSuccess ? attributes_of<float>() : a;
   });
-  return e;
 }
 
 // persistent blocks for `tiles` output tiles: one per SM
