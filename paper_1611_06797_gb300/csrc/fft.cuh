@@ -13,6 +13,8 @@
 #include <cuda_runtime.h>
 #include <cmath>
 
+#include "once_device.h"
+
 namespace ltmp2 {
 
 // Aligned to its full size, so that a complex value moves as one 64-bit (float) or 128-bit
@@ -64,9 +66,7 @@ static __constant__ float2 c_tw32[kTwTotal];
 inline double2 h_tw64[kTwTotal];
 inline float2 h_tw32[kTwTotal];
 
-inline void fill_host_twiddles() {
-  static bool done = false;
-  if (done) return;
+inline void compute_host_twiddles() {
   const double two_pi = 6.283185307179586476925286766559;
   int off = 0;
   for (int s = 0; s < kNumFftSizes; ++s) {
@@ -87,7 +87,11 @@ inline void fill_host_twiddles() {
     }
     off += n;
   }
-  done = true;
+}
+// once per process, from any thread
+inline void fill_host_twiddles() {
+  static const bool done = (compute_host_twiddles(), true);
+  (void)done;
 }
 
 static inline cudaError_t upload_twiddles() {
@@ -97,15 +101,12 @@ static inline cudaError_t upload_twiddles() {
   return cudaMemcpyToSymbol(c_tw32, h_tw32, sizeof(h_tw32));
 }
 
-// the same, once per device in each translation unit (the callers serialise)
+// the same, once per device in each translation unit, from any thread
 static inline cudaError_t upload_twiddles_once() {
-  static bool done[64] = {false};
+  static OncePerDevice once;
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess || (dev < 64 && done[dev])) return e;
-  e = upload_twiddles();
-  if (e == cudaSuccess && dev < 64) done[dev] = true;
-  return e;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e == cudaSuccess ? once.run(dev, [] { return upload_twiddles(); }) : e;
 }
 
 template <typename T> struct TwTable;

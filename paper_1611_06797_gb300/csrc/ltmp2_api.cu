@@ -861,11 +861,11 @@ int capture_rounds(ltmp2_batch *b, ltmp2_ctx *const *ctxs, int n, const int *n_t
     rounds[i] = n_tau[i] * nslab[i];
     rmax = std::max(rmax, rounds[i]);
   }
-  if (smem_p > 200 * 1024 || smem_c > 200 * 1024) return LTMP2_ERR_UNSUPPORTED;
+  if (smem_p > kPersistSmem || smem_c > kPersistSmem) return LTMP2_ERR_UNSUPPORTED;
   if (cudaMalloc(&b->d_plans, sizeof(Plan) * n) != cudaSuccess || cudaMalloc(&b->d_counters, 2 * sizeof(int)) != cudaSuccess)
     return LTMP2_ERR_OOM;
   int rc = cuda_status(cudaMemcpy(b->d_plans, plans.data(), sizeof(Plan) * n, cudaMemcpyHostToDevice));
-  if (!rc) rc = cuda_status(Path<T>::persist_attributes(smem_p, smem_c));
+  if (!rc) rc = cuda_status(Path<T>::persist_attributes());
   const int blocks_p = Path<T>::persist_blocks(true, smem_p), blocks_c = Path<T>::persist_blocks(false, smem_c);
   if (!rc && (blocks_p < 1 || blocks_c < 1)) rc = LTMP2_ERR_CUDA;
   if (rc) return rc;

@@ -2,10 +2,10 @@
 // kernels_f64.cu / kernels_f32.cu, which explicitly instantiate Path<T>.
 #pragma once
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "once_device.h"
 #include "plane_block.h"
 #include "sized.h"
 #include "sym.cuh"
@@ -131,20 +131,17 @@ struct ScopedStage {
 };
 
 template <typename T> cudaError_t Path<T>::init_device() {
-  // once per device and process; contexts set up from several host threads serialise here
-  static bool done[64] = {false};
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
+  static OncePerDevice once;
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  const cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev < 64 && done[dev]) return cudaSuccess;
   // twiddle tables and dynamic shared memory limits of the FFT kernels
-  for (int n : kFftSizes)
-    if (e == cudaSuccess) with_size(n, [&](auto c) { e = Sized<T, decltype(c)::value>::init(); });
-  if (e != cudaSuccess) return e;
-  if (dev < 64) done[dev] = true;
-  return cudaSuccess;
+  return once.run(dev, [] {
+    cudaError_t r = cudaSuccess;
+    for (int n : kFftSizes)
+      if (r == cudaSuccess) with_size(n, [&](auto c) { r = Sized<T, decltype(c)::value>::init(); });
+    return r;
+  });
 }
 
 template <typename T>
@@ -550,11 +547,9 @@ cudaError_t Path<T>::slab_k(const Plan &p, int gp0, int np, double coef, cudaStr
 
 template <typename T> size_t Path<T>::plane_smem_for(const Plan &p, int ib) { return plane_smem<T>(p, 2, ib); }
 
-template <typename T> cudaError_t Path<T>::persist_attributes(size_t plane_smem_b, size_t col_smem_b) {
+template <typename T> cudaError_t Path<T>::persist_attributes() {
   cudaError_t e = PersistPlanes<T>::init();
   if (e == cudaSuccess) e = PersistColumns<T>::init();
-  if (e == cudaSuccess) e = PersistPlanes<T>::attributes(plane_smem_b);
-  if (e == cudaSuccess) e = PersistColumns<T>::attributes(col_smem_b);
   return e;
 }
 

@@ -45,9 +45,9 @@ __global__ void __launch_bounds__(kPersistThreads) k_planes_persist(const Plan *
   }
 }
 
-template <typename T> cudaError_t PersistPlanes<T>::init() { return upload_twiddles_once(); }
-template <typename T> cudaError_t PersistPlanes<T>::attributes(size_t smem) {
-  return cudaFuncSetAttribute(k_planes_persist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename T> cudaError_t PersistPlanes<T>::init() {
+  const cudaError_t e = upload_twiddles_once();
+  return e == cudaSuccess ? cudaFuncSetAttribute(k_planes_persist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPersistSmem) : e;
 }
 template <typename T> int PersistPlanes<T>::blocks_per_sm(size_t smem) {
   int per = 0;
@@ -95,9 +95,9 @@ __global__ void __launch_bounds__(kPersistThreads) k_zcol_persist(const Plan *__
   }
 }
 
-template <typename T> cudaError_t PersistColumns<T>::init() { return upload_twiddles_once(); }
-template <typename T> cudaError_t PersistColumns<T>::attributes(size_t smem) {
-  return cudaFuncSetAttribute(k_zcol_persist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename T> cudaError_t PersistColumns<T>::init() {
+  const cudaError_t e = upload_twiddles_once();
+  return e == cudaSuccess ? cudaFuncSetAttribute(k_zcol_persist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPersistSmem) : e;
 }
 template <typename T> int PersistColumns<T>::blocks_per_sm(size_t smem) {
   int per = 0;

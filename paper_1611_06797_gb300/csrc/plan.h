@@ -227,6 +227,7 @@ constexpr int kMaxLevels = 16;   // nested cutoffs of the internal extrapolation
 // (plane items: N planes x columns; column items: pairs) and their slab.
 constexpr int kBatchMax = 16;
 constexpr int kPersistThreads = 128;
+constexpr int kPersistSmem = 200 * 1024;   // shared memory of the persistent kernels, at most
 struct BatchRound {
   int nsys = 0;
   int first[kBatchMax + 1] = {0};   // item prefix over the active systems
@@ -287,7 +288,7 @@ template <typename T> struct Path {
   static cudaError_t zcol_persist(const Plan *d_plans, const struct BatchRound &r, int *counter, int blocks,
                                   size_t smem, cudaStream_t st);
   static size_t plane_smem_for(const Plan &p, int ib);
-  static cudaError_t persist_attributes(size_t plane_smem, size_t col_smem);
+  static cudaError_t persist_attributes();
   static int persist_blocks(bool planes, size_t smem);
   // plane kernel `kernel` with `ib` occupied planes per block fits the launch limits
   static bool plane_feasible(const Plan &p, int kernel, int ib);

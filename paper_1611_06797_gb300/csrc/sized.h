@@ -23,16 +23,15 @@ template <typename T, int N> struct Sized {
   static void zcol_k(const Plan &p, int gp0, int np, int npairs, int threads, size_t smem, cudaStream_t st);
 };
 
-// persistent kernels of the batching form: shared-memory limit, blocks per SM, launch
+// persistent kernels of the batching form: twiddle tables and shared-memory limit, blocks per SM, launch.
+// The limit is the same for every batch: several threads may create batches of different sizes.
 template <typename T> struct PersistPlanes {
   static cudaError_t init();
-  static cudaError_t attributes(size_t smem);
   static int blocks_per_sm(size_t smem);
   static void launch(const Plan *d_plans, const BatchRound &r, int *counter, int blocks, size_t smem, cudaStream_t st);
 };
 template <typename T> struct PersistColumns {
   static cudaError_t init();
-  static cudaError_t attributes(size_t smem);
   static int blocks_per_sm(size_t smem);
   static void launch(const Plan *d_plans, const BatchRound &r, int *counter, int blocks, size_t smem, cudaStream_t st);
 };
