@@ -181,12 +181,12 @@ int ltmp2_set_slab_size(ltmp2_ctx *ctx, int n);
  * system's direct term and accumulation.  Otherwise every system is one graph branch.
  * FP64 energies equal ltmp2_energy's to rounding of the summation order.              */
 
-/* Autotuner: times one slab of the path for each candidate (slab sizes down from the
- * setup capacity; in LTMP2_FP32 also the two tensor-core GEMM layouts) and keeps the
- * fastest per primary G', then the plane FFT kernel and its block shape.  The choice is cached per (grid, n_pw, n_occ, |A|, precision,
- * real-orbital flag) for the process and applied to ctx.  slab, gemm_variant: NULL or
- * receive the choice (gemm_variant = -1 in LTMP2_FP64).  Errors: INVALID_ARG, CUDA,
- * TIMEOUT.                                                                          */
+/* Autotuner: times a slab's work on the path that ltmp2_energy takes for each slab size
+ * down from the setup capacity and keeps the fastest per column, then the plane FFT
+ * kernel and its block shape; set-up's own choices stay unless another is 5 % (2 %) faster.
+ * The choice is cached per (grid, n_pw, n_occ, |A|, precision, real-orbital flag) for the
+ * process and applied to ctx.  slab, gemm_variant: NULL or receive the choice
+ * (gemm_variant = -1 in LTMP2_FP64, else 5).  Errors: INVALID_ARG, CUDA, TIMEOUT.      */
 int ltmp2_autotune(ltmp2_ctx *ctx, int *slab, int *gemm_variant);
 
 /* Settings in effect for ctx: values[0] slab size, [1] tensor-core GEMM layout (5, or 4 for general orbitals; one kernel serves both; -1 in

@@ -294,6 +294,10 @@ int setup_sym(ltmp2_ctx *c, const std::vector<int> &prim, const std::vector<int>
   c->sym_order = order;
   return set_sym_rows(c, nullptr);
 }
+// Plane kernel of a set-up: FP64 has one; FP32 on lines up to 27, pairs of columns by blocks (24^3: 82.6
+// against 97.2 ms, 27^3: 50.5 against 54.4 ms per pass, 18^3 and 20^3: 5 to 25 % faster); longer lines
+// hold too many registers in pairs, and the warp-autonomous kernel is 5 to 20 % faster
+int default_plane_kernel(const Plan &p) { return p.precision == LTMP2_FP32 && p.n > 27 ? 3 : 2; }
 // every G' at the Gamma point, by the Green's-function route
 bool use_sym(const Plan &p) { return p.msym && p.nk == 0 && p.route == 0; }
 
@@ -608,8 +612,9 @@ int energy_common(ltmp2_ctx *ctx, int n_tau, const double *tau, const double *w,
 
 
 // ---------------------------------------------------------------- autotuner
-// Slab size (primary G' per pass) and tensor-core GEMM variant, chosen by timing one
-// slab per candidate; cached per (grid, N_pw, N_occ, |A|, precision, real) bucket.
+// Slab size (primary G' per pass), chosen by timing, per candidate, one symmetric pass where whole
+// energies go by them, else one slab; then the plane kernel and its block, chosen by timing the
+// plane pass alone; cached per (grid, N_pw, N_occ, |A|, precision, real) bucket.
 struct TuneKey {
   int n, n_pw, n_occ, n_aux, precision, real;
   bool operator<(const TuneKey &o) const {
@@ -648,69 +653,81 @@ template <typename T> int tune_ctx(ltmp2_ctx *c, int *slab_out, int *var_out) {
   }
   std::vector<int> slabs;
   for (int sl = std::min(c->slab_capacity, p.n_prim); sl >= 1 && slabs.size() < 4; sl /= 2) slabs.push_back(sl);
-  const std::vector<int> variants{p.tc ? 5 : -1};
+  const int variant = p.tc ? 5 : -1;
+  const bool sym = use_sym(p);
   cudaEvent_t a = nullptr, b = nullptr;
   if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return LTMP2_ERR_CUDA;
   double best = 1e300;
-  int best_slab = slabs.front(), best_var = variants.front();
-  int rc = LTMP2_OK;
-  for (int v : variants) {
-    if ((rc = apply_tuning(c, slabs.front(), v, p.plane_kernel, p.plane_ib))) break;
-    if (Path<T>::green(p, 1.0, c->stream, nullptr) != cudaSuccess) { rc = LTMP2_ERR_CUDA; break; }
-    for (int sl : slabs) {
-      p.max_prim = sl;
-      // one untimed pass, then two timed ones (weight 0: accumulators unchanged)
-      for (int rep = 0; rep < 3 && !rc; ++rep) {
-        if (rep == 1) cudaEventRecord(a, c->stream);
-        if (Path<T>::slab(p, 0, sl, 0.0, c->stream, nullptr) != cudaSuccess) rc = LTMP2_ERR_CUDA;
+  int best_slab = slabs.front();
+  int rc = apply_tuning(c, slabs.front(), variant, p.plane_kernel, p.plane_ib);
+  if (!rc && Path<T>::green(p, 1.0, c->stream, nullptr) != cudaSuccess) rc = LTMP2_ERR_CUDA;
+  for (int sl : slabs) {
+    if (rc) break;
+    p.max_prim = sl;
+    double work = sl;
+    // one untimed pass, then two timed ones (weight 0: accumulators unchanged)
+    for (int rep = 0; rep < 3 && !rc; ++rep) {
+      if (rep == 1) cudaEventRecord(a, c->stream);
+      const cudaError_t e = sym ? Path<T>::sym_probe(p, c->stream, &work) : Path<T>::slab(p, 0, sl, 0.0, c->stream, nullptr);
+      if (e != cudaSuccess) rc = LTMP2_ERR_CUDA;
+    }
+    if (rc) break;
+    cudaEventRecord(b, c->stream);
+    if (cudaEventSynchronize(b) != cudaSuccess) { rc = LTMP2_ERR_CUDA; break; }
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, a, b);
+    // set-up's slab, the first, unless another is 5 % faster: one pass at one Laplace point stands for a
+    // whole energy (at 2 %, 27^3 in FP64 took half the slab and 1 % more time)
+    if (ms / work < (best_slab == slabs.front() ? 0.95 : 1.0) * best) { best = ms / work; best_slab = sl; }
+  }
+  // plane kernel and its block size, timed alone on the columns of one warm slab: set-up's choice
+  // first, which another has to beat by 2 % (the timings' scatter), then per kernel its default block
+  // and others.  (20^3 in FP64: 9.9 ms with the default of 3 planes, 11.8 ms with the best of 2, 4, 8, 16.)
+  const int def_pk = default_plane_kernel(p);
+  int best_pk = def_pk, best_ib = 0;
+  if (!rc) rc = apply_tuning(c, best_slab, variant, p.plane_kernel, p.plane_ib);
+  if (!rc && Path<T>::slab(p, 0, best_slab, 0.0, c->stream, nullptr) != cudaSuccess) rc = LTMP2_ERR_CUDA;
+  if (!rc) {
+    const int ncols = best_slab * p.slots_per_prim() * p.n_occ;
+    constexpr bool kFp64 = std::is_same<T, double>::value;
+    std::vector<std::pair<int, int>> shapes{{def_pk, 0}};
+    static const int kIbs[2][4] = {{2, 4, 8, 16}, {1, 2, 3, 4}};   // planes per block; kernel 3: per warp step
+    for (int pk = kFp64 ? 2 : 0; pk < (kFp64 ? 3 : 4); ++pk) {   // FP64 has one plane kernel
+      if (pk != def_pk) shapes.emplace_back(pk, 0);
+      for (int ib : kIbs[pk == 3 ? 1 : 0])
+        if (ib <= p.n_occ) shapes.emplace_back(pk, ib);
+    }
+    double best_plane = 1e300;
+    for (const auto &sh : shapes) {
+      if (Path<T>::plane_pass(p, ncols, sh.first, sh.second, c->stream) != cudaSuccess) {  // infeasible shape
+        cudaGetLastError();
+        continue;
       }
-      if (rc) break;
+      cudaEventRecord(a, c->stream);
+      for (int rep = 0; rep < 2; ++rep) Path<T>::plane_pass(p, ncols, sh.first, sh.second, c->stream);
       cudaEventRecord(b, c->stream);
       if (cudaEventSynchronize(b) != cudaSuccess) { rc = LTMP2_ERR_CUDA; break; }
       float ms = 0.f;
       cudaEventElapsedTime(&ms, a, b);
-      const double per_prim = ms / (2.0 * sl);
-      if (per_prim < best) { best = per_prim; best_slab = sl; best_var = v; }
-    }
-    if (rc) break;
-  }
-  // plane kernel and its block size, timed alone on the columns of one warm slab
-  int best_pk = 0, best_ib = 0;
-  if (!rc) rc = apply_tuning(c, best_slab, best_var, p.plane_kernel, p.plane_ib);
-  if (!rc && Path<T>::slab(p, 0, best_slab, 0.0, c->stream, nullptr) != cudaSuccess) rc = LTMP2_ERR_CUDA;
-  if (!rc) {
-    const int ncols = best_slab * p.slots_per_prim() * p.n_occ;
-    double best_plane = 1e300;
-    static const int kIbs[2][4] = {{2, 4, 8, 16}, {1, 2, 3, 4}};   // planes per block; kernel 3: per warp step
-    // FP64 has one plane kernel
-    for (int pk = std::is_same<T, double>::value ? 2 : 0; pk < (std::is_same<T, double>::value ? 3 : 4) && !rc; ++pk)
-      for (int ibk = 0; ibk < 4; ++ibk) {
-        const int ib = kIbs[pk == 3 ? 1 : 0][ibk];
-        if (ib > p.n_occ) continue;
-        if (Path<T>::plane_pass(p, ncols, pk, ib, c->stream) != cudaSuccess) {  // infeasible shape
-          cudaGetLastError();
-          continue;
-        }
-        cudaEventRecord(a, c->stream);
-        for (int rep = 0; rep < 2; ++rep) Path<T>::plane_pass(p, ncols, pk, ib, c->stream);
-        cudaEventRecord(b, c->stream);
-        if (cudaEventSynchronize(b) != cudaSuccess) { rc = LTMP2_ERR_CUDA; break; }
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, a, b);
-        if (ms < best_plane) { best_plane = ms; best_pk = pk; best_ib = ib; }
+      const bool from_default = best_pk == def_pk && best_ib == 0;
+      if (ms < (from_default ? 0.98 : 1.0) * best_plane) {
+        best_plane = ms;
+        best_pk = sh.first;
+        best_ib = sh.second;
       }
+    }
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
   if (!rc) rc = check_tc_flag(c);
-  if (!rc) rc = apply_tuning(c, best_slab, best_var, best_pk, best_ib);
+  if (!rc) rc = apply_tuning(c, best_slab, variant, best_pk, best_ib);
   if (rc) return rc;
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
-    g_tune_cache[key] = {best_slab, best_var, best_pk, best_ib};
+    g_tune_cache[key] = {best_slab, variant, best_pk, best_ib};
   }
   *slab_out = best_slab;
-  *var_out = p.tc ? best_var : -1;
+  *var_out = variant;
   return LTMP2_OK;
 }
 
@@ -1025,10 +1042,7 @@ int ltmp2_setup(const ltmp2_system *sys, ltmp2_ctx **out) {
   }
   Plan &p = c->p;
   p = hp.p;
-  // plane kernel: FP64 has one; FP32 on lines up to 27, pairs of columns by blocks (24^3: 82.6 against
-  // 97.2 ms, 27^3: 50.5 against 54.4 ms per pass, 18^3 and 20^3: 5 to 25 % faster); longer lines hold
-  // too many registers in pairs, and the warp-autonomous kernel is 5 to 20 % faster
-  p.plane_kernel = sys->precision == LTMP2_FP32 && p.n > 27 ? 3 : 2;
+  p.plane_kernel = default_plane_kernel(p);
   std::memcpy(c->lattice, sys->lattice, sizeof(c->lattice));
   c->ecut_aux = hp.ecut_aux;
   c->aux_g2 = hp.aux_g2;

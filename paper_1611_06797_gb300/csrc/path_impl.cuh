@@ -400,43 +400,70 @@ cudaError_t Path<T>::slab_post(const Plan &p, int gp0, int np, double coef, cuda
 // pair slots of a pass over sym_nj orbitals from sym_j0
 static int sym_pairs(const Plan &p) { return p.sym_nj * p.sym_j0 + p.sym_nj * (p.sym_nj + 1) / 2; }
 
+// orbitals per pass and G' per part of it: columns as of a slab; whole orbitals j if they fit, else one j
+// in several parts
+static void sym_shape(const Plan &p, int &nj, int &np_max) {
+  const int budget = p.max_prim * p.slots_per_prim() * p.n_occ;
+  nj = std::max(1, std::min(std::min(budget / p.n_idx, p.n_occ), p.sym_nj_cap));
+  np_max = std::max(1, std::min(p.n_idx, budget / nj));
+}
+
+// The pass of orbitals p.sym_j0 .. + p.sym_nj in parts of np_max G': its matrices S_ij and the rows of the
+// exchange sums
+template <typename T>
+static cudaError_t sym_pass(const Plan &p, int np_max, cudaStream_t st, StageTimer *tm, long long *launches) {
+  const int n_idx = p.n_idx, threads = std::min(256, ((p.n_daux + 31) / 32) * 32);
+  const size_t smem = (size_t)p.sym_planes * n_idx * sizeof(cpx<T>);
+  cudaError_t e;
+  for (int g0 = 0; g0 < n_idx; g0 += np_max) {
+    const int np = std::min(np_max, n_idx - g0), ncols = np * p.sym_nj;
+    if ((e = Path<T>::slab_pre(p, g0, np, st, tm)) != cudaSuccess) return e;
+    {
+      ScopedStage s(tm, kStagePlane);
+      if ((e = launch_planes<T>(p, ncols, p.plane_kernel, p.plane_ib, st)) != cudaSuccess) return e;
+    }
+    {
+      ScopedStage s(tm, kStageColumn);
+      if (!with_size(p.n, [&](auto c) { Sized<T, decltype(c)::value>::zsym(p, g0, ncols, threads, smem, st); }))
+        return cudaErrorInvalidValue;
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    *launches += Path<T>::pre_launches(p) + 2;
+  }
+  ScopedStage s(tm, kStageColumn);
+  k_xsym<T><<<dim3(sym_pairs(p), (n_idx + 31) / 32), 256, 0, st>>>(p, p.sym_rows);
+  *launches += 1;
+  return cudaGetLastError();
+}
+
+template <typename T> cudaError_t Path<T>::sym_probe(const Plan &p0, cudaStream_t st, double *columns) {
+  Plan p = p0;
+  p.prim = p.sym_order;
+  int np_max = 0;
+  sym_shape(p, p.sym_nj, np_max);
+  // the middle orbitals: a column has the items of an energy's mean column, or half an item more
+  p.sym_j0 = (p.n_occ - p.sym_nj + 1) / 2;
+  *columns = (double)p.n_idx * p.sym_nj;
+  long long launches = 0;
+  return sym_pass<T>(p, np_max, st, nullptr, &launches);
+}
+
 template <typename T>
 cudaError_t Path<T>::sym_tau(const Plan &p0, double coef, cudaStream_t st, StageTimer *tm, long long *launches) {
   Plan p = p0;
   p.prim = p.sym_order;   // the slots of a pass: every G' of the index set, in its order
-  const int n_idx = p.n_idx, no = p.n_occ;
-  // columns per pass as of a slab; whole orbitals j if they fit, else one j in several parts
-  const int budget = p.max_prim * p.slots_per_prim() * no;
-  const int nj = std::max(1, std::min(std::min(budget / n_idx, no), p.sym_nj_cap));
-  const int np_max = std::max(1, std::min(n_idx, budget / nj));
-  const size_t smem = (size_t)p.sym_planes * n_idx * sizeof(cpx<T>);
-  const int threads = std::min(256, ((p.n_daux + 31) / 32) * 32);
+  const int no = p.n_occ;
+  int nj, np_max;
+  sym_shape(p, nj, np_max);
   cudaError_t e;
   for (p.sym_j0 = 0; p.sym_j0 < no; p.sym_j0 += nj) {
     p.sym_nj = std::min(nj, no - p.sym_j0);
-    for (int g0 = 0; g0 < n_idx; g0 += np_max) {
-      const int np = std::min(np_max, n_idx - g0), ncols = np * p.sym_nj;
-      if ((e = slab_pre(p, g0, np, st, tm)) != cudaSuccess) return e;
-      {
-        ScopedStage s(tm, kStagePlane);
-        if ((e = launch_planes<T>(p, ncols, p.plane_kernel, p.plane_ib, st)) != cudaSuccess) return e;
-      }
-      {
-        ScopedStage s(tm, kStageColumn);
-        if (!with_size(p.n, [&](auto c) { Sized<T, decltype(c)::value>::zsym(p, g0, ncols, threads, smem, st); }))
-          return cudaErrorInvalidValue;
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      }
-      *launches += pre_launches(p) + 2;
-    }
+    if ((e = sym_pass<T>(p, np_max, st, tm, launches)) != cudaSuccess) return e;
     ScopedStage s(tm, kStageColumn);
-    const int pairs = sym_pairs(p);
-    k_xsym<T><<<dim3(pairs, (n_idx + 31) / 32), 256, 0, st>>>(p, p.sym_rows);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // real orbitals: the rows are the primary G', each standing for -G' too
-    k_xsym_sum<T><<<pairs, 128, 0, st>>>(p, p.sym_rows, (p.real_orb ? 2.0 : 1.0) * coef);
+    k_xsym_sum<T><<<sym_pairs(p), 128, 0, st>>>(p, p.sym_rows, (p.real_orb ? 2.0 : 1.0) * coef);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    *launches += 2;
+    *launches += 1;
   }
   {
     ScopedStage s(tm, kStageDirect);

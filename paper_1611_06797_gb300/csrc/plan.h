@@ -275,6 +275,9 @@ template <typename T> struct Path {
                           StageTimer *tm);
   // one tau of a whole energy by the pairs' symmetry: every G', exchange and direct sums
   static cudaError_t sym_tau(const Plan &p, double coef, cudaStream_t st, StageTimer *tm, long long *launches);
+  // one symmetric pass at the middle orbitals and its number of columns (the autotuner's slab timing;
+  // accumulators untouched)
+  static cudaError_t sym_probe(const Plan &p, cudaStream_t st, double *columns);
   // opposite-spin direct term of a tau from the channels' S_jj: acc [na][nb] accumulated (part: scratch)
   static cudaError_t sym_cross(const Plan &pa, const Plan &pb, double coef, double *part, double *acc, cudaStream_t st);
   // the slab in phases: up to w in real space (gather, transformed-state GEMM, z transform),

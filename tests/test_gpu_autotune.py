@@ -1,0 +1,43 @@
+"""An autotuned context is no slower than an untuned one: set-up's own plane-kernel block is among the
+autotuner's candidates, and the slab size is timed on the path that whole energies take."""
+import numpy as np
+import pytest
+
+import paper_1611_06797_gb300 as L
+from synth import ModelSolidSpec, build_model_solid
+
+pytestmark = pytest.mark.gpu
+
+
+def _planes(ctx, tau, w):
+    """The plane stage and the whole of one energy in ms, the least of five."""
+    L.ltmp2_energy(ctx, tau, w)
+    L.ltmp2_set_profiling(ctx, True)
+    best = np.full(2, 1e300)
+    for _ in range(5):
+        L.ltmp2_reset_stage_times(ctx)
+        e = L.ltmp2_energy(ctx, tau, w)
+        st = L.ltmp2_stage_times(ctx)
+        best = np.minimum(best, [st["plane_fft"]["ms"], sum(v["ms"] for v in st.values())])
+    L.ltmp2_set_profiling(ctx, False)
+    return best, e
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("n,a,r2,wells,n_occ", [(18, 12.0, 45, 8, 16), (20, 13.7, 56, 12, 24), (36, 9.0, 64, 6, 12)])
+def test_tuned_is_no_slower(n, a, r2, wells, n_occ, precision):
+    s = build_model_solid(ModelSolidSpec(f"tune{n}", a=a, grid=n, r2=r2, wells=wells, n_occ=n_occ, n_tau=2, seed=n),
+                          device="cuda")
+    tau, w, _ = L.ltmp2_laplace_grid(s.gap, s.width, 2)
+    ctx = L.setup_from_solid(s, precision=getattr(L, precision.upper()), real=True)
+    plain, e = _planes(ctx, tau, w)
+    slab, _ = L.ltmp2_autotune(ctx)
+    tuned, et = _planes(ctx, tau, w)
+    t = L.ltmp2_get_tuning(ctx)
+    L.ltmp2_destroy(ctx)
+    assert 1 <= slab
+    # the scatter of the timings that the choice rests on
+    assert (tuned <= 1.04 * plain).all(), (tuned, plain, t)
+    rel = 1e-13 if precision == "fp64" else 2e-6   # the same sums in passes of another size
+    assert abs(et[0] - e[0]) <= rel * abs(e[0]) and abs(et[1] - e[1]) <= rel * abs(e[0])
+    assert np.abs(et[2] - e[2]).max() <= rel * abs(e[0])
