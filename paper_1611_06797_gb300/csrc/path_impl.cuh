@@ -408,8 +408,7 @@ static void sym_shape(const Plan &p, int &nj, int &np_max) {
   np_max = std::max(1, std::min(p.n_idx, budget / nj));
 }
 
-// The pass of orbitals p.sym_j0 .. + p.sym_nj in parts of np_max G': its matrices S_ij and the rows of the
-// exchange sums
+// The matrices S_ij of the pass of orbitals p.sym_j0 .. + p.sym_nj, in parts of np_max G'
 template <typename T>
 static cudaError_t sym_pass(const Plan &p, int np_max, cudaStream_t st, StageTimer *tm, long long *launches) {
   const int n_idx = p.n_idx, threads = std::min(256, ((p.n_daux + 31) / 32) * 32);
@@ -430,9 +429,11 @@ static cudaError_t sym_pass(const Plan &p, int np_max, cudaStream_t st, StageTim
     }
     *launches += Path<T>::pre_launches(p) + 2;
   }
-  ScopedStage s(tm, kStageColumn);
-  k_xsym<T><<<dim3(sym_pairs(p), (n_idx + 31) / 32), 256, 0, st>>>(p, p.sym_rows);
-  *launches += 1;
+  return cudaSuccess;
+}
+// the rows of the pass's exchange sums
+template <typename T> static cudaError_t launch_xsym(const Plan &p, cudaStream_t st) {
+  k_xsym<T><<<dim3(sym_pairs(p), (p.n_idx + 31) / 32), 256, 0, st>>>(p, p.sym_rows);
   return cudaGetLastError();
 }
 
@@ -445,7 +446,8 @@ template <typename T> cudaError_t Path<T>::sym_probe(const Plan &p0, cudaStream_
   p.sym_j0 = (p.n_occ - p.sym_nj + 1) / 2;
   *columns = (double)p.n_idx * p.sym_nj;
   long long launches = 0;
-  return sym_pass<T>(p, np_max, st, nullptr, &launches);
+  const cudaError_t e = sym_pass<T>(p, np_max, st, nullptr, &launches);
+  return e == cudaSuccess ? launch_xsym<T>(p, st) : e;
 }
 
 template <typename T>
@@ -460,10 +462,11 @@ cudaError_t Path<T>::sym_tau(const Plan &p0, double coef, cudaStream_t st, Stage
     p.sym_nj = std::min(nj, no - p.sym_j0);
     if ((e = sym_pass<T>(p, np_max, st, tm, launches)) != cudaSuccess) return e;
     ScopedStage s(tm, kStageColumn);
+    if ((e = launch_xsym<T>(p, st)) != cudaSuccess) return e;
     // real orbitals: the rows are the primary G', each standing for -G' too
     k_xsym_sum<T><<<sym_pairs(p), 128, 0, st>>>(p, p.sym_rows, (p.real_orb ? 2.0 : 1.0) * coef);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    *launches += 1;
+    *launches += 2;
   }
   {
     ScopedStage s(tm, kStageDirect);
