@@ -1274,24 +1274,23 @@ template <typename X> __device__ __forceinline__ X warp_sum16(X (&v)[16]) {
 template <typename T, bool CPLX, typename F>
 __device__ __forceinline__ void direct_block(int naux, int ni, int nj, F &&load, double2 (&red)[4][16]) {
   constexpr int B = 4, kP = CPLX ? 2 : 1;
-  constexpr bool kComp = std::is_same<T, float>::value;   // FP32: 32 products, then compensated
+  constexpr bool kFp32 = std::is_same<T, float>::value;   // FP32: 32 terms, then added to FP64 sums
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  T s[kP][B * B], hi[kComp ? kP : 1][B * B], low[kComp ? kP : 1][B * B];
-  auto zero = [](T *q) {
+  T s[kP][B * B];
+  double total[kFp32 ? kP : 1][B * B];
 #pragma unroll
-    for (int a = 0; a < B * B; ++a) q[a] = T(0);
-  };
+  for (int c = 0; c < kP; ++c)
 #pragma unroll
-  for (int c = 0; c < kP; ++c) {
-    zero(s[c]);
-    if (kComp) { zero(hi[c]); zero(low[c]); }
-  }
+    for (int q = 0; q < B * B; ++q) {
+      s[c][q] = T(0);
+      if (kFp32) total[c][q] = 0.0;
+    }
   auto carry = [&] {
 #pragma unroll
     for (int c = 0; c < kP; ++c)
 #pragma unroll
       for (int q = 0; q < B * B; ++q) {
-        kadd(hi[c][q], low[c][q], s[c][q]);
+        total[c][q] += (double)s[c][q];
         s[c][q] = T(0);
       }
   };
@@ -1310,16 +1309,14 @@ __device__ __forceinline__ void direct_block(int naux, int ni, int nj, F &&load,
         if (CPLX) sy = fma(x[a].x, y[b].y, fma(x[a].y, y[b].x, sy));
       }
     }
-    if (kComp && (++count & 31) == 0) carry();
+    if (kFp32 && (++count & 31) == 0) carry();
   }
-  if (kComp) carry();
+  if (kFp32) carry();
   double h[kP];
 #pragma unroll
   for (int c = 0; c < kP; ++c) {
-    double d[B * B];
-#pragma unroll
-    for (int q = 0; q < B * B; ++q) d[q] = kComp ? (double)hi[c][q] - (double)low[c][q] : (double)s[c][q];
-    h[c] = warp_sum16(d);
+    if constexpr (kFp32) h[c] = warp_sum16(total[c]);
+    else h[c] = warp_sum16(s[c]);
   }
   const double hx = h[0], hy = CPLX ? h[kP - 1] : 0.0;
   if (lane % 2 == 0) red[warp][lane / 2] = make_double2(hx, hy);

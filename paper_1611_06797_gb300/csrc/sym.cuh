@@ -167,7 +167,7 @@ template <typename T> __global__ void k_xsym_sum(Plan p, const double *__restric
 // two channels' plans (the same one for a closed shell; then only blocks with j >= i are there).
 // The warps take the rows' 32-column chunks in turn, a lane a column: no product is padded, which in
 // FP64 (2 FMA per clock and SM) is what counts: 32 x 32 tiles through shared memory took 1.7 ms
-// per Laplace point on the 8^3 system with 2 occupied.  FP32 sums are compensated.
+// per Laplace point on the 8^3 system with 2 occupied.  FP32: sums of 64 products, added in FP64.
 template <typename T>
 __global__ void __launch_bounds__(256) k_dsym(Plan p, Plan q, bool triangle, double *__restrict__ part) {
   constexpr int B = 4;
@@ -186,12 +186,21 @@ __global__ void __launch_bounds__(256) k_dsym(Plan p, Plan q, bool triangle, dou
   const bool gen = p.sym_planes == 1;
   const T *v = vtab<T>(p);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  constexpr bool kComp = std::is_same<T, float>::value;
-  T acc[B][B], hi[B][B], cmp[B][B];
+  constexpr bool kFp32 = std::is_same<T, float>::value;
+  T acc[B * B];
+  double sum[kFp32 ? B * B : 1];
 #pragma unroll
-  for (int a = 0; a < B; ++a)
+  for (int k = 0; k < B * B; ++k) {
+    acc[k] = T(0);
+    if (kFp32) sum[k] = 0.0;
+  }
+  auto carry = [&] {
 #pragma unroll
-    for (int b = 0; b < B; ++b) acc[a][b] = hi[a][b] = cmp[a][b] = T(0);
+    for (int k = 0; k < B * B; ++k) {
+      sum[k] += (double)acc[k];
+      acc[k] = T(0);
+    }
+  };
   const int2 rows = p.sym_groups[blockIdx.x];
   const cpx<T> *Ma = (const cpx<T> *)p.mdsym + i0 * stride, *Mb = (const cpx<T> *)q.mdsym + j0 * stride;
   // the rows' 32-column chunks go round the warps
@@ -219,30 +228,20 @@ __global__ void __launch_bounds__(256) k_dsym(Plan p, Plan q, bool triangle, dou
           const T xr = w * x[a].x, xi = gen ? -(w * x[a].y) : w * x[a].y;
 #pragma unroll
           for (int b = 0; b < B; ++b)
-            if (j0 + b < nj) acc[a][b] = fma(xr, y[b].x, fma(xi, y[b].y, acc[a][b]));
+            if (j0 + b < nj) acc[a * B + b] = fma(xr, y[b].x, fma(xi, y[b].y, acc[a * B + b]));
         }
       }
-      if (kComp && (++count & 15) == 0) {   // at most 64 products in plain FP32 (a lane past the end skips a turn)
-#pragma unroll
-        for (int a = 0; a < B; ++a)
-#pragma unroll
-          for (int b = 0; b < B; ++b) {
-            kadd(hi[a][b], cmp[a][b], acc[a][b]);
-            acc[a][b] = T(0);
-          }
-      }
+      if (kFp32 && (++count & 15) == 0) carry();   // at most 64 products in plain FP32 (a lane past the end skips a turn)
     }
     chunk += (end + 31) / 32;
   }
-  double sum[B * B];
-#pragma unroll
-  for (int a = 0; a < B; ++a)
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-      if (kComp) kadd(hi[a][b], cmp[a][b], acc[a][b]);
-      sum[a * B + b] = kComp ? (double)hi[a][b] - (double)cmp[a][b] : (double)acc[a][b];
-    }
-  const double s = warp_sum16(sum);
+  double s;
+  if constexpr (kFp32) {
+    carry();
+    s = warp_sum16(sum);
+  } else {
+    s = warp_sum16(acc);
+  }
   if (lane % 2 == 0) red[warp][lane / 2] = s;
   __syncthreads();
   if (threadIdx.x < B * B) {
