@@ -165,6 +165,13 @@ int dalloc_bytes(ltmp2_ctx *c, void **ptr, size_t bytes) {
   return LTMP2_OK;
 }
 
+// give an allocation back before the context goes
+void dfree(ltmp2_ctx *c, void **ptr) {
+  c->allocs.erase(std::remove(c->allocs.begin(), c->allocs.end(), *ptr), c->allocs.end());
+  cudaFree(*ptr);   // waits for what uses it
+  *ptr = nullptr;
+}
+
 template <typename T> struct CT { T x, y; };
 
 template <typename T>
@@ -302,7 +309,8 @@ int default_plane_kernel(const Plan &p) { return p.precision == LTMP2_FP32 && p.
 bool use_sym(const Plan &p) { return p.msym && p.nk == 0 && p.route == 0; }
 
 // exact-slice tensor-core products of a context whose slabs have up to max_cols columns over nz
-// k points, and the virtuals by plane wave that they read (also the CUDA cores' virtual-space route)
+// k points, and the virtuals by plane wave that they read (also the CUDA cores' virtual-space route);
+// without room for them the products run on the CUDA cores
 template <typename T> int setup_products(ltmp2_ctx *c, size_t max_cols, int nz, bool simt) {
   Plan &p = c->p;
   const int nk = nz;
@@ -310,14 +318,18 @@ template <typename T> int setup_products(ltmp2_ctx *c, size_t max_cols, int nz, 
   void **vt = p.real_basis ? &p.rvt : &p.cvt;
   int rc;
   if (simt && !p.real_basis) return LTMP2_OK;
-  if ((rc = dalloc_bytes(c, vt, (p.real_basis ? sizeof(T) : sizeof(CT<T>)) * (size_t)nk * p.n_v * p.n_pw))) return rc;
+  rc = dalloc_bytes(c, vt, (p.real_basis ? sizeof(T) : sizeof(CT<T>)) * (size_t)nk * p.n_v * p.n_pw);
+  if (rc) return rc == LTMP2_ERR_OOM ? LTMP2_OK : rc;
   cudaError_t e = Path<T>::transpose_virtuals(p, *vt, c->stream);
   if (e != cudaSuccess || simt) return cuda_status(e);
   const int slices = std::is_same<T, double>::value ? 8 : 4;
   void *mem = nullptr;
   const int rows = (int)(max_cols / nz);
   rc = dalloc_bytes(c, &mem, oz_bytes(slices, rows, p.n_pw, p.n_v, nz, !p.real_basis));
-  if (rc == LTMP2_ERR_OOM) return LTMP2_OK;   // no room for the slices: the CUDA-core products
+  if (rc == LTMP2_ERR_OOM) {
+    if (!p.real_basis) dfree(c, vt);   // read by the slices alone
+    return LTMP2_OK;
+  }
   if (rc) return rc;
   e = oz_init(c->oz, mem, slices, rows, p.n_pw, p.n_v, nz, !p.real_basis);
   if (e == cudaSuccess) e = oz_set_virtuals<T>(c->oz, p.cv, *vt, c->stream);
