@@ -117,7 +117,9 @@ typedef struct {
 /* Validate the input, copy it to the current CUDA device and precompute the
  * tau-independent parts (occupied orbitals on the grid, the aux set A and v(G),
  * index tables).  The caller keeps ownership of every array in *sys; nothing is
- * retained.  On success *out owns the device memory until ltmp2_destroy().
+ * retained.  On success *out owns the device memory until ltmp2_destroy().  The first
+ * whole energy of a system whose pair matrices exceed 4 GB takes those (at most 12 GB of
+ * a pass and n_occ diagonal ones, and a quarter of the free memory, else it runs without).
  * Errors: INVALID_ARG, GAP, NOT_ORTHONORMAL, GRID, NOT_REAL, OOM, CUDA.           */
 int ltmp2_setup(const ltmp2_system *sys, ltmp2_ctx **out);
 

@@ -101,9 +101,13 @@ struct ltmp2_ctx {
   std::vector<double> lev_ecut;
   std::vector<int> lev_count;
   bool lev_alloc = false, lev_done = false;
-  // whole energies by the pairs' symmetry: the index set on the host, and room for its row groups
+  // whole energies by the pairs' symmetry: the outer loop's G' and the position of -G, until the matrices are
+  // there (sym_tried); the index set on the host, and room for its row groups; L(G) of the levels in effect
+  std::vector<int> prim, aux_neg;
+  bool sym_tried = false;
   std::vector<int> sym_order;
   int2 *d_sym_groups = nullptr;
+  std::vector<unsigned char> lev;
   // spin-unrestricted pairing (this context as the alpha channel): opposite-spin scratch
   double *d_cross_y = nullptr, *d_cross_acc = nullptr, *d_cross_sum = nullptr, *d_cross_part = nullptr;
   int cross_nb = 0;
@@ -218,11 +222,11 @@ constexpr int kSymGroups = 304 + 2 * kMaxLevels;   // row groups of the direct t
 
 // Row groups of the lower triangle, of about equal work, none across a level's boundary, and the
 // rows of each level (the rows are sorted by |G|^2, so a level is a prefix).
-int set_sym_rows(ltmp2_ctx *c, const std::vector<unsigned char> *lev) {
+int set_sym_rows(ltmp2_ctx *c) {
   Plan &p = c->p;
   if (!p.msym) return LTMP2_OK;
   const int n = p.n_idx;
-  auto level = [&](int r) { return lev ? (int)(*lev)[c->sym_order[r]] : 1; };
+  auto level = [&](int r) { return c->lev.empty() ? 1 : (int)c->lev[c->sym_order[r]]; };
   for (int k = 0; k < kMaxLevels; ++k) {
     int rows = 0;
     while (rows < n && level(rows) >= k + 1) ++rows;
@@ -243,25 +247,44 @@ int set_sym_rows(ltmp2_ctx *c, const std::vector<unsigned char> *lev) {
   }
   if ((int)g.size() > kSymGroups) return LTMP2_ERR_INVALID_ARG;
   p.n_groups = (int)g.size();
-  return cuda_status(cudaMemcpy(c->d_sym_groups, g.data(), g.size() * sizeof(int2), cudaMemcpyHostToDevice));
+  const cudaError_t e = cudaMemcpy(c->d_sym_groups, g.data(), g.size() * sizeof(int2), cudaMemcpyHostToDevice);
+  return cuda_status(e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e);   // there before any stream reads it
 }
 
-// Index set and matrices of the pairs' symmetry, where they take at most a quarter of the free
-// memory and their rows fit the column kernel's shared memory; else the energies go by slabs of G'.
-template <typename T>
-int setup_sym(ltmp2_ctx *c, const std::vector<int> &prim, const std::vector<int> &aux_neg) {
-  Plan &p = c->p;
-  const size_t cs = sizeof(CT<T>);
+// Bytes of the matrices of the pairs' symmetry and orbitals per pass; 0 where a row does not fit the column
+// kernel's shared memory
+size_t sym_bytes(const Plan &p, int &nj) {
+  const size_t cs = p.precision == LTMP2_FP64 ? 16 : 8;
   const int planes = p.real_orb ? 2 : 1, n = p.real_orb ? p.n_prim : 2 * p.n_prim, no = p.n_occ;
-  if (n < 1 || (size_t)planes * n * cs > 200 * 1024) return LTMP2_OK;
+  if (n < 1 || (size_t)planes * n * cs > 200 * 1024) return 0;
   const size_t pair = (size_t)planes * n * n * cs;
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return LTMP2_ERR_CUDA;
-  // orbitals per pass: a slab's columns, and at most 12 GB of pairs
-  int nj = std::min(no, std::max(1, p.max_prim * p.slots_per_prim() * no / n));
+  // a slab's columns (its capacity, whatever its size now), and at most 12 GB of pairs
+  nj = std::min(no, std::max(1, p.max_prim * p.slots_per_prim() * no / n));
   while (nj > 1 && (size_t)nj * no * pair > ((size_t)12 << 30)) --nj;
   const size_t pairs = (size_t)nj * no - (size_t)nj * (nj - 1) / 2;
-  if ((pairs + no) * pair > free_b / 4) return LTMP2_OK;
+  return (pairs + no) * pair;
+}
+// Set-up takes the matrices up to this size; larger ones come with the first energy that reads them: a
+// context that runs ranges of G' or persistent batches alone never does.  Taking them costs 1 ms per GB,
+// which a first energy would show where they are small (the 24^3 system in FP32: 1.9 of 197 ms).
+constexpr size_t kSymAtSetup = (size_t)4 << 30;
+
+// Index set and matrices of the pairs' symmetry, where they take at most a quarter of the free
+// memory; else the energies go by slabs of G'.
+int setup_sym(ltmp2_ctx *c) {
+  Plan &p = c->p;
+  const std::vector<int> &prim = c->prim, &aux_neg = c->aux_neg;
+  Plan cap = p;
+  cap.max_prim = c->slab_capacity;
+  int nj = 0;
+  const size_t bytes = sym_bytes(cap, nj);
+  size_t free_b = 0, total_b = 0;
+  if (bytes == 0) return LTMP2_OK;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return LTMP2_ERR_CUDA;
+  if (bytes > free_b / 4) return LTMP2_OK;
+  const int planes = p.real_orb ? 2 : 1, n = p.real_orb ? p.n_prim : 2 * p.n_prim, no = p.n_occ;
+  const size_t pair = (size_t)planes * n * n * (p.precision == LTMP2_FP64 ? 16 : 8);
+  const size_t pairs = (size_t)nj * no - (size_t)nj * (nj - 1) / 2;
   std::vector<int> order(prim), pos(p.n_aux, -1);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return c->aux_g2[a] < c->aux_g2[b]; });
   if (!p.real_orb) {
@@ -280,11 +303,14 @@ int setup_sym(ltmp2_ctx *c, const std::vector<int> &prim, const std::vector<int>
   int *d_order = nullptr, *d_pos = nullptr;
   void *m = nullptr, *md = nullptr;
   double *rows = nullptr, *part = nullptr;
+  const size_t before = c->allocs.size();
   if ((rc = dalloc(c, &d_order, (size_t)n)) || (rc = dalloc(c, &d_pos, (size_t)p.n_aux)) ||
       (rc = dalloc(c, &c->d_sym_groups, (size_t)kSymGroups)) || (rc = dalloc_bytes(c, &m, pairs * pair)) ||
       (rc = dalloc_bytes(c, &md, (size_t)no * pair)) || (rc = dalloc(c, &rows, pairs * n)) ||
-      (rc = dalloc(c, &part, (size_t)kSymGroups * no * no)))
+      (rc = dalloc(c, &part, (size_t)kSymGroups * no * no))) {
+    for (; c->allocs.size() > before; c->allocs.pop_back()) cudaFree(c->allocs.back());
     return rc == LTMP2_ERR_OOM ? LTMP2_OK : rc;
+  }
   if ((rc = cuda_status(cudaMemcpy(d_order, order.data(), n * sizeof(int), cudaMemcpyHostToDevice))) ||
       (rc = cuda_status(cudaMemcpy(d_pos, pos.data(), p.n_aux * sizeof(int), cudaMemcpyHostToDevice))))
     return rc;
@@ -299,7 +325,7 @@ int setup_sym(ltmp2_ctx *c, const std::vector<int> &prim, const std::vector<int>
   p.mdsym = md;
   p.msym = m;
   c->sym_order = order;
-  return set_sym_rows(c, nullptr);
+  return set_sym_rows(c);
 }
 // Plane kernel of a set-up: FP64 has one; FP32 on lines up to 27, pairs of columns by blocks (24^3: 82.6
 // against 97.2 ms, 27^3: 50.5 against 54.4 ms per pass, 18^3 and 20^3: 5 to 25 % faster); longer lines
@@ -307,6 +333,16 @@ int setup_sym(ltmp2_ctx *c, const std::vector<int> &prim, const std::vector<int>
 int default_plane_kernel(const Plan &p) { return p.precision == LTMP2_FP32 && p.n > 27 ? 3 : 2; }
 // every G' at the Gamma point, by the Green's-function route
 bool use_sym(const Plan &p) { return p.msym && p.nk == 0 && p.route == 0; }
+// before a whole energy: its matrices, once
+int ensure_sym(ltmp2_ctx *c) {
+  if (c->sym_tried || c->p.nk > 0 || c->p.route != 0) return LTMP2_OK;
+  c->sym_tried = true;
+  try {
+    return setup_sym(c);
+  } catch (const std::bad_alloc &) {
+    return LTMP2_ERR_OOM;
+  }
+}
 
 // exact-slice tensor-core products of a context whose slabs have up to max_cols columns over nz
 // k points, and the virtuals by plane wave that they read (also the CUDA cores' virtual-space route);
@@ -414,7 +450,10 @@ int setup_precision(ltmp2_ctx *c, const ltmp2_system *sys, const std::vector<int
     p.tc = &c->tc;
   }
   if ((rc = setup_products<T>(c, max_cols, 1, (sys->flags & LTMP2_FLAG_SIMT_GEMM) != 0))) return rc;
-  if ((rc = setup_sym<T>(c, hp.prim, hp.aux_neg))) return rc;
+  c->prim = hp.prim;
+  c->aux_neg = hp.aux_neg;
+  int nj = 0;
+  if (sym_bytes(p, nj) <= kSymAtSetup && (rc = ensure_sym(c))) return rc;
   e = Path<T>::setup_occupied(p, cocc, c->stream);
   if (e != cudaSuccess) return cuda_status(e);
   e = cudaStreamSynchronize(c->stream);
@@ -598,6 +637,7 @@ int energy_common(ltmp2_ctx *ctx, int n_tau, const double *tau, const double *w,
   if (rc) return rc;
   if (gp_begin < 0 || gp_end > ctx->p.n_prim || gp_begin > gp_end) return LTMP2_ERR_INVALID_ARG;
   DeviceGuard g(ctx->device);
+  if (gp_begin == 0 && gp_end == ctx->p.n_prim && (rc = ensure_sym(ctx))) return rc;
   rc = ctx->p.precision == LTMP2_FP64 ? run_energy<double>(ctx, n_tau, tau, w, gp_begin, gp_end)
                                       : run_energy<float>(ctx, n_tau, tau, w, gp_begin, gp_end);
   if (rc) return rc;
@@ -663,6 +703,7 @@ template <typename T> int tune_ctx(ltmp2_ctx *c, int *slab_out, int *var_out) {
       return rc;
     }
   }
+  if (const int src = ensure_sym(c)) return src;
   std::vector<int> slabs;
   for (int sl = std::min(c->slab_capacity, p.n_prim); sl >= 1 && slabs.size() < 4; sl /= 2) slabs.push_back(sl);
   const int variant = p.tc ? 5 : -1;
@@ -1485,6 +1526,7 @@ int ltmp2_batch_create(ltmp2_ctx *const *ctxs, int n, const int *n_tau, const do
   }
   std::vector<Plan> plans(n);
   for (int i = 0; i < n; ++i) {
+    if (const int src = ensure_sym(ctxs[i])) return fail(src);
     plans[i] = ctxs[i]->p;
     if (const int trc = own_tables(b, plans[i])) return fail(trc);
   }
@@ -1606,6 +1648,7 @@ int ltmp2_energy_uhf(ltmp2_ctx *alpha, ltmp2_ctx *beta, int n_tau, const double 
     return LTMP2_ERR_INVALID_ARG;
   if (pa.n_lev > 1 || pb.n_lev > 1 || pa.pair_keep || pb.pair_keep) return LTMP2_ERR_UNSUPPORTED;
   DeviceGuard g(alpha->device);
+  if ((rc = ensure_sym(alpha)) || (rc = ensure_sym(beta))) return rc;
   // a common slab size; restored afterwards
   const int keep_a = pa.max_prim, keep_b = pb.max_prim;
   const int slab = std::min(keep_a, keep_b);
@@ -1615,8 +1658,11 @@ int ltmp2_energy_uhf(ltmp2_ctx *alpha, ltmp2_ctx *beta, int n_tau, const double 
     if ((rc = dalloc(alpha, &alpha->d_cross_acc, nab))) return rc;
     if ((rc = dalloc(alpha, &alpha->d_cross_sum, 1))) return rc;
     alpha->d_cross_part = nullptr;
-    if (use_sym(pa) && use_sym(pb) && (rc = dalloc(alpha, &alpha->d_cross_part, (size_t)kSymGroups * nab))) return rc;
     alpha->cross_nb = pb.n_occ;
+  }
+  if (use_sym(pa) && use_sym(pb) && !alpha->d_cross_part) {
+    rc = dalloc(alpha, &alpha->d_cross_part, (size_t)kSymGroups * pa.n_occ * pb.n_occ);
+    if (rc && rc != LTMP2_ERR_OOM) return rc;   // without room the slabs' cross term runs
   }
   pa.max_prim = pb.max_prim = slab;
   rc = pa.precision == LTMP2_FP64 ? enqueue_uhf<double>(alpha, beta, n_tau, tau, w, &alpha->kernel_launches)
@@ -1700,7 +1746,8 @@ int ltmp2_set_extrapolation(ltmp2_ctx *ctx, int n_c, double alpha) {
   if (n_c <= 1) {
     DeviceGuard g(ctx->device);
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return LTMP2_ERR_CUDA;
-    const int rc = set_sym_rows(ctx, nullptr);
+    ctx->lev.clear();
+    const int rc = set_sym_rows(ctx);
     if (rc) return rc;
     p.n_lev = 0;
     ctx->lev_ecut.clear();
@@ -1759,7 +1806,8 @@ int ltmp2_set_extrapolation(ltmp2_ctx *ctx, int n_c, double alpha) {
   if (e == cudaSuccess)
     e = cudaMemcpy((void *)p.lev_start, start.data(), (n_c + 1) * sizeof(int), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_status(e);
-  if ((rc = set_sym_rows(ctx, &lev))) return rc;
+  ctx->lev = lev;
+  if ((rc = set_sym_rows(ctx))) return rc;
   p.n_lev = n_c;
   ctx->lev_ecut = ecut;
   ctx->lev_count = count;
