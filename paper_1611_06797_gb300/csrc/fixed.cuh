@@ -91,6 +91,15 @@ __host__ __device__ __forceinline__ long long fx_shr(long long x, int s) {
   return s > 0 ? (x + (1ll << (s - 1))) >> s : x;
 }
 
+// ---------------------------------------------------------------- scales
+constexpr int kFxBits = 61;          // |fixed-point value| <= 2^61, the bound given by the 2-norms
+constexpr int kFxNotFinite = 1 << 20;   // exponent of a state with a NaN or an infinity
+// e with 2^e > sqrt(norm2); smaller squares than 2^-962 count as that
+__host__ __device__ __forceinline__ int fx_exponent(double norm2) {
+  if (!(norm2 < 1e300)) return kFxNotFinite;
+  return norm2 < 0x1p-962 ? -480 : (ilogb(norm2) >> 1) + 1;
+}
+
 // ---------------------------------------------------------------- radix kernels
 template <int DIR> struct Radix<long long, 3, DIR> {
   typedef cpx<long long> C;

@@ -43,13 +43,6 @@ template <typename T> struct Codensity {
   static __device__ __forceinline__ cpx<T> real(cpx<T> a) { return a; }
   static __device__ __forceinline__ T scale(const Plan &, int, size_t) { return T(1); }
 };
-constexpr int kFxBits = 61;          // |fixed-point value| <= 2^61, the bound given by the 2-norms
-constexpr int kFxNotFinite = 1 << 20;   // exponent of a state with a NaN or an infinity
-// e with 2^e > sqrt(norm2); squares below 1e-290 count as zero
-__device__ __forceinline__ int fx_exponent(double norm2) {
-  if (!(norm2 < 1e300)) return kFxNotFinite;
-  return norm2 < 1e-290 ? -480 : (ilogb(norm2) >> 1) + 1;
-}
 __device__ __forceinline__ double fx_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 template <> struct Codensity<double> {
   typedef long long W;
