@@ -1366,13 +1366,10 @@ template <typename T> __global__ void __launch_bounds__(128) k_direct_w(Plan p, 
   }
 }
 
-// ---------------------------------------------------------------- pair descriptors
-// Per occupied orbital: z_k = (1/N) sum_t |u(t)|^2 exp(2 pi i t_k / n), k = x, y, z
-// (periodic centroid from arg z_k, spread from |z_k|).  out[i][6] = (Re, Im) x 3.
 // Direct term, tiled: block (G' of the slab, 32 x 32 tile of (i, j)); the G sum runs in
 // chunks of 32 staged in shared memory (M_ii for the tile's i, M_jj at -G or conjugated for
 // its j, v(G)).  Each thread owns one j and four i; every 32-term chunk is summed in T and
-// added to a double accumulator, as in k_direct.
+// added to a double accumulator.
 template <typename T>
 __global__ void __launch_bounds__(256) k_direct_tiled(Plan p, int np, const cpx<T> *__restrict__ mdiag,
                                                       double2 *__restrict__ yd) {
@@ -1425,6 +1422,9 @@ __global__ void __launch_bounds__(256) k_direct_tiled(Plan p, int np, const cpx<
   }
 }
 
+// ---------------------------------------------------------------- pair descriptors
+// Per occupied orbital: z_k = (1/N) sum_t |u(t)|^2 exp(2 pi i t_k / n), k = x, y, z
+// (periodic centroid from arg z_k, spread from |z_k|).  out[i][6] = (Re, Im) x 3.
 template <typename T> __global__ void k_orb_moments(Plan p, double *__restrict__ out) {
   const int i = blockIdx.x, n = p.n;
   const size_t n3 = (size_t)n * n * n;

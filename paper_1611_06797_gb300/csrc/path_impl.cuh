@@ -364,8 +364,11 @@ cudaError_t Path<T>::slab_post(const Plan &p, int gp0, int np, double coef, cuda
   {
     ScopedStage s(tm, kStageDirect);
     int th = no < 128 ? ((no + 31) / 32) * 32 : 128;
-    // FP32: the shared-memory tiled kernel; FP64 is bound by the FP64 pipe, and the warp-level
-    // sums pad nothing and take the real part alone where only that enters
+    // FP32 (general orbitals, or the tensor-core product off): the shared-memory tiled kernel, which reads
+    // each co-density once per 32 others: two Laplace points of one or two slabs of 48 / 64 / 96 / 128
+    // occupied take 0.78 / 1.27 / 1.38 / 0.86 ms, 1.24 / 2.27 / 3.39 / 3.35 ms by warp-level sums (which pad
+    // nothing: 0.23 against 0.09 ms with 8 occupied, 1.33 against 1.16 ms with 32).  FP64 is bound by the
+    // FP64 pipe, and the warp-level sums take the real part alone where only that enters.
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
       if (!lev && p.tc && p.tc->direct_on()) {   // real orbitals: one tensor-core product per G'
@@ -376,7 +379,7 @@ cudaError_t Path<T>::slab_post(const Plan &p, int gp0, int np, double coef, cuda
     if (done) {
     } else if (lev) {
       k_direct_lev<T><<<dim3(np, no), th, 0, st>>>(p, np, (const cpx<T> *)p.mdiag, p.yd);
-    } else if (std::is_same<T, float>::value) {
+    } else if constexpr (std::is_same<T, float>::value) {
       const int t = (no + 31) / 32;
       k_direct_tiled<T><<<dim3(np, t, t), 256, 0, st>>>(p, np, (const cpx<T> *)p.mdiag, p.yd);
     } else {
