@@ -54,7 +54,30 @@ def test_fp64_matches_oracle(name, phases, real):
     eref = ref["e_d"] + ref["e_x"]
     assert np.abs(ep - eref).max() < TOL_FP64
     assert np.abs(ep - ep.T).max() < 1e-12
-    assert abs(im[0]) < 1e-10 and abs(im[1]) < 1e-10
+    assert abs(im[0]) < 1e-10 and abs(im[1]) < 1e-10   # whole energies: identically zero (and ep symmetric)
+
+
+@pytest.mark.parametrize("name", ["tiny2", "cfg1"])
+def test_fp64_slabs_of_general_orbitals_match_oracle(name):
+    """Two ranges of the outer G' loop, which keep M(G, G') and M(-G, -G') apart and sum their products as
+    complex numbers: the oracle's energies, and imaginary residues at rounding."""
+    s = solid(name, random_phases=True)
+    tau, w = _quad(s, s.spec.n_tau)
+    ref = _oracle(s, tau, w)
+    ctx = L.setup_from_solid(s, precision=L.FP64, real=False)
+    n = L.ltmp2_num_primary_gprime(ctx)
+    total, residues = None, []
+    for b, e in ((0, n // 3), (n // 3, n)):
+        part = L.ltmp2_energy_partial(ctx, tau, w, b, e)
+        residues.append(L.ltmp2_last_imag(ctx))
+        total = part if total is None else tuple(x + y for x, y in zip(total, part))
+    L.ltmp2_destroy(ctx)
+    ed, ex, pd, px = total
+    tol = 1e-12 * abs(ref["E_d"])   # FP64 sums of 1e5 terms
+    assert abs(ed - ref["E_d"]) < tol and abs(ex - ref["E_x"]) < tol
+    assert np.abs(pd - ref["e_d"]).max() < tol and np.abs(px - ref["e_x"]).max() < tol
+    assert all(abs(x) < tol for im in residues for x in im)
+    assert any(x != 0.0 for im in residues for x in im)   # summed, not written as zero
 
 
 def test_slab_sizes_and_ragged_tail_agree():
@@ -177,9 +200,10 @@ def test_plane_kernels_and_block_shapes_agree(name, real):
 
 @pytest.mark.parametrize("name", ["tiny2", "cfg1"])
 def test_precision_form_green_and_direct_choices(name):
-    """The precision form's Green's function (compensated CUDA-core sums by default, or
-    3xTF32 on the tensor cores, set up at first use) and its direct term (tensor cores by
-    default, or CUDA cores): every combination within 0.1 meV/atom of the FP64 path."""
+    """The precision form's Green's function (exact slices by default, or 3xTF32, set up at first
+    use) and its direct term (of slabs: tensor cores by default, or CUDA cores; a whole energy takes
+    it from the pair matrices): every combination within 0.1 meV/atom of the FP64 path, whole and
+    in two ranges of G'."""
     s = solid(name)
     tau, w = _quad(s, s.spec.n_tau)
     d64, x64, p64, _ = _gpu(s, tau, w, L.FP64, real=True)
@@ -193,6 +217,10 @@ def test_precision_form_green_and_direct_choices(name):
         assert (t["green_tc"], t["direct_tc"]) == (g, d)
         ed, ex, ep = L.ltmp2_energy(ctx, tau, w)
         assert abs(ed - d64) < bound and abs(ex - x64) < bound and np.abs(ep - p64).max() < bound, (g, d)
+        n = L.ltmp2_num_primary_gprime(ctx)
+        a, b = L.ltmp2_energy_partial(ctx, tau, w, 0, n // 2), L.ltmp2_energy_partial(ctx, tau, w, n // 2, n)
+        assert abs(a[0] + b[0] - d64) < bound and abs(a[1] + b[1] - x64) < bound, (g, d)
+        assert np.abs(a[2] + b[2] + a[3] + b[3] - p64).max() < bound, (g, d)
     with pytest.raises(L.Ltmp2Error):
         L.ltmp2_set_tuning(ctx, green_tc=2)
     L.ltmp2_destroy(ctx)
