@@ -250,6 +250,29 @@ def measured_alu(L):
             "kind": "measured in this run: independent FMA chains over a full grid, CUDA events, best of 5"}
 
 
+# A line of 24 complex values in 64-bit fixed point (8 x 3): 252 additions and 28 products, 11.0 clocks of an
+# SM at the measured 50 and 4.7 a clock, for 5 n log2 n = 550 counted operations
+FX_LINE_OPS_PER_CLK = 5.0 * 24 * math.log2(24) / (252 / 50.0 + 28 / 4.7)
+
+
+def _own_units(stage, flops, per_launch_ms, precision, simt, peaks, peak_kind):
+    """The stage's work on the units that do it: FP16 slice products (10 or 36 per real product) at the
+    measured bf16 rate, and the FP64 path's line transforms at the rate of 64-bit integer operations."""
+    if not simt and stage in ("w_gemm", "green_gemm"):
+        products = 36.0 if precision == 0 else 10.0
+        peak = peaks["bf16_tflops"]
+        kind = f"{peak_kind} bf16; {products:.0f} FP16 slice products per product"
+        work = flops * products
+    elif stage == "plane_fft" and precision == 0:
+        peak = FX_LINE_OPS_PER_CLK * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e12
+        kind = f"64-bit integer additions and products, {SM_COUNT} SMs at {SM_MAX_MHZ:.0f} MHz, counted as 5 n log2 n per line"
+        work = flops
+    else:
+        return None
+    rate = work / (per_launch_ms / 1e3) / 1e12
+    return {"achieved": rate, "peak": peak, "frac": rate / peak, "peak_kind": kind}
+
+
 def _stage_bound(stage, st, costs, precision, simt, peaks, peak_kind, alu):
     """achieved = algorithmic work per launch / mean launch time (CUDA events around each
     launch on the library's stream), against the rate that bounds the stage."""
@@ -273,6 +296,10 @@ def _stage_bound(stage, st, costs, precision, simt, peaks, peak_kind, alu):
         achieved = work / (per_launch_ms / 1e3) / 1e12
         out.update({"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                     "peak_kind": pk, "work_per_launch": work})
+        own = _own_units(stage, costs[stage]["flops"] / st[stage]["launches"], per_launch_ms, precision, simt, peaks,
+                         peak_kind)
+        if own:
+            out["own_units"] = own
     traffic = traffic_for(stage, precision)
     if traffic:
         # DRAM bytes of a full launch (the stored capture) over the mean launch time: the
@@ -291,7 +318,8 @@ def roofline_of(st, costs, precision, simt, peaks, peak_kind, alu):
     r = _stage_bound(dom, st, costs, precision, simt, peaks, peak_kind, alu)
     return {"kernel": dom, "bound": r["bound"], "achieved": r["achieved"], "peak": r["peak"], "unit": "TFLOP/s",
             "frac": r["frac"], "peak_kind": r["peak_kind"], "traffic": traffic_for(dom, precision),
-            "work_per_launch": r["work_per_launch"], "avg_launch_ms": r["avg_launch_ms"]}
+            "work_per_launch": r["work_per_launch"], "avg_launch_ms": r["avg_launch_ms"],
+            "own_units": r.get("own_units")}
 
 
 def stage_rooflines(st, costs, precision, simt, peaks, peak_kind, alu):

@@ -58,12 +58,15 @@ extern "C" {
 #define LTMP2_ERR_NOT_REAL (-10)       /* LTMP2_FLAG_REAL_ORBITALS set but c(-G) != conj c(G) */
 
 /* ---------------------------------------------------------------- precision */
-/* LTMP2_FP64: complex128 FFTs, FP64 GEMMs, FP64 accumulation (the plain path).   */
+/* LTMP2_FP64: the plain path.  Products of FP64 accuracy from 8 exact integer slices   */
+/*             per operand; the states' z transform in complex128, their x and y          */
+/*             transforms and the co-densities' in 64-bit fixed point scaled by the       */
+/*             states' 2-norms (roundings of 2^-61 of the norms); FP64 sums.              */
 /* LTMP2_FP32: complex64 FFTs; the Green's function and the transformed states on     */
 /*             tcgen05 tensor cores from 4 exact integer slices of 7 bits per        */
 /*             operand (28 bits below a row's maximum, exact sums); with real        */
 /*             orbitals the direct-term products sum_G v M_ii conj(M_jj) per G' in   */
-/*             3xTF32 split precision (hi*hi + hi*lo + lo*hi); per-pair, per-tau     */
+/*             3xTF32 split precision (hi*hi + hi*lo + lo*hi) in slabs; per-pair, per-tau */
 /*             and final sums in FP64.                                               */
 #define LTMP2_FP64 0
 #define LTMP2_FP32 1
@@ -180,7 +183,9 @@ int ltmp2_set_slab_size(ltmp2_ctx *ctx, int n);
  * run on its own branch, then ONE persistent plane-FFT launch and ONE persistent column
  * launch serve the co-density items of all those systems (resident thread blocks take
  * (system, column, plane) and (system, pair) items from a device counter), then each
- * system's direct term and accumulation.  Otherwise every system is one graph branch.
+ * system's direct term and accumulation.  Otherwise every system is one graph branch,
+ * which runs ltmp2_energy's passes over pairs i <= j; the rounds run every ordered pair and
+ * take up to twice the time of branches (12^3 to 40^3, 4 to 8 equal systems).
  * FP64 energies equal ltmp2_energy's to rounding of the summation order.              */
 
 /* Autotuner: times a slab's work on the path that ltmp2_energy takes for each slab size
@@ -191,8 +196,9 @@ int ltmp2_set_slab_size(ltmp2_ctx *ctx, int n);
  * (gemm_variant = -1 in LTMP2_FP64, else 5).  Errors: INVALID_ARG, CUDA, TIMEOUT.      */
 int ltmp2_autotune(ltmp2_ctx *ctx, int *slab, int *gemm_variant);
 
-/* Settings in effect for ctx: values[0] slab size, [1] tensor-core GEMM layout (5, or 4 for general orbitals; one kernel serves both; -1 in
- * FP64 or with LTMP2_FLAG_SIMT_GEMM), [2] plane FFT kernel (0 full-plane passes,
+/* Settings in effect for ctx: values[0] slab size, [1] tensor-core GEMM layout (5; general
+ * orbitals also take 4 from ltmp2_set_tuning, which is kept and changes nothing: one kernel is
+ * left; -1 in FP64 or with LTMP2_FLAG_SIMT_GEMM), [2] plane FFT kernel (0 full-plane passes,
  * 1 compacted passes, 2 product in registers with a compact intermediate, in LTMP2_FP32 on
  * pairs of columns, 3 every warp on its own occupied planes and no block barriers; set-up
  * chooses 3 in LTMP2_FP32 on grids above 27^3, else 2; LTMP2_FP64 has one kernel, which
@@ -200,8 +206,9 @@ int ltmp2_autotune(ltmp2_ctx *ctx, int *slab, int *gemm_variant);
  * kernel 3 per warp step (0 = default; a launch takes no more than fit), [4] the precision form's
  * Green's function and transformed states in 3xTF32 (1; set up at first use) or from
  * exact slices (0, the default: the 3xTF32 build's plain FP32 sums over K = n_v left
- * 4x the error in E_d on the 36^3 workload), [5] its direct-term
- * contraction on the tensor cores (1, the default) or the CUDA cores (0); [4] and [5] are
+ * 4x the error in E_d on the 36^3 workload), [5] the direct-term
+ * contraction of slabs on the tensor cores (1, the default) or the CUDA cores (0; whole
+ * energies take it from the pair matrices either way); [4] and [5] are
  * -1 where there is no choice (FP64, general orbitals, LTMP2_FLAG_SIMT_GEMM).
  * The autotuner also chooses [2] and [3], timing the plane kernel alone.  values holds
  * LTMP2_TUNING_VALUES entries.                                                          */
@@ -379,9 +386,9 @@ int ltmp2_set_route(ltmp2_ctx *ctx, int route);
  * holds a NaN or an infinity gives NaN.
  * ltmp2_dgemm_nt: C = A B^T with that scheme.  A [m][lda], B [n][ldb], C [m][ldc]: DEVICE
  * pointers to row-major doubles (first k columns of A and B used), lda, ldb >= k,
- * ldc >= n.  Allocates and frees its own slice buffers (about 32 (m + n) k bytes) and
+ * ldc >= n.  Allocates and frees its own slice buffers (about 16 (m + n) k bytes) and
  * synchronises the device.  Errors: INVALID_ARG, OOM, CUDA, TIMEOUT (a bounded wait
- * inside the kernel ran out; C is then not written).                                     */
+ * inside the kernel ran out; C is then incomplete).                                      */
 int ltmp2_dgemm_nt(int m, int n, int k, const double *a, int lda, const double *b, int ldb, double *c, int ldc);
 
 /* ---------------------------------------------------------------- virtuals per Laplace point

@@ -709,16 +709,18 @@ struct alignas(16) cpx2 { fx2 x, y; };   // complex, both parts split
 // FP64 form of planes3_body on 64-bit fixed point (fixed.cuh).  The FP64 pipe bound the same
 // passes in double (85 % of its issue rate); a launch of 3488 columns of 32 occupied on 24^3 took
 // 62.3 ms in double, 11.5 ms on integers with a full 64 x 64 bit product, and takes 9.8 ms with
-// split halves and one copy of the transform (the column kernel: 14.1 -> 4.2 ms).  Now bound by the
-// issue of its 2,500 instructions a plane (half of the issue slots) at three warps per scheduler,
-// which its registers (4 per point and thread) allow.
+// split halves and one copy of the transform (the column kernel: 14.1 -> 4.2 ms).  Now bound by latency
+// at the three warps per scheduler that its registers allow (4 per point and thread): on 18^3, 152
+// registers, 44 % of the issue slots, the integer multiplier 48 % busy; a warp waits 1.6 cycles per
+// instruction at barriers and 1.5 for the previous result.
 //  w plane: scaled by 2^(61 - e), 2^e > ||w||_2 of the plane (n ||z1||_2 by Parseval), inverse
 //           transformed in fixed point; every partial sum of the transform is at most
 //           sum |z1| <= sqrt(n_dorb) ||z1||_2 < ||w||_2;
 //  x pass : phi_i comes as phi 2^(61 - uen), 2^uen > ||phi_i||_2 of the plane, and phi and w as
 //           two signed halves (fx_split), which makes their product three IMAD.WIDE; the product
 //           is conj(phi_i) w 2^(61 - uen - e), and every partial sum of its forward transform
-//           is at most ||phi_i||_2 ||w||_2 (Cauchy-Schwarz): below 2^61;
+//           is at most ||phi_i||_2 ||w||_2 (Cauchy-Schwarz): below 2^61 (so a rounding is 2^-61 of the
+//           norms' product wherever it falls: small elements keep fewer bits than in FP64, large ones more);
 //  y pass, copy: as in planes3_body; the copy shifts to the item's scale 2^(61 - uen3 - wen3), from
 //           the norms over all planes, so that the column kernel's sums over z stay below 2^61.
 template <int N>

@@ -1505,6 +1505,11 @@ int ltmp2_batch_create(ltmp2_ctx *const *ctxs, int n, const int *n_tau, const do
   // lockstep: when one system needs many more rounds than the others, most rounds hold that
   // system alone and the lockstep only adds synchronisation (the 8-system workload: 6 to
   // 850 rounds, 0.59x the systems run one after another; independent branches: about 1x).
+  // Rounds run slabs, every ordered pair; branches run whole energies' symmetric passes, half of the
+  // transforms.  Balanced batches, ms by rounds / by branches / one after another: 12^3 x 8 FP64 13.8 / 8.0 /
+  // 13.9, 18^3 x 6 FP64 528 / 256 / 262, FP32 122 / 60 / 63, 36^3 x 4 FP64 1779 / 1285 / 1304 (before the
+  // symmetry 18^3 FP64 1705 / 1694 / 1733, 36^3 6694 / 8022 / 8044): the line stays where callers know
+  // it (ltmp2_batch_mode), a caller that wants branches gives one system another slab size.
   bool persist = n <= kBatchMax;
   int rmin = 0, rmax = 0;
   for (int i = 0; i < n; ++i) {

@@ -83,8 +83,7 @@ __global__ void __launch_bounds__(256) k_zsym(Plan p, int gp0) {
 
 // Exchange sums of a pass: block (pair, row tile); rows[pair][g'] = v(g') sum_{p <= g'} c v(p)
 // Re[S(p, g') conj S(g', p)] (second plane: Re[S(-p, g') S(-g', p)]), c = 2 below the diagonal and 1
-// on it.  32 x 32 tiles, the transposed one through shared memory; FP32 terms of one
-// tile are summed in FP32, tiles in FP64.  Bound by reading S once (12.7 GB per Laplace point of the
+// on it.  32 x 32 tiles, the transposed one through shared memory; every term is added in FP64.  Bound by reading S once (12.7 GB per Laplace point of the
 // 24^3 system in FP64).
 template <typename T> __global__ void __launch_bounds__(256) k_xsym(Plan p, double *__restrict__ rows) {
   __shared__ cpx<T> tile[2][32][33];

@@ -60,3 +60,19 @@ def test_stored_traffic_is_keyed_by_the_kernel_sources():
         t = bench.traffic_for("plane_fft", precision)
         assert t is None or t > 0
     assert bench.traffic_for("accumulate", 0) is None
+
+
+def test_own_units_bound_the_stage():
+    """The FP16 slice products against the bf16 rate, the fixed-point transforms against the integer rate."""
+    costs = _costs([3039], [0])
+    peaks = {"hbm_gbs": 6760.6, "bf16_tflops": 1905.5}
+    alu = {"fp64": 1.2, "fp32": 73.0, "kind": "test"}
+    st = {"w_gemm": {"ms": 100.0, "launches": 10}, "plane_fft": {"ms": 400.0, "launches": 8}}
+    for precision, products in ((0, 36.0), (1, 10.0)):
+        r = bench.stage_rooflines(st, costs, precision, False, peaks, "measured", alu)
+        w = r["w_gemm"]["own_units"]
+        assert math.isclose(w["achieved"], costs["w_gemm"]["flops"] / 10 * products / 10e-3 / 1e12) and w["peak"] == 1905.5
+        assert ("own_units" in r["plane_fft"]) == (precision == 0)
+    r = bench.stage_rooflines(st, costs, 0, True, peaks, "measured", alu)
+    assert "own_units" not in r["w_gemm"]            # CUDA-core products have the FP64 rate
+    assert 14.0 < r["plane_fft"]["own_units"]["peak"] < 18.0
