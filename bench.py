@@ -524,7 +524,7 @@ def main():
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "s_per_E_MP2": ms_step / 1e3,
         "higher_is_better": True, "scaling": "strong", "vs_baseline": None,
-        "dtype": "f64" if primary == L.FP64 else "c64/tf32x3/f64-sum",
+        "dtype": "f64" if primary == L.FP64 else "c64/exact-slices/f64-sum",
         "data": "synthetic: seeded Gaussian-well model solid, orbitals from dense diagonalisation",
         "config": {"workload": _workload_desc(spec), "n_pw": sizes["n_pw"], "n_aux": sizes["n_aux"],
                    "n_occ": sizes["n_occ"], "grid": sizes["grid"], "n_tau": n_tau, "pairs": pairs,
@@ -710,7 +710,7 @@ def form_batch(L, torch, local, steps, warmup, alu=None):
     return {
         "metric": METRIC, "value": units / (ms / 1e3), "unit": UNIT, "n_gpus": 1, "steps": steps,
         "warmup": warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "c64/tf32x3/f64-sum",
+        "vs_baseline": None, "dtype": "c64/exact-slices/f64-sum",
         "data": "synthetic: 8 seeded Gaussian-well model solids, orbitals from dense diagonalisation",
         "config": {"workload": "batching form: " + ", ".join(
             f"{s.spec.wells} wells {s.spec.grid}^3 {s.n_pw} PW {s.n_occ} occ {s.spec.n_tau} tau" for s in solids),
@@ -804,7 +804,7 @@ def run_learned(args, local):
     return {
         "metric": METRIC, "value": pairs * spec.n_tau / (ms_scr / 1e3), "unit": UNIT, "n_gpus": 1,
         "steps": 1, "warmup": 1, "ms_per_step": ms_scr, "s_per_E_MP2": ms_scr / 1e3, "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "c64/tf32x3/f64-sum",
+        "scaling": "weak", "vs_baseline": None, "dtype": "c64/exact-slices/f64-sum",
         "data": "synthetic: seeded Gaussian-well model solids, orbitals from dense diagonalisation",
         "config": {"workload": _workload_desc(spec) + "; learned form: pair model trained on " +
                    ",".join(train_names) + f" ({len(y)} exact pair labels)", "budget_meV_per_atom": 0.1,
@@ -909,7 +909,7 @@ def form_cfg3(L, torch, local, steps, warmup, alu=None):
     return {
         "metric": METRIC, "value": pairs * n_tau / (ms / 1e3), "unit": UNIT, "n_gpus": 1, "steps": steps,
         "warmup": warmup, "ms_per_step": ms, "s_per_E_MP2": ms / 1e3, "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "c64/tf32x3/f64-sum",
+        "scaling": "weak", "vs_baseline": None, "dtype": "c64/exact-slices/f64-sum",
         "data": "synthetic: seeded Gaussian-well model solid, orbitals from dense diagonalisation",
         "config": {"workload": _workload_desc(spec), "n_pw": sizes["n_pw"], "n_aux": sizes["n_aux"],
                    "n_occ": sizes["n_occ"], "grid": sizes["grid"], "n_tau": n_tau, "pairs": pairs,
