@@ -280,7 +280,7 @@ def _stage_bound(stage, st, costs, precision, simt, peaks, peak_kind, alu):
     out = {"avg_launch_ms": per_launch_ms}
     if stage in costs:
         work = costs[stage]["flops"] / st[stage]["launches"]
-        if not simt and (stage == "w_gemm" or (stage == "green_gemm" and precision == 0)):
+        if not simt and stage in ("w_gemm", "green_gemm"):
             # counted as TF32-rate work, 3 products per FP32 product and 36 per FP64 product, so that
             # the figures of earlier builds compare; the kernels form 10 (4 exact slices) and 36
             # (8 exact slices) FP16 products, whose rate is the bf16 one

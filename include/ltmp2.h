@@ -191,6 +191,7 @@ int ltmp2_set_slab_size(ltmp2_ctx *ctx, int n);
 /* Autotuner: times a slab's work on the path that ltmp2_energy takes for each slab size
  * down from the setup capacity and keeps the fastest per column, then the plane FFT
  * kernel and its block shape; set-up's own choices stay unless another is 5 % (2 %) faster.
+ * Takes the pair matrices first, as a whole energy does (see ltmp2_setup).
  * The choice is cached per (grid, n_pw, n_occ, |A|, precision, real-orbital flag) for the
  * process and applied to ctx.  slab, gemm_variant: NULL or receive the choice
  * (gemm_variant = -1 in LTMP2_FP64, else 5).  Errors: INVALID_ARG, CUDA, TIMEOUT.      */
